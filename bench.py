@@ -43,12 +43,12 @@ APPLY_K = 5          # apply throughput: the degree-5 point of the ~16 MDoF swee
 METRIC = "SIPG apply DoF/s & %roofline; solve s/MDoF to 1e-10 rel. res. vs plain FP64 MG"
 
 # DRAM bytes per launch of the solve's dominant kernel, per DoF: ncu
-# dram__bytes_read.sum + dram__bytes_write.sum of dg_integrate_kernel<double,5,
-# Cartesian> on this workload's mesh (111,714,048 + 13,050,368 bytes over
-# 4,096,000 DoF in one captured launch; the command is in traffic_source).
-DOMINANT_DRAM_BYTES_PER_DOF = (111714048 + 13050368) / 4096000
+# dram__bytes_read.sum + dram__bytes_write.sum of dg_box_kernel<double,5> on
+# this workload's mesh (33.07 + 0.42 MB over 4,096,000 DoF in one captured
+# launch, the output still in L2 at its end; the command is in traffic_source).
+DOMINANT_DRAM_BYTES_PER_DOF = (33070000 + 418820) / 4096000
 DOMINANT_NCU_COMMAND = ("ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum "
-                        "--clock-control none -k regex:dg_integrate -s 4 -c 1 python -m "
+                        "--clock-control none -k regex:dg_box -s 4 -c 1 python -m "
                         "paper_1910_01900_gb300.sweep --k 4 --curved 0 --precision 0 --m 32 --repeats 2 "
                         "(dram bytes of one launch on the workload's 32^3 k=4 mesh)")
 
@@ -220,7 +220,7 @@ def run_gb300(args):
     v64 = torch.empty_like(u64)
     with torch.cuda.stream(stream):
         ctx.time_apply(u64, v64, 3)
-        te_w, ti_w = ctx.time_apply(u64, v64, 20)
+        _, ti_w = ctx.time_apply(u64, v64, 20)   # one pass on axis-aligned cells
     del u64, v64
     ctx32.close()
     # the extra workload: 16^3 curved k = 5 solves, FP64 and mixed
@@ -254,9 +254,9 @@ def run_gb300(args):
     clocks = summarize_clocks(samples)
     peak64 = fma_peak(0)
     hbm = measured_peaks().get("hbm_gbs")
-    fe_w, fi_w = flops_alg(k, bool(deform))
-    # dominant kernel of the FP64 solve: the DG integration pass (face fluxes +
-    # transposed sweeps) of the finest level; its algorithmic work per launch is fi_w * N
+    _, fi_w = flops_alg(k, bool(deform))
+    # dominant kernel of the FP64 solve: the one-pass DG operator of the finest
+    # level; its algorithmic work per launch is fi_w * N
     ach = fi_w * N / (ti_w * 1e-3)
     fa_e, fa_i = flops_alg(APPLY_K, True)
     apply64 = Na / ((ta_e64 + ta_i64) * 1e-3)
@@ -289,13 +289,12 @@ def run_gb300(args):
                                  "ms": float(np.mean(te)), "iterations": int(np.median(ite))},
                         "mixed": {"value": s_per_mdof(float(np.mean(te32)) * 1e-3, Ne), "unit": "s/MDoF",
                                   "ms": float(np.mean(te32)), "iterations": int(np.median(ite32))}},
-        "roofline": {"kernel": "dg_integrate_kernel<double,5,Cartesian> (finest level of the workload)",
+        "roofline": {"kernel": "dg_box_kernel<double,5> (finest level of the workload)",
                      "bound": "alu", "achieved": ach / 1e12, "peak": peak64 / 1e12, "unit": "TFLOP/s",
                      "frac": ach / peak64,
                      "traffic": DOMINANT_DRAM_BYTES_PER_DOF * N if DOMINANT_DRAM_BYTES_PER_DOF else None,
                      "traffic_source": DOMINANT_NCU_COMMAND,
-                     "ms_per_launch": ti_w, "eval_pass_ms_per_launch": te_w,
-                     "ops_per_dof": fi_w,
+                     "ms_per_launch": ti_w, "ops_per_dof": fi_w,
                      "peak_source": "FP64 FMA rate measured in this run (sipg_fma_peak, all SMs); "
                                     "152 SMs x 2 DFMA/clk x 2 flops x 2.07 GHz = 1.259 TFLOP/s by unit count"},
         "gpu_launches": int(launches),

@@ -304,7 +304,8 @@ sipg_status sipg_solve_host(sipg_ctx *ctx, const double *b_host, double *x_host,
 
 /* Per-launch device time of the last sipg_operator_apply-style launches
  * recorded with events on the context stream: the DG evaluation pass and the
- * DG integration pass, in milliseconds (for roofline accounting). */
+ * DG integration pass, in milliseconds (for roofline accounting).  On
+ * axis-aligned cells the operator is one pass, reported as the second. */
 sipg_status sipg_time_apply(sipg_ctx *ctx, int precision, const void *u_dev, void *v_dev,
                             int repeats, float *ms_eval, float *ms_integrate);
 

@@ -27,9 +27,29 @@ constexpr int kBatchThreads = 256;
 
 // this translation unit's copy of the 1D tables (constant memory is per unit)
 template <>
-void upload_tables_batch<double>(const Tables<double> &t) { upload_tables_tu(t); }
+void upload_tables_batch<double>(const Tables<double> &t, const BoxTables<double> &bt) {
+  upload_tables_tu(t);
+  upload_box_tu(bt);
+}
 template <>
-void upload_tables_batch<float>(const Tables<float> &t) { upload_tables_tu(t); }
+void upload_tables_batch<float>(const Tables<float> &t, const BoxTables<float> &bt) {
+  upload_tables_tu(t);
+  upload_box_tu(bt);
+}
+
+// an item of an axis-aligned problem: block w.cell0 of its mesh, the block's
+// shape packed in w.ncta (the plan's, whatever the problem's own launches use)
+static int pack_shape(const BoxShape &b) { return (b.w[0] - 1) | (b.w[1] - 1) << 1 | (b.w[2] - 1) << 2 | b.bricks << 3; }
+template <typename T, int N>
+__device__ __forceinline__ void dg_box_item(const DGArgs<T> &a, const WorkItem &w, unsigned char *sm) {
+  BoxShape b;
+  b.w[0] = (w.ncta & 1) + 1;
+  b.w[1] = ((w.ncta >> 1) & 1) + 1;
+  b.w[2] = ((w.ncta >> 2) & 1) + 1;
+  b.bricks = w.ncta >> 3;
+  const int wx = b.w[0] * b.bricks, nx = (a.m[0] + wx - 1) / wx, ny = (a.m[1] + b.w[1] - 1) / b.w[1], r = w.cell0 / nx;
+  dg_box_body<T, N>(a, vec_ptrs(a, 0), b, w.cell0 - r * nx, r % ny, r / ny, sm);
+}
 
 // segs (optional): the flexible-CG systems; a problem whose system has left
 // the iteration (segs[p].active == 0, set on the device) is skipped too
@@ -45,12 +65,14 @@ __global__ void __launch_bounds__(kBatchThreads, sizeof(T) == 4 ? 6 : 3)
     const WorkItem w = items[it];
     const BatchProb<T> &P = probs[w.p];
     if (P.active && (!segs || segs[w.p].active)) {
-#define SIPG_BATCH_CASE(NN)                                              \
-  case NN:                                                               \
-    if (INTEGRATE)                                                       \
-      dg_integrate_body<T, NN, CURVED>(P.a, vec_ptrs(P.a, 0), w.cell0, w.ncta, sm); \
-    else                                                                 \
-      dg_eval_body<T, NN, CURVED>(P.a, vec_ptrs(P.a, 0), w.cell0, w.ncta, sm); \
+#define SIPG_BATCH_CASE(NN)                                                          \
+  case NN:                                                                           \
+    if constexpr (!CURVED)                                                           \
+      dg_box_item<T, NN>(P.a, w, smem_raw);                                          \
+    else if constexpr (INTEGRATE)                                                    \
+      dg_integrate_body<T, NN>(P.a, vec_ptrs(P.a, 0), w.cell0, w.ncta, sm);          \
+    else                                                                             \
+      dg_eval_body<T, NN>(P.a, vec_ptrs(P.a, 0), w.cell0, w.ncta, sm);               \
     break;
       switch (P.n) {
         SIPG_BATCH_CASE(2)
@@ -233,8 +255,10 @@ cudaError_t launch_batch_fcg_cond(const int *any, cudaGraphConditionalHandle h, 
 // ------------------------------------------------------------------ host side
 
 template <typename T>
-cudaError_t batch_plan_build(BatchPlan<T> &P, const std::vector<DGArgs<T>> &args, const std::vector<int> &ns) {
+cudaError_t batch_plan_build(BatchPlan<T> &P, const std::vector<DGArgs<T>> &args, const std::vector<int> &ns,
+                             bool curved) {
   const int np = (int)args.size();
+  P.curved = curved;
   P.probs.resize(np);
   P.items.clear();
   size_t smem = 0;
@@ -243,13 +267,28 @@ cudaError_t batch_plan_build(BatchPlan<T> &P, const std::vector<DGArgs<T>> &args
     P.probs[p].n = ns[p];
     P.probs[p].active = 1;
     const int n = ns[p], cb = kBatchThreads / (n * n);
+    if (!curved) {   // the block shape of kBatchThreads threads
+      const BoxShape w = dg_box_shape<T>(n, args[p].m, cb * kBoxLanes<T>);
+      int nb = args[p].ncells > 0;
+      for (int d = 0; d < 3; ++d) {
+        const int wd = w.w[d] * (d == 0 ? w.bricks : 1);
+        nb *= (args[p].m[d] + wd - 1) / wd;
+      }
+      smem = std::max(smem, (size_t)box_groups<T>(w) * box_group_values(n) * 8);
+      for (int b = 0; b < nb; ++b) P.items.push_back({p, b, pack_shape(w)});
+      continue;
+    }
     smem = std::max(smem, (size_t)cb * cell_values(n) * sizeof(T));
     for (int c = 0; c < args[p].ncells; c += cb) P.items.push_back({p, c, std::min(cb, args[p].ncells - c)});
   }
   // longest items first (cost ~ cells x n^4), then static striding over the grid
   std::stable_sort(P.items.begin(), P.items.end(), [&](const WorkItem &x, const WorkItem &y) {
-    const double cx = (double)x.ncta * std::pow((double)ns[x.p], 4), cy = (double)y.ncta * std::pow((double)ns[y.p], 4);
-    return cx > cy;
+    auto cost = [&](const WorkItem &w) {
+      const int n = ns[w.p];
+      const double cells = curved ? w.ncta : kBatchThreads / (n * n);
+      return cells * std::pow((double)n, 4);
+    };
+    return cost(x) > cost(y);
   });
   P.smem = smem;
   cudaError_t e;
@@ -258,9 +297,9 @@ cudaError_t batch_plan_build(BatchPlan<T> &P, const std::vector<DGArgs<T>> &args
   if ((e = cudaMemcpy(P.d_items, P.items.data(), P.items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice)) !=
       cudaSuccess)
     return e;
-  auto k0 = dg_batched_kernel<T, false, false>, k1 = dg_batched_kernel<T, false, true>;
+  auto k1 = dg_batched_kernel<T, false, true>;
   auto k2 = dg_batched_kernel<T, true, false>, k3 = dg_batched_kernel<T, true, true>;
-  for (auto k : {k0, k1, k2, k3})
+  for (auto k : {k1, k2, k3})
     if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
       return e;
   int dev, nsm, occ = 1;
@@ -291,7 +330,7 @@ cudaError_t batch_apply(BatchPlan<T> &P, cudaStream_t s) {
                                   cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return e;
   if (P.items.empty()) return cudaSuccess;
-  if ((e = batch_dg_pass<T>(P, P.d_probs, false, nullptr, s)) != cudaSuccess) return e;
+  if (P.curved && (e = batch_dg_pass<T>(P, P.d_probs, false, nullptr, s)) != cudaSuccess) return e;
   return batch_dg_pass<T>(P, P.d_probs, true, nullptr, s);
 }
 
@@ -305,8 +344,7 @@ cudaError_t batch_dg_pass(const BatchPlan<T> &P, const BatchProb<T> *probs, bool
     if (integrate) dg_batched_kernel<T, true, true><<<P.grid, kBatchThreads, P.smem, s>>>(probs, P.d_items, ni, segs);
     else dg_batched_kernel<T, true, false><<<P.grid, kBatchThreads, P.smem, s>>>(probs, P.d_items, ni, segs);
   } else {
-    if (integrate) dg_batched_kernel<T, false, true><<<P.grid, kBatchThreads, P.smem, s>>>(probs, P.d_items, ni, segs);
-    else dg_batched_kernel<T, false, false><<<P.grid, kBatchThreads, P.smem, s>>>(probs, P.d_items, ni, segs);
+    dg_batched_kernel<T, false, true><<<P.grid, kBatchThreads, P.smem, s>>>(probs, P.d_items, ni, segs);
   }
   note_launch();
   return cudaGetLastError();
@@ -352,9 +390,9 @@ cudaError_t launch_vec_batched(const VecTask *tasks, const NodeItem *items, int 
 }
 
 template cudaError_t batch_plan_build<double>(BatchPlan<double> &, const std::vector<DGArgs<double>> &,
-                                              const std::vector<int> &);
+                                              const std::vector<int> &, bool);
 template cudaError_t batch_plan_build<float>(BatchPlan<float> &, const std::vector<DGArgs<float>> &,
-                                             const std::vector<int> &);
+                                             const std::vector<int> &, bool);
 template void batch_plan_free<double>(BatchPlan<double> &);
 template void batch_plan_free<float>(BatchPlan<float> &);
 template cudaError_t batch_apply<double>(BatchPlan<double> &, cudaStream_t);

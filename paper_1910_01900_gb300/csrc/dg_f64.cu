@@ -4,22 +4,31 @@
 namespace sipg {
 
 template <>
-void upload_tables_dg<double>(const Tables<double> &t) { upload_tables_tu(t); }
-template <>
-cudaError_t launch_dg_eval<double>(int n, bool curved, const DGArgs<double> &a, cudaStream_t s, int cb) {
-  return dispatch_dg<double>(0, 0, n, curved, &a, s, cb);
+void upload_tables_dg<double>(const Tables<double> &t, const BoxTables<double> &bt) {
+  upload_tables_tu(t);
+  upload_box_tu(bt);
 }
 template <>
-cudaError_t launch_dg_integrate<double>(int n, bool curved, const DGArgs<double> &a, cudaStream_t s, int cb) {
-  return dispatch_dg<double>(1, 0, n, curved, &a, s, cb);
+cudaError_t launch_dg_eval<double>(int n, const DGArgs<double> &a, cudaStream_t s, int cb) {
+  return dispatch_dg<double>(0, n, &a, s, cb);
 }
 template <>
-int dg_cells_per_block<double>(int n) { return default_cb(n); }
+cudaError_t launch_dg_integrate<double>(int n, const DGArgs<double> &a, cudaStream_t s, int cb) {
+  return dispatch_dg<double>(1, n, &a, s, cb);
+}
+template <>
+cudaError_t launch_dg_box<double>(int n, const DGArgs<double> &a, cudaStream_t s) {
+  return dispatch_dg<double>(2, n, &a, s, 0);
+}
+template <>
+BoxShape dg_box_shape<double>(int n, const int m[3], int cb) { return box_shape<double>(n, m, cb); }
+template <>
+int dg_cells_per_block<double>(int n, bool curved) { return curved ? default_cb(n) : box_default_cells<double>(n); }
 template <>
 int dg_max_cells_per_block<double>(int n) { return max_cb(n, sizeof(double)); }
 template <>
 cudaError_t dg_blocks_per_sm<double>(int n, bool curved, int pass, int cb, int *blocks) {
-  return dispatch_dg<double>(pass, 1, n, curved, nullptr, nullptr, cb, blocks);
+  return dispatch_dg<double>(3, n, nullptr, nullptr, cb, curved, pass == 1, blocks);
 }
 template <>
 cudaError_t prepare_dg_kernels<double>() { return prep_dg_all<double>(); }

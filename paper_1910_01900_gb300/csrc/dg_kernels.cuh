@@ -26,8 +26,11 @@
 // and on Dirichlet faces A = dA (2 tau_e u - q), B = -dA u; on Neumann faces
 // A = B = 0.  This is the per-side form of
 //   -{d_n v}[u] - [v]{d_n u} + tau [v][u]  and  -d_n v u - v d_n u + 2 tau v u.
+//
+// Axis-aligned cells take one pass (dg_box.cuh); these two serve curved cells,
+// structured or not.
 #pragma once
-#include "sumfac.cuh"
+#include "dg_box.cuh"
 
 namespace sipg {
 
@@ -70,18 +73,10 @@ __device__ __forceinline__ void interpolate_from_global(const T *__restrict__ uc
   }
 }
 
-template <typename T>
-struct VecPtrs {
-  const T *u;
-  T *out;
-  const T *x, *xp, *b;
-  T *grad, *trace;
-};
-
 // Evaluation pass for the cells cell0 .. cell0+ncta-1 of one problem, on a
 // thread block of blockDim.x >= ncta * N^2 threads with 4 ncta N^3 values of
 // shared memory at sm.  Shared by the per-problem and the batched kernels.
-template <typename T, int N, bool CURVED, bool UNSTR = false>
+template <typename T, int N, bool UNSTR = false>
 __device__ __forceinline__ void dg_eval_body(const DGArgs<T> &a, const VecPtrs<T> &v, const int cell0, const int ncta, T *sm) {
   constexpr int N2 = N * N, N3 = N2 * N, TT = Tile<N>::T3;
   const int NT = blockDim.x;
@@ -90,37 +85,24 @@ __device__ __forceinline__ void dg_eval_body(const DGArgs<T> &a, const VecPtrs<T
   T *su = sm + cl * Tile<N>::CS;
 
   interpolate_from_global<T, N>(v.u + (size_t)(cell0 + (act ? cl : 0)) * N3, su, act, l);
-  // the gradient at the Gauss points (curved cells: the metric mixes its
-  // components; an axis-aligned cell needs none of it here: its normal
-  // derivatives come from the values through D^T l below, and its cell term
-  // from the values through the collocation stiffness in the integration pass)
-  if constexpr (CURVED) {
-    if (act) {
+  // the gradient at the Gauss points
+  if (act) {
 #pragma unroll 1
-      for (int d = 0; d < 3; ++d) {
-        int base, stride;
-        line_of<N>(d, l, base, stride);
-        T x[N], y[N];
-        load_line<T, N>(su, base, stride, x);
-        apply_mat<T, N, MD>(x, y);
-        store_line<T, N>(su + (1 + d) * TT, base, stride, y);
-      }
+    for (int d = 0; d < 3; ++d) {
+      int base, stride;
+      line_of<N>(d, l, base, stride);
+      T x[N], y[N];
+      load_line<T, N>(su, base, stride, x);
+      apply_mat<T, N, MD>(x, y);
+      store_line<T, N>(su + (1 + d) * TT, base, stride, y);
     }
-    __syncthreads();
   }
+  __syncthreads();
   if (!a.recompute) {
-    if constexpr (CURVED) {
-      T *gg = v.grad + (size_t)cell0 * 3 * N3;
-      for (int i = tid; i < ncta * 3 * N3; i += NT) {
-        const int c = i / (3 * N3), r = i - c * 3 * N3, comp = r / N3;
-        gg[i] = sm[c * Tile<N>::CS + (1 + comp) * TT + Tile<N>::idx(r - comp * N3)];
-      }
-    } else {   // the values at the Gauss points, [cell][n^3]
-      T *gg = v.grad + (size_t)cell0 * N3;
-      for (int i = tid; i < ncta * N3; i += NT) {
-        const int c = i / N3;
-        gg[i] = sm[c * Tile<N>::CS + Tile<N>::idx(i - c * N3)];
-      }
+    T *gg = v.grad + (size_t)cell0 * 3 * N3;
+    for (int i = tid; i < ncta * 3 * N3; i += NT) {
+      const int c = i / (3 * N3), r = i - c * 3 * N3, comp = r / N3;
+      gg[i] = sm[c * Tile<N>::CS + (1 + comp) * TT + Tile<N>::idx(r - comp * N3)];
     }
   }
   if (!act) return;
@@ -144,47 +126,34 @@ __device__ __forceinline__ void dg_eval_body(const DGArgs<T> &a, const VecPtrs<T
       v0 = fma(t.l0[N][q], x[q], v0);
       v1 = fma(t.l1[N][q], x[q], v1);
     }
-    T q0, q1;
-    if constexpr (!CURVED) {
-      // l_s . (D x) = (D^T l_s) . x: the normal derivative from the values
-      T g0 = t.dl0[N][0] * x[0], g1 = t.dl1[N][0] * x[0];
+    T gr0[3], gr1[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      T g[N];
+      load_line<T, N>(su + (1 + b) * TT, base, stride, g);
+      T g0 = t.l0[N][0] * g[0], g1 = t.l1[N][0] * g[0];
 #pragma unroll
       for (int q = 1; q < N; ++q) {
-        g0 = fma(t.dl0[N][q], x[q], g0);
-        g1 = fma(t.dl1[N][q], x[q], g1);
+        g0 = fma(t.l0[N][q], g[q], g0);
+        g1 = fma(t.l1[N][q], g[q], g1);
       }
-      q0 = -a.ih[d] * g0;
-      q1 = a.ih[d] * g1;
-    } else {
-      T gr0[3], gr1[3];
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        T g[N];
-        load_line<T, N>(su + (1 + b) * TT, base, stride, g);
-        T g0 = t.l0[N][0] * g[0], g1 = t.l1[N][0] * g[0];
-#pragma unroll
-        for (int q = 1; q < N; ++q) {
-          g0 = fma(t.l0[N][q], g[q], g0);
-          g1 = fma(t.l1[N][q], g[q], g1);
-        }
-        gr0[b] = g0;
-        gr1[b] = g1;
-      }
-      const T *c0, *c1;
-      if constexpr (UNSTR) {   // own side's J^-1 n of the faces xi_d = 0 and xi_d = 1
-        c0 = a.fc[0] + ((size_t)cell * 6 + 2 * d) * 3 * N2 + l;
-        c1 = c0 + 3 * N2;
-      } else {
-        const int t1 = d == 0 ? 1 : 0, t2 = d == 2 ? 1 : 2;
-        const size_t nfp = (size_t)a.m[t1] * a.m[t2];
-        const size_t f0 = (size_t)ijk[d] * nfp + ijk[t1] + (size_t)a.m[t1] * ijk[t2];
-        const size_t f1 = f0 + nfp;
-        c0 = a.fc[d] + (f0 * 2 + 1) * 3 * N2 + l;   // this cell is the upper cell of plane i_d
-        c1 = a.fc[d] + (f1 * 2 + 0) * 3 * N2 + l;   // and the lower cell of plane i_d+1
-      }
-      q0 = c0[0] * gr0[0] + c0[N2] * gr0[1] + c0[2 * N2] * gr0[2];
-      q1 = c1[0] * gr1[0] + c1[N2] * gr1[1] + c1[2 * N2] * gr1[2];
+      gr0[b] = g0;
+      gr1[b] = g1;
     }
+    const T *c0, *c1;
+    if constexpr (UNSTR) {   // own side's J^-1 n of the faces xi_d = 0 and xi_d = 1
+      c0 = a.fc[0] + ((size_t)cell * 6 + 2 * d) * 3 * N2 + l;
+      c1 = c0 + 3 * N2;
+    } else {
+      const int t1 = d == 0 ? 1 : 0, t2 = d == 2 ? 1 : 2;
+      const size_t nfp = (size_t)a.m[t1] * a.m[t2];
+      const size_t f0 = (size_t)ijk[d] * nfp + ijk[t1] + (size_t)a.m[t1] * ijk[t2];
+      const size_t f1 = f0 + nfp;
+      c0 = a.fc[d] + (f0 * 2 + 1) * 3 * N2 + l;   // this cell is the upper cell of plane i_d
+      c1 = a.fc[d] + (f1 * 2 + 0) * 3 * N2 + l;   // and the lower cell of plane i_d+1
+    }
+    const T q0 = c0[0] * gr0[0] + c0[N2] * gr0[1] + c0[2 * N2] * gr0[2];
+    const T q1 = c1[0] * gr1[0] + c1[N2] * gr1[1] + c1[2 * N2] * gr1[2];
     T *tr = v.trace + ((size_t)cell * 6 + 2 * d) * 2 * N2 + l;
     tr[0] = v0;
     tr[N2] = q0;
@@ -194,7 +163,7 @@ __device__ __forceinline__ void dg_eval_body(const DGArgs<T> &a, const VecPtrs<T
 }
 
 // Integration pass (same thread and shared-memory contract as the evaluation).
-template <typename T, int N, bool CURVED, bool UNSTR = false>
+template <typename T, int N, bool UNSTR = false>
 __device__ __forceinline__ void dg_integrate_body(const DGArgs<T> &a, const VecPtrs<T> &v, const int cell0, const int ncta,
                                                   T *sm) {
   constexpr int N2 = N * N, N3 = N2 * N, TT = Tile<N>::T3;
@@ -202,25 +171,9 @@ __device__ __forceinline__ void dg_integrate_body(const DGArgs<T> &a, const VecP
   const int tid = threadIdx.x, cl = tid / N2, l = tid - cl * N2;
   const bool act = cl < ncta;
   T *st = sm + cl * Tile<N>::CS;   // value accumulator, then the integrated tile
-  T *sg = st + TT;            // three gradient components (curved); the values (axis-aligned)
+  T *sg = st + TT;            // three gradient components
 
-  if constexpr (!CURVED) {
-    // An axis-aligned cell's term is sum_d alpha_d (D_d^T W D_d) applied to
-    // the values at the Gauss points; W is a tensor product, so along a line
-    // of direction d it is the collocation stiffness KG = D^T diag(w) D times
-    // the line's weight alpha_d w_t1 w_t2: one product per direction (with the
-    // face terms below) instead of a derivative and a transposed derivative.
-    if (a.recompute) {
-      interpolate_from_global<T, N>(v.u + (size_t)(cell0 + (act ? cl : 0)) * N3, sg, act, l);
-    } else {
-      const T *gg = v.grad + (size_t)cell0 * N3;
-      for (int i = tid; i < ncta * N3; i += NT) {
-        const int c = i / N3;
-        sm[c * Tile<N>::CS + TT + Tile<N>::idx(i - c * N3)] = gg[i];
-      }
-      __syncthreads();
-    }
-  } else if (a.recompute) {
+  if (a.recompute) {
     // gradient at the Gauss points again from u: 3 interpolation and 3
     // collocation-derivative sweeps (the value slot st is free until the faces)
     interpolate_from_global<T, N>(v.u + (size_t)(cell0 + (act ? cl : 0)) * N3, st, act, l);
@@ -242,20 +195,18 @@ __device__ __forceinline__ void dg_integrate_body(const DGArgs<T> &a, const VecP
       sm[c * Tile<N>::CS + (1 + comp) * TT + Tile<N>::idx(r - comp * N3)] = gg[i];
     }
   }
-  if constexpr (CURVED) {
-    __syncthreads();
-    for (int i = tid; i < ncta * N3; i += NT) {
-      const int c = i / N3, p = i - c * N3, tp = Tile<N>::idx(p);
-      T *s = sm + c * Tile<N>::CS + TT + tp;
-      const T g0 = s[0], g1 = s[TT], g2 = s[2 * TT];
-      const T *M = a.metric + (size_t)(cell0 + c) * 6 * N3 + p;
-      const T xx = M[0], yy = M[N3], zz = M[2 * N3], xy = M[3 * N3], xz = M[4 * N3], yz = M[5 * N3];
-      s[0] = xx * g0 + xy * g1 + xz * g2;
-      s[TT] = xy * g0 + yy * g1 + yz * g2;
-      s[2 * TT] = xz * g0 + yz * g1 + zz * g2;
-    }
-    __syncthreads();
+  __syncthreads();
+  for (int i = tid; i < ncta * N3; i += NT) {
+    const int c = i / N3, p = i - c * N3, tp = Tile<N>::idx(p);
+    T *s = sm + c * Tile<N>::CS + TT + tp;
+    const T g0 = s[0], g1 = s[TT], g2 = s[2 * TT];
+    const T *M = a.metric + (size_t)(cell0 + c) * 6 * N3 + p;
+    const T xx = M[0], yy = M[N3], zz = M[2 * N3], xy = M[3 * N3], xz = M[4 * N3], yz = M[5 * N3];
+    s[0] = xx * g0 + xy * g1 + xz * g2;
+    s[TT] = xy * g0 + yy * g1 + yz * g2;
+    s[2 * TT] = xz * g0 + yz * g1 + zz * g2;
   }
+  __syncthreads();
 
   const int cell = cell0 + cl;
   // cell coordinates and strides as scalars picked by direction (indexing a
@@ -311,17 +262,12 @@ __device__ __forceinline__ void dg_integrate_body(const DGArgs<T> &a, const VecP
           }
           continue;
         }
-        T dA;
         const size_t face = (size_t)(ijk(d) + s) * nfp + ftan;
-        if constexpr (CURVED) {
-          dA = a.fdA[d][face * N2 + l];
-          const T *c = a.fc[d] + (face * 2 + (s ? 0 : 1)) * 3 * N2 + l;
-          cvec[s][0] = c[0];
-          cvec[s][1] = c[N2];
-          cvec[s][2] = c[2 * N2];
-        } else {
-          dA = a.fwcart[d * N2 + l];
-        }
+        const T dA = a.fdA[d][face * N2 + l];
+        const T *c = a.fc[d] + (face * 2 + (s ? 0 : 1)) * 3 * N2 + l;
+        cvec[s][0] = c[0];
+        cvec[s][1] = c[N2];
+        cvec[s][2] = c[2 * N2];
         const bool has_nb = s ? (ijk(d) < mdim(d) - 1) : (ijk(d) > 0);
         if (has_nb) {
           const int nb = cell + (s ? cstride(d) : -cstride(d));
@@ -347,27 +293,9 @@ __device__ __forceinline__ void dg_integrate_body(const DGArgs<T> &a, const VecP
       // next; D^T applied to l_s is the fixed vector dl_s, so that term goes
       // into the value tile here as dl_s(q) times the coefficient (one
       // read-modify-write line less per direction, the same sum).
-      T bn0, bn1;
-      if constexpr (!CURVED) {
-        bn0 = -a.ih[d] * B[0];
-        bn1 = a.ih[d] * B[1];
-      } else {
-        bn0 = (d == 0 ? cvec[0][0] : (d == 1 ? cvec[0][1] : cvec[0][2])) * B[0];
-        bn1 = (d == 0 ? cvec[1][0] : (d == 1 ? cvec[1][1] : cvec[1][2])) * B[1];
-      }
-      if constexpr (!CURVED && sizeof(T) == 4) {
-        // the cell term along this line: KG times the line's weight, with the faces
-        T x[N], y[N];
-        load_line<T, N>(sg, base, stride, x);
-        apply_mat<T, N, MKG>(x, y);
-        const T cw = a.fwcart[d * N2 + l] * a.ih[d];
-#pragma unroll
-        for (int q = 0; q < N; ++q) {
-          T *p = st + base + q * stride;
-          const T f = fma(t.l0[N][q], A[0], fma(t.l1[N][q], A[1], fma(t.dl0[N][q], bn0, t.dl1[N][q] * bn1)));
-          *p = fma(cw, y[q], d == 0 ? f : f + *p);
-        }
-      } else if (d == 0) {
+      const T bn0 = (d == 0 ? cvec[0][0] : (d == 1 ? cvec[0][1] : cvec[0][2])) * B[0];
+      const T bn1 = (d == 0 ? cvec[1][0] : (d == 1 ? cvec[1][1] : cvec[1][2])) * B[1];
+      if (d == 0) {
 #pragma unroll
         for (int q = 0; q < N; ++q)
           st[base + q * stride] = fma(t.l0[N][q], A[0], fma(t.l1[N][q], A[1], fma(t.dl0[N][q], bn0, t.dl1[N][q] * bn1)));
@@ -378,54 +306,33 @@ __device__ __forceinline__ void dg_integrate_body(const DGArgs<T> &a, const VecP
           *p = fma(t.l0[N][q], A[0], fma(t.l1[N][q], A[1], fma(t.dl0[N][q], bn0, fma(t.dl1[N][q], bn1, *p))));
         }
       }
-      if constexpr (CURVED) {
-        // the tangential gradient components (J^-1 n has all three)
+      // the tangential gradient components (J^-1 n has all three)
 #pragma unroll
-        for (int bb = 0; bb < 3; ++bb) {
-          if (bb == d) continue;
-          const T b0 = cvec[0][bb] * B[0], b1 = cvec[1][bb] * B[1];
-          T *g = sg + bb * TT;
+      for (int bb = 0; bb < 3; ++bb) {
+        if (bb == d) continue;
+        const T b0 = cvec[0][bb] * B[0], b1 = cvec[1][bb] * B[1];
+        T *g = sg + bb * TT;
 #pragma unroll
-          for (int q = 0; q < N; ++q) {
-            T *p = g + base + q * stride;
-            *p = fma(t.l0[N][q], b0, fma(t.l1[N][q], b1, *p));
-          }
+        for (int q = 0; q < N; ++q) {
+          T *p = g + base + q * stride;
+          *p = fma(t.l0[N][q], b0, fma(t.l1[N][q], b1, *p));
         }
       }
     }
     __syncthreads();
   }
-  if constexpr (CURVED) {
 #pragma unroll 1
-    for (int d = 0; d < 3; ++d) {
-      if (act) {
-        int base, stride;
-        line_of<N>(d, l, base, stride);
-        T x[N], y[N];
-        load_line<T, N>(sg + d * TT, base, stride, x);
-        apply_mat<T, N, MDt>(x, y);
+  for (int d = 0; d < 3; ++d) {
+    if (act) {
+      int base, stride;
+      line_of<N>(d, l, base, stride);
+      T x[N], y[N];
+      load_line<T, N>(sg + d * TT, base, stride, x);
+      apply_mat<T, N, MDt>(x, y);
 #pragma unroll
-        for (int q = 0; q < N; ++q) st[base + q * stride] += y[q];
-      }
-      __syncthreads();
+      for (int q = 0; q < N; ++q) st[base + q * stride] += y[q];
     }
-  } else if constexpr (sizeof(T) == 8) {
-    // FP64: the cell term after the faces (within the face loop the sweep's
-    // registers and the face coefficients' would not fit together)
-#pragma unroll 1
-    for (int d = 0; d < 3; ++d) {
-      if (act) {
-        int base, stride;
-        line_of<N>(d, l, base, stride);
-        T x[N], y[N];
-        load_line<T, N>(sg, base, stride, x);
-        apply_mat<T, N, MKG>(x, y);
-        const T cw = a.fwcart[d * N2 + l] * a.ih[d];
-#pragma unroll
-        for (int q = 0; q < N; ++q) st[base + q * stride] = fma(cw, y[q], st[base + q * stride]);
-      }
-      __syncthreads();
-    }
+    __syncthreads();
   }
 #pragma unroll 1
   for (int d = 0; d < 2; ++d) {
@@ -491,21 +398,35 @@ __device__ __forceinline__ VecPtrs<T> vec_ptrs(const DGArgs<T> &a, const int r) 
 template <typename T>
 constexpr int kMinCellBlocks = sizeof(T) == 4 ? 2 : 1;
 
-template <typename T, int N, bool CURVED, bool MULTI>
+template <typename T, int N, bool MULTI>
 __global__ void __launch_bounds__(kCellThreads, kMinCellBlocks<T>) dg_eval_kernel(const DGArgs<T> a, const int cb) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int grp = MULTI ? blockIdx.x / a.nv : blockIdx.x, vec = MULTI ? blockIdx.x - grp * a.nv : 0;
   const int cell0 = grp * cb;
-  dg_eval_body<T, N, CURVED>(a, vec_ptrs(a, vec), cell0, min(cb, a.ncells - cell0), reinterpret_cast<T *>(smem_raw));
+  dg_eval_body<T, N>(a, vec_ptrs(a, vec), cell0, min(cb, a.ncells - cell0), reinterpret_cast<T *>(smem_raw));
 }
 
-template <typename T, int N, bool CURVED, bool MULTI>
+template <typename T, int N, bool MULTI>
 __global__ void __launch_bounds__(kCellThreads, kMinCellBlocks<T>) dg_integrate_kernel(const DGArgs<T> a, const int cb) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int grp = MULTI ? blockIdx.x / a.nv : blockIdx.x, vec = MULTI ? blockIdx.x - grp * a.nv : 0;
   const int cell0 = grp * cb;
-  dg_integrate_body<T, N, CURVED>(a, vec_ptrs(a, vec), cell0, min(cb, a.ncells - cell0),
+  dg_integrate_body<T, N>(a, vec_ptrs(a, vec), cell0, min(cb, a.ncells - cell0),
                                   reinterpret_cast<T *>(smem_raw));
+}
+
+// Axis-aligned cells: one pass; grid x, y, z are the blocks of a.box from oy,
+// oz on (MULTI: nz blocks of each vector behind one another).
+template <typename T, int N, bool MULTI>
+__global__ void __launch_bounds__(kCellThreads) dg_box_kernel(const DGArgs<T> a, const int oy, const int oz,
+                                                              const int nz) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  int gz = blockIdx.z, vec = 0;
+  if constexpr (MULTI) {
+    vec = gz / nz;
+    gz -= vec * nz;
+  }
+  dg_box_body<T, N>(a, vec_ptrs(a, vec), a.box, blockIdx.x, oy + blockIdx.y, oz + gz, smem_raw);
 }
 
 // Unstructured meshes: single-vector passes with general (curved) cell and
@@ -514,7 +435,7 @@ template <typename T, int N>
 __global__ void __launch_bounds__(kCellThreads, kMinCellBlocks<T>) dg_eval_unstr_kernel(const DGArgs<T> a, const int cb) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int cell0 = blockIdx.x * cb;
-  dg_eval_body<T, N, true, true>(a, vec_ptrs(a, 0), cell0, min(cb, a.ncells - cell0), reinterpret_cast<T *>(smem_raw));
+  dg_eval_body<T, N, true>(a, vec_ptrs(a, 0), cell0, min(cb, a.ncells - cell0), reinterpret_cast<T *>(smem_raw));
 }
 
 template <typename T, int N>
@@ -522,7 +443,7 @@ __global__ void __launch_bounds__(kCellThreads, kMinCellBlocks<T>) dg_integrate_
                                                                                             const int cb) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int cell0 = blockIdx.x * cb;
-  dg_integrate_body<T, N, true, true>(a, vec_ptrs(a, 0), cell0, min(cb, a.ncells - cell0),
+  dg_integrate_body<T, N, true>(a, vec_ptrs(a, 0), cell0, min(cb, a.ncells - cell0),
                                       reinterpret_cast<T *>(smem_raw));
 }
 

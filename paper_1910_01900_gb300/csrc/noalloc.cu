@@ -5,10 +5,10 @@
 // reserved the device memory for itself, or a time-stepping loop that must
 // not allocate (or synchronize on an allocation) once it has started.  This
 // entry point serves them: the caller passes only the input and output
-// vectors, and the scratch that the two DG passes need (reference gradients,
-// face traces, penalty and weight tables) lives in one file-scope device
-// array of fixed size, allocated by the CUDA runtime when the library is
-// loaded and held by every GPU that loads it until the process exits.
+// vectors, and the scratch that the DG pass needs (the penalties) lives in one
+// file-scope device array of fixed size, allocated by the CUDA runtime when
+// the library is loaded and held by every GPU that loads it until the process
+// exits.
 //
 // Host code cannot use the array's name as a device address (in host code it
 // is only a host-side stand-in; a kernel given it would fault or, where the
@@ -21,54 +21,38 @@
 
 namespace {
 
-// Maximum scratch: 64 MiB (enough for about 1.4 million DoF at k = 3).
+// Largest problem: what 64 MiB of gradients, traces and tables would hold
+// (about 1.4 million DoF at k = 3), the limit of this entry point.  The one
+// pass of axis-aligned cells needs the penalties alone, 8 of at least 584
+// bytes per cell by that count.
 constexpr size_t kScratchBytes = size_t(64) << 20;
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
+static __device__ __align__(256) double g_noalloc_tau[kScratchBytes / 584 + 32];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 void *g_scratch_addr[kMaxDevices] = {};
 
-struct Weights1D {
-  double w[sipg::kMaxN];
-};
-
-// Cartesian cell and face weights and the penalty tau_e (Section 2, same
-// definitions as the context path) written into the scratch.
-__global__ void noalloc_prep_kernel(double *wcart, double *fwcart, double *tau, int n, Weights1D W, double h0,
-                                    double h1, double h2, int m0, int m1, int m2, double factor) {
-  const int n2 = n * n, n3 = n2 * n;
+// The penalty tau_e (Section 2, same definition as the context path) of every
+// cell, written into the scratch.
+__global__ void noalloc_prep_kernel(double *tau, int n, double h0, double h1, double h2, int m0, int m1, int m2,
+                                    double factor) {
   const double h[3] = {h0, h1, h2};
   const int m[3] = {m0, m1, m2};
   const double vol = h0 * h1 * h2;
   const long ncells = (long)m0 * m1 * m2;
-  const long total = 3L * n3 + 3L * n2 + ncells;
-  for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
-    if (idx < 3L * n3) {
-      const int d = (int)(idx / n3), p = (int)(idx - (long)d * n3);
-      const int i = p % n, j = (p / n) % n, k = p / n2;
-      const double w = W.w[i] * W.w[j] * W.w[k];
-      wcart[idx] = w * vol / (h[d] * h[d]);
-    } else if (idx < 3L * n3 + 3L * n2) {
-      const long r = idx - 3L * n3;
-      const int d = (int)(r / n2), l = (int)(r - (long)d * n2);
+  for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < ncells; e += (long)gridDim.x * blockDim.x) {
+    const int ijk[3] = {(int)(e % m0), (int)((e / m0) % m1), (int)(e / ((long)m0 * m1))};
+    double a_int = 0, a_bd = 0;
+    for (int d = 0; d < 3; ++d) {
       const int t1 = d == 0 ? 1 : 0, t2 = d == 2 ? 1 : 2;
-      fwcart[r] = W.w[l % n] * W.w[l / n] * h[t1] * h[t2];
-    } else {
-      const long e = idx - 3L * n3 - 3L * n2;
-      const int ijk[3] = {(int)(e % m0), (int)((e / m0) % m1), (int)(e / ((long)m0 * m1))};
-      double a_int = 0, a_bd = 0;
-      for (int d = 0; d < 3; ++d) {
-        const int t1 = d == 0 ? 1 : 0, t2 = d == 2 ? 1 : 2;
-        const double area = h[t1] * h[t2];
-        for (int s = 0; s < 2; ++s) {
-          const bool bd = s ? (ijk[d] == m[d] - 1) : (ijk[d] == 0);
-          if (bd) a_bd += area;
-          else a_int += area;
-        }
+      const double area = h[t1] * h[t2];
+      for (int s = 0; s < 2; ++s) {
+        const bool bd = s ? (ijk[d] == m[d] - 1) : (ijk[d] == 0);
+        if (bd) a_bd += area;
+        else a_int += area;
       }
-      tau[e] = factor * (double)n * n * (0.5 * a_int + a_bd) / vol;
     }
+    tau[e] = factor * (double)n * n * (0.5 * a_int + a_bd) / vol;
   }
 }
 
@@ -137,15 +121,19 @@ extern "C" sipg_status sipg_operator_apply_noalloc(const sipg_mesh *mesh, int de
     if (!g_scratch_addr[dev]) {
       // set-up, once per device, with that device current
       void *p = nullptr;
-      const cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
+      const cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_tau);
       if (e != cudaSuccess || !p) {
         sipg::set_global_error(std::string("cudaGetSymbolAddress failed: ") + cudaGetErrorString(e));
         return SIPG_ECUDA;
       }
       static Tables<double> tab;
+      static BoxTables<double> box;
       static std::once_flag built;
-      std::call_once(built, [] { build_tables(tab); });
-      upload_tables_dg<double>(tab);
+      std::call_once(built, [] {
+        build_tables(tab);
+        build_box_tables(box);
+      });
+      upload_tables_dg<double>(tab, box);
       cudaError_t ue = cudaGetLastError();
       if (ue == cudaSuccess) ue = prepare_dg_kernels<double>();
       if (ue != cudaSuccess) {
@@ -157,21 +145,13 @@ extern "C" sipg_status sipg_operator_apply_noalloc(const sipg_mesh *mesh, int de
     base = (unsigned char *)g_scratch_addr[dev];
   }
   cudaStream_t s = (cudaStream_t)stream;
-  double *grad = (double *)base;
-  double *trace = (double *)(base + b_grad);
-  double *tau = (double *)(base + b_grad + b_trace);
-  double *wcart = (double *)(base + b_grad + b_trace + b_tau);
-  double *fwcart = (double *)(base + b_grad + b_trace + b_tau + b_w);
-  const Rules1D &r = rules(n);
-  Weights1D W{};
-  for (int i = 0; i < n; ++i) W.w[i] = r.wq[i];
+  double *tau = (double *)base;
   double h[3];
   for (int d = 0; d < 3; ++d) h[d] = (mesh->hi[d] - mesh->lo[d]) / mesh->m[d];
-  const long total = 3L * n3 + 3L * n2 + E;
   const int bs = 256;
-  const int grid = (int)std::min<long>((total + bs - 1) / bs, 152L * 8);
-  noalloc_prep_kernel<<<grid, bs, 0, s>>>(wcart, fwcart, tau, n, W, h[0], h[1], h[2], mesh->m[0], mesh->m[1],
-                                          mesh->m[2], penalty_factor);
+  const int grid = (int)std::min<long long>((E + bs - 1) / bs, 152LL * 8);
+  noalloc_prep_kernel<<<grid, bs, 0, s>>>(tau, n, h[0], h[1], h[2], mesh->m[0], mesh->m[1], mesh->m[2],
+                                          penalty_factor);
   note_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
@@ -181,20 +161,14 @@ extern "C" sipg_status sipg_operator_apply_noalloc(const sipg_mesh *mesh, int de
   DGArgs<double> a{};
   a.u = u_dev;
   a.out = v_dev;
-  a.grad = grad;
-  a.trace = trace;
-  a.wcart = wcart;
-  a.fwcart = fwcart;
   a.tau = tau;
-  for (int d = 0; d < 3; ++d) {
-    a.ih[d] = 1.0 / h[d];
-    a.m[d] = mesh->m[d];
-  }
+  for (int d = 0; d < 3; ++d) a.m[d] = mesh->m[d];
+  dg_box_scales(a, h);
+  a.box = dg_box_shape<double>(n, a.m, 0);
   a.ncells = (int)E;
   for (int q = 0; q < 6; ++q) a.bc[q] = mesh->bc[q];
   a.mode = 0;
-  e = launch_dg_eval<double>(n, false, a, s);
-  if (e == cudaSuccess) e = launch_dg_integrate<double>(n, false, a, s);
+  e = launch_dg_box<double>(n, a, s);
   if (e != cudaSuccess) {
     sipg::set_global_error(std::string("launch failed: ") + cudaGetErrorString(e));
     return SIPG_ECUDA;

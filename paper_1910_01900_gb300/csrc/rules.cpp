@@ -124,6 +124,73 @@ void even_odd(const std::vector<double> &M, int n, int par, double *E, double *O
   (void)par;
 }
 
+// 1D mass and stiffness matrices of the GL basis under the Gauss rule
+void mass_stiffness(const Rules1D &r, std::vector<double> &M1, std::vector<double> &K1) {
+  const int n = r.n;
+  M1.assign(n * n, 0.0);
+  K1.assign(n * n, 0.0);
+  for (int i = 0; i < n; ++i)
+    for (int j = 0; j < n; ++j)
+      for (int q = 0; q < n; ++q) {
+        M1[i * n + j] += r.wq[q] * r.S[q * n + i] * r.S[q * n + j];
+        K1[i * n + j] += r.wq[q] * r.Sd[q * n + i] * r.Sd[q * n + j];
+      }
+}
+
+void set(double &to, long double v) { to = (double)v; }
+void set(F2 &to, long double v) { to.x = to.y = (float)v; }
+
+// The line operator of axis-aligned cells: M1^-1 applied (in long double, by
+// elimination; M1 is positive definite) to K1 with the own parts of the
+// fluxes and to the end columns; see BoxTables.
+template <typename T>
+void box_tables(const Rules1D &r, const std::vector<double> &M1, const std::vector<double> &K1,
+                BoxTables<T> &t) {
+  const int n = r.n, s = n - 2, h = n / 2, hc = (n + 1) / 2, w = n + 2;
+  std::vector<double> q0(n), q1(n);
+  for (int j = 0; j < n; ++j) {
+    q0[j] = -r.lp0[j];
+    q1[j] = r.lp1[j];
+    set(t.qh[s][j], 0.5L * q1[j]);
+  }
+  // columns 0..n-1: the matrix; n: e_0; n + 1: q_0 / 2
+  std::vector<long double> A(M1.begin(), M1.end()), B((size_t)n * w, 0.0L);
+  for (int i = 0; i < n; ++i) {
+    for (int j = 0; j < n; ++j) {
+      long double v = K1[i * n + j];
+      v -= 0.5L * ((i == 0 ? q0[j] : 0.0) + (j == 0 ? q0[i] : 0.0));
+      v -= 0.5L * ((i == n - 1 ? q1[j] : 0.0) + (j == n - 1 ? q1[i] : 0.0));
+      B[i * w + j] = v;
+    }
+    B[i * w + n] = i == 0 ? 1.0L : 0.0L;
+    B[i * w + n + 1] = 0.5L * q0[i];
+  }
+  for (int k = 0; k < n; ++k)
+    for (int i = 0; i < n; ++i) {
+      if (i == k) continue;
+      const long double f = A[i * n + k] / A[k * n + k];
+      for (int j = 0; j < n; ++j) A[i * n + j] -= f * A[k * n + j];
+      for (int j = 0; j < w; ++j) B[i * w + j] -= f * B[k * w + j];
+    }
+  for (int i = 0; i < n; ++i)
+    for (int j = 0; j < w; ++j) B[i * w + j] /= A[i * n + i];
+  for (int i = 0; i < hc; ++i) {
+    const int m = n - 1 - i;
+    for (int j = 0; j < hc; ++j) {
+      const int k = n - 1 - j;   // the middle column stands for itself
+      set(t.HE[s][i * 7 + j], j == k ? B[i * w + j] : 0.5L * (B[i * w + j] + B[i * w + k]));
+      set(t.ME[s][i * 5 + j], j == k ? (long double)M1[i * n + j] : 0.5L * ((long double)M1[i * n + j] + M1[i * n + k]));
+      if (i >= h || j >= h) continue;
+      set(t.HO[s][i * 6 + j], 0.5L * (B[i * w + j] - B[i * w + k]));
+      set(t.MO[s][i * 4 + j], 0.5L * ((long double)M1[i * n + j] - M1[i * n + k]));
+    }
+    for (int c = 0; c < 2; ++c) {   // the lower end's column; the upper end's is its mirror image
+      set(t.HE[s][i * 7 + hc + c], 0.5L * (B[i * w + n + c] + B[m * w + n + c]));
+      if (i < h) set(t.HO[s][i * 6 + h + c], 0.5L * (B[i * w + n + c] - B[m * w + n + c]));
+    }
+  }
+}
+
 }  // namespace
 
 void gauss_rule(int n, std::vector<double> &x, std::vector<double> &w) { x = gauss_points(n, w); }
@@ -188,13 +255,8 @@ void build_tables(Tables<T> &t) {
     put(St, +1, t.StE[n], t.StO[n]);
     put(r.D, -1, t.DE[n], t.DO[n]);
     put(Dt, -1, t.DtE[n], t.DtO[n]);
-    std::vector<double> M1(n * n, 0.0), K1(n * n, 0.0);
-    for (int i = 0; i < n; ++i)
-      for (int j = 0; j < n; ++j)
-        for (int q = 0; q < n; ++q) {
-          M1[i * n + j] += r.wq[q] * r.S[q * n + i] * r.S[q * n + j];
-          K1[i * n + j] += r.wq[q] * r.Sd[q * n + i] * r.Sd[q * n + j];
-        }
+    std::vector<double> M1, K1;
+    mass_stiffness(r, M1, K1);
     if (n <= 4)
       for (int i = 0; i < n * n; ++i) {
         t.M1[n][i] = (T)M1[i];
@@ -202,13 +264,6 @@ void build_tables(Tables<T> &t) {
       }
     put(M1, +1, t.M1E[n], t.M1O[n]);
     put(K1, +1, t.K1E[n], t.K1O[n]);
-    std::vector<double> KG(n * n, 0.0);
-    for (int i = 0; i < n; ++i)
-      for (int j = 0; j < n; ++j)
-        for (int q = 0; q < n; ++q) KG[i * n + j] += r.D[q * n + i] * r.wq[q] * r.D[q * n + j];
-    if (n <= 4)
-      for (int i = 0; i < n * n; ++i) t.KG[n][i] = (T)KG[i];
-    put(KG, +1, t.KGE[n], t.KGO[n]);
     for (int q = 0; q < n; ++q) {
       t.l0[n][q] = (T)r.l0[q];
       t.l1[n][q] = (T)r.l1[q];
@@ -222,6 +277,19 @@ void build_tables(Tables<T> &t) {
     }
   }
 }
+template <typename T>
+void build_box_tables(BoxTables<T> &t) {
+  std::memset((void *)&t, 0, sizeof(t));
+  for (int n = 2; n <= kMaxN; ++n) {
+    const Rules1D &r = rules(n);
+    std::vector<double> M1, K1;
+    mass_stiffness(r, M1, K1);
+    box_tables(r, M1, K1, t);
+  }
+}
+template void build_box_tables<double>(BoxTables<double> &);
+template void build_box_tables<float>(BoxTables<float> &);
+
 template void build_tables<double>(Tables<double> &);
 template void build_tables<float>(Tables<float> &);
 

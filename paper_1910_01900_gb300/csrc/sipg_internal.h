@@ -30,6 +30,22 @@ void gauss_rule(int n, std::vector<double> &x, std::vector<double> &w);   // any
 std::vector<double> lagrange_values(const std::vector<double> &nodes, double x);
 std::vector<double> lagrange_derivs(const std::vector<double> &nodes, double x);
 
+// What one lane of the axis-aligned DG pass computes with: two FP32 values
+// (packed arithmetic on two cells) or one FP64 value.
+struct alignas(8) F2 {
+  float x, y;
+};
+template <typename T>
+struct BoxNum;
+template <>
+struct BoxNum<float> {
+  using type = F2;
+};
+template <>
+struct BoxNum<double> {
+  using type = double;
+};
+
 // Device-side 1D tables for all n in one block, uploaded to constant memory of
 // every translation unit that launches sum-factorisation kernels.
 template <typename T>
@@ -49,12 +65,29 @@ struct Tables {
   // (both M[i][j] = M[n-1-i][n-1-j]): the factors of the Cartesian FE cell matrix
   T M1[kMaxN + 1][16], K1[kMaxN + 1][16];
   T M1E[kMaxN + 1][25], M1O[kMaxN + 1][20], K1E[kMaxN + 1][25], K1O[kMaxN + 1][20];
-  // the collocation stiffness at the Gauss points, KG[i][j] = sum_q D[q][i] w_q D[q][j]
-  // (KG[i][j] = KG[n-1-i][n-1-j]): the cell term of an axis-aligned DG cell along one direction
-  T KG[kMaxN + 1][16], KGE[kMaxN + 1][25], KGO[kMaxN + 1][20];
 };
 template <typename T>
 void build_tables(Tables<T> &t);
+
+// The tables of axis-aligned DG cells (dg_box.cuh), n = 2..9 at index n - 2:
+// HE, HO even-odd blocks of M1^-1 [K1 - (e0 q0^T + q0 e0^T + e1 q1^T + q1 e1^T)/2,
+// e_s, q_s/2], rows of hc + 2 (stride 7) and h + 2 (stride 6): the matrix, then
+// the end columns; ME, MO even-odd blocks of M1 (strides 5, 4); qh = q1/2.
+// e_s: an end's unit vector, q_s: the outward end derivative of the GL basis.
+template <typename T>
+struct BoxTables {
+  using V = typename BoxNum<T>::type;
+  V HE[kMaxN - 1][35], HO[kMaxN - 1][24], ME[kMaxN - 1][25], MO[kMaxN - 1][20], qh[kMaxN - 1][kMaxN];
+};
+template <typename T>
+void build_box_tables(BoxTables<T> &t);
+
+// Cells of a thread block of the axis-aligned DG pass: bricks bricks side by
+// side in x, each of w[d] = 1 or 2 cells per direction.
+struct BoxShape {
+  int w[3] = {2, 1, 1};
+  int bricks = 1;
+};
 
 // Arguments of the DG evaluation / integration passes.
 template <typename T>
@@ -64,12 +97,15 @@ struct DGArgs {
   T *grad;             // scratch: reference gradient at Gauss points, [cell][3][n^3]
   T *trace;            // scratch: face traces, [cell][6 faces][2 (value, d_n)][n^2]
   const T *metric;     // curved: [cell][6][n^3] = w|detJ| J^-1 J^-T (xx,yy,zz,xy,xz,yz)
-  const T *wcart;      // Cartesian: [3][n^3] = w_q * prod(h)/h_d^2
+  const T *wcart;      // Cartesian (setup's diagonal): [3][n^3] = w_q * prod(h)/h_d^2
   const T *fdA[3];     // curved: [face][n^2] area element times weights
   const T *fc[3];      // curved: [face][2 roles][3][n^2] = J^-1 n_outward (own side)
-  const T *fwcart;     // Cartesian: [3][n^2] = w_q1 w_q2 h_t1 h_t2
+  const T *fwcart;     // Cartesian (setup's diagonal): [3][n^2] = w_q1 w_q2 h_t1 h_t2
   const T *tau;        // [cell] penalty tau_e
-  T ih[3];             // Cartesian 1/h_d
+  // Cartesian: 1/h_d, h_d, alpha_d / alpha_z of y and x, alpha_z (alpha_d =
+  // prod(h) / h_d^2), and the cells a thread block takes
+  T ih[3], hd[3], ralpha[2], alphaz;
+  BoxShape box;
   int m[3];
   int ncells;
   int bc[6];
@@ -92,6 +128,20 @@ struct DGArgs {
   // fc[0] [cell][6][3][n^2] (own side J^-1 n, n the outward unit normal)
   const int2 *ufn = nullptr;
 };
+
+// the Cartesian scale factors of a from the cell sizes
+template <typename T>
+void dg_box_scales(DGArgs<T> &a, const double h[3]) {
+  double al[3];
+  for (int d = 0; d < 3; ++d) al[d] = h[0] * h[1] * h[2] / (h[d] * h[d]);
+  for (int d = 0; d < 3; ++d) {
+    a.hd[d] = (T)h[d];
+    a.ih[d] = (T)(1.0 / h[d]);
+  }
+  a.ralpha[0] = (T)(al[1] / al[2]);
+  a.ralpha[1] = (T)(al[0] / al[2]);
+  a.alphaz = (T)al[2];
+}
 
 // Arguments of the FE cell pass and the node gather pass.
 template <typename T>
@@ -143,6 +193,7 @@ struct Level {
   // use (cb0, the autotuner's choice or a set value; 0 = compiled default)
   int cb[2][3] = {{0, 0, 0}, {0, 0, 0}};
   int cb0[2][3] = {{0, 0, 0}, {0, 0, 0}};
+  BoxShape box[2];   // axis-aligned DG level: block shape at cb[precision][1]
   // FE levels of low degree: assembled stencil [(2p+1)^3][nodes] in both
   // precisions (nullptr: matrix-free)
   void *stencil[2] = {nullptr, nullptr};
@@ -156,21 +207,29 @@ struct Level {
 
 // Launchers (one per precision; defined in the kernel translation units).
 template <typename T>
-void upload_tables_dg(const Tables<T> &t);
+void upload_tables_dg(const Tables<T> &t, const BoxTables<T> &bt);
 template <typename T>
 void upload_tables_fe(const Tables<T> &t);
 template <typename T>
-void upload_tables_batch(const Tables<T> &t);
+void upload_tables_batch(const Tables<T> &t, const BoxTables<T> &bt);
 
+// curved cells: the two passes at cb cells per block (0 = default)
 template <typename T>
-cudaError_t launch_dg_eval(int n, bool curved, const DGArgs<T> &a, cudaStream_t s, int cb = 0);
+cudaError_t launch_dg_eval(int n, const DGArgs<T> &a, cudaStream_t s, int cb = 0);
 template <typename T>
-cudaError_t launch_dg_integrate(int n, bool curved, const DGArgs<T> &a, cudaStream_t s, int cb = 0);
+cudaError_t launch_dg_integrate(int n, const DGArgs<T> &a, cudaStream_t s, int cb = 0);
+// axis-aligned cells: one pass, a.box cells per block
 template <typename T>
-int dg_cells_per_block(int n);
+cudaError_t launch_dg_box(int n, const DGArgs<T> &a, cudaStream_t s);
+// the block shape of at most cb cells (0 = default) for a mesh of m cells
+template <typename T>
+BoxShape dg_box_shape(int n, const int m[3], int cb);
+template <typename T>
+int dg_cells_per_block(int n, bool curved = true);   // curved: the cell passes' default (FE too)
 template <typename T>
 int dg_max_cells_per_block(int n);
-// resident blocks per SM of a DG pass (0 evaluation, 1 integration) at cb cells per block
+// resident blocks per SM of a DG pass (0 evaluation, 1 integration; on
+// axis-aligned cells 1 is the one pass) at cb cells per block
 template <typename T>
 cudaError_t dg_blocks_per_sm(int n, bool curved, int pass, int cb, int *blocks);
 
@@ -308,7 +367,7 @@ struct BatchProb {
 };
 
 struct WorkItem {
-  int p, cell0, ncta;
+  int p, cell0, ncta;   // axis-aligned DG cells: block number (x fastest); its shape is in the plan
 };
 
 // Per-problem segments for the batched vector kernels.
@@ -373,7 +432,8 @@ struct BatchPlan {
 };
 
 template <typename T>
-cudaError_t batch_plan_build(BatchPlan<T> &P, const std::vector<DGArgs<T>> &args, const std::vector<int> &ns);
+cudaError_t batch_plan_build(BatchPlan<T> &P, const std::vector<DGArgs<T>> &args, const std::vector<int> &ns,
+                             bool curved);
 template <typename T>
 void batch_plan_free(BatchPlan<T> &P);
 template <typename T>

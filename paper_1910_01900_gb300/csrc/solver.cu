@@ -13,6 +13,7 @@
 #include <stdexcept>
 #include <string>
 #include <tuple>
+#include <type_traits>
 
 #include "geometry.h"
 #include "sipg_internal.h"
@@ -217,9 +218,10 @@ DGArgs<T> dg_args(sipg_ctx *c, const Level &L) {
   for (int d = 0; d < 3; ++d) {
     a.fdA[d] = (const T *)L.fdA[pi][d];
     a.fc[d] = (const T *)L.fc[pi][d];
-    a.ih[d] = (T)(1.0 / L.h[d]);
     a.m[d] = L.m[d];
   }
+  a.box = L.box[pi];
+  dg_box_scales(a, L.h);
   a.fwcart = (const T *)L.fwcart[pi];
   a.tau = (const T *)L.tau[pi];
   a.ufn = L.ufn;
@@ -269,8 +271,12 @@ void apply_level(sipg_ctx *c, int l, const T *u, T *out, int mode, const T *x = 
     a.c1 = c1;
     a.c2 = c2;
     a.c3 = c3;
-    CK(launch_dg_eval<T>(L.n, L.curved, a, c->stream, L.cb[pidx<T>()][0]));
-    CK(launch_dg_integrate<T>(L.n, L.curved, a, c->stream, L.cb[pidx<T>()][1]));
+    if (!L.curved) {
+      CK(launch_dg_box<T>(L.n, a, c->stream));
+    } else {
+      CK(launch_dg_eval<T>(L.n, a, c->stream, L.cb[pidx<T>()][0]));
+      CK(launch_dg_integrate<T>(L.n, a, c->stream, L.cb[pidx<T>()][1]));
+    }
   } else {
     FEArgs<T> a = fe_args<T>(c, L);
     a.u = u;
@@ -845,7 +851,7 @@ std::vector<int> tile_candidates(const Level &L, int pass, int keep) {
     score.push_back({(double)L.ncells / ((double)waves * slots * cb) * lanes, cb});
   }
   std::stable_sort(score.begin(), score.end(), [](const auto &x, const auto &y) { return x.first > y.first; });
-  std::vector<int> out{dg_cells_per_block<T>(L.n)};
+  std::vector<int> out{dg_cells_per_block<T>(L.n, L.kind != 0 || L.curved)};
   for (const auto &sc : score) {
     if ((int)out.size() > keep) break;
     if (std::find(out.begin(), out.end(), sc.second) == out.end()) out.push_back(sc.second);
@@ -889,11 +895,14 @@ void autotune_level(sipg_ctx *c, int l, int pass) {
   int best_cb = cands[0];
   for (int cb : cands) {
     auto run = [&]() {
-      if (pass == 0) CK(launch_dg_eval<T>(L.n, L.curved, a, c->stream, cb));
-      else if (pass == 1) CK(launch_dg_integrate<T>(L.n, L.curved, a, c->stream, cb));
+      if (pass < 2 && !L.curved) {
+        a.box = dg_box_shape<T>(L.n, L.m, cb);
+        CK(launch_dg_box<T>(L.n, a, c->stream));
+      } else if (pass == 0) CK(launch_dg_eval<T>(L.n, a, c->stream, cb));
+      else if (pass == 1) CK(launch_dg_integrate<T>(L.n, a, c->stream, cb));
       else CK(launch_fe_cells<T>(L.n, L.curved, f, false, c->stream, cb));
     };
-    if (pass == 1) CK(launch_dg_eval<T>(L.n, L.curved, a, c->stream, 0));   // valid scratch for the integration
+    if (pass == 1 && L.curved) CK(launch_dg_eval<T>(L.n, a, c->stream, 0));   // valid scratch for the integration
     run();
     CK(cudaEventRecord(e0, c->stream));
     const int reps = 5;
@@ -919,21 +928,32 @@ void autotune_level(sipg_ctx *c, int l, int pass) {
 void init_device_tables() {
   static Tables<double> td;
   static Tables<float> tf;
+  static BoxTables<double> bd;
+  static BoxTables<float> bf;
   static std::once_flag built;
   std::call_once(built, [] {
     build_tables(td);
     build_tables(tf);
+    build_box_tables(bd);
+    build_box_tables(bf);
   });
-  upload_tables_dg<double>(td);
-  upload_tables_dg<float>(tf);
+  upload_tables_dg<double>(td, bd);
+  upload_tables_dg<float>(tf, bf);
   upload_tables_fe<double>(td);
   upload_tables_fe<float>(tf);
-  upload_tables_batch<double>(td);
-  upload_tables_batch<float>(tf);
+  upload_tables_batch<double>(td, bd);
+  upload_tables_batch<float>(tf, bf);
   CK(cudaGetLastError());
   CK(prepare_dg_kernels<double>());
   CK(prepare_dg_kernels<float>());
   CK(prepare_fe_kernels());
+}
+
+// the block shapes of an axis-aligned DG level for its widths
+void set_box(Level &L) {
+  if (L.kind != 0 || L.curved) return;
+  L.box[0] = dg_box_shape<double>(L.n, L.m, L.cb[0][1]);
+  L.box[1] = dg_box_shape<float>(L.n, L.m, L.cb[1][1]);
 }
 
 // Default tile widths of every level: the compiled default, lowered on
@@ -947,10 +967,12 @@ void default_tile_widths(sipg_ctx *c) {
   for (Level &L : c->lv)
     for (int pi = 0; pi < 2; ++pi)
       for (int pass = 0; pass < 3; ++pass) {
-        int cb = dg_cells_per_block<double>(L.n);
+        const bool box = L.kind == 0 && !L.curved;
+        int cb = pi ? dg_cells_per_block<float>(L.n, !box) : dg_cells_per_block<double>(L.n, !box);
         if (nsm > 0 && (L.ncells + cb - 1) / cb < nsm) cb = (int)std::max<int64_t>(1, (L.ncells + nsm - 1) / nsm);
         L.cb[pi][pass] = L.cb0[pi][pass] = cb;
       }
+  for (Level &L : c->lv) set_box(L);
 }
 
 void setup(sipg_ctx *c) {
@@ -1031,7 +1053,7 @@ void setup(sipg_ctx *c) {
     L.ndofs = s.kind == 0 ? L.ncells * n3 : (int64_t)L.grid[0] * L.grid[1] * L.grid[2];
     build_level_geometry(c, L, s.md, s.kind == 0);
     if (s.kind == 1) ebuf_len = std::max(ebuf_len, L.ncells * n3);
-    if (s.kind == 0) {
+    if (s.kind == 0 && L.curved) {   // axis-aligned cells need no scratch
       dg_grad_len = std::max(dg_grad_len, L.ncells * 3 * n3);
       dg_trace_len = std::max(dg_trace_len, L.ncells * 12 * (int64_t)L.n * L.n);
     }
@@ -1070,10 +1092,12 @@ void setup(sipg_ctx *c) {
     for (int l = c->solver ? 1 : c->L; l <= c->L; ++l) {
       const int k = c->lv[l].kind;
       if (k == 1 && c->lv[l].deg <= P.fe_assemble) continue;   // assembled stencil: no cell pass to tune
-      for (int pass = k == 0 ? 0 : 2; pass <= (k == 0 ? 1 : 2); ++pass) {
+      // axis-aligned DG levels have one pass (1)
+      for (int pass = k == 0 ? (c->lv[l].curved ? 0 : 1) : 2; pass <= (k == 0 ? 1 : 2); ++pass) {
         autotune_level<double>(c, l, pass);
         autotune_level<float>(c, l, pass);
       }
+      set_box(c->lv[l]);
     }
   }
   c->scal = dalloc<double>(c, 64);
@@ -2316,23 +2340,20 @@ sipg_status sipg_time_apply(sipg_ctx *c, int precision, const void *u, void *v, 
     cudaEvent_t ev[3];
     for (auto &e : ev) CK(cudaEventCreate(&e));
     float te = 0, ti = 0;
+    auto timed = [&](auto a) {
+      using T = std::remove_const_t<std::remove_pointer_t<decltype(a.u)>>;
+      constexpr int pi = pidx<T>();
+      a.u = (const T *)u;
+      a.out = (T *)v;
+      if (L.curved) CK(launch_dg_eval<T>(L.n, a, c->stream, L.cb[pi][0]));
+      CK(cudaEventRecord(ev[1], c->stream));
+      if (L.curved) CK(launch_dg_integrate<T>(L.n, a, c->stream, L.cb[pi][1]));
+      else CK(launch_dg_box<T>(L.n, a, c->stream));
+    };
     for (int r = 0; r < repeats; ++r) {
       CK(cudaEventRecord(ev[0], c->stream));
-      if (precision == 0) {
-        DGArgs<double> a = dg_args<double>(c, L);
-        a.u = (const double *)u;
-        a.out = (double *)v;
-        CK(launch_dg_eval<double>(L.n, L.curved, a, c->stream, L.cb[0][0]));
-        CK(cudaEventRecord(ev[1], c->stream));
-        CK(launch_dg_integrate<double>(L.n, L.curved, a, c->stream, L.cb[0][1]));
-      } else {
-        DGArgs<float> a = dg_args<float>(c, L);
-        a.u = (const float *)u;
-        a.out = (float *)v;
-        CK(launch_dg_eval<float>(L.n, L.curved, a, c->stream, L.cb[1][0]));
-        CK(cudaEventRecord(ev[1], c->stream));
-        CK(launch_dg_integrate<float>(L.n, L.curved, a, c->stream, L.cb[1][1]));
-      }
+      if (precision == 0) timed(dg_args<double>(c, L));
+      else timed(dg_args<float>(c, L));
       CK(cudaEventRecord(ev[2], c->stream));
       CK(cudaEventSynchronize(ev[2]));
       float a1, a2;
@@ -2353,8 +2374,10 @@ sipg_status sipg_tile_shape(const sipg_ctx *c, int level, int precision, int pas
       level > c->L || (c->lv[level].kind == 0) != (pass < 2))
     return SIPG_EINVAL;
   const int v = c->lv[level].cb[precision][pass];
-  const int n = c->lv[level].n;
-  *cells_per_block = v ? v : (precision == 0 ? dg_cells_per_block<double>(n) : dg_cells_per_block<float>(n));
+  const Level &L = c->lv[level];
+  const bool cells = L.kind != 0 || L.curved;
+  *cells_per_block =
+      v ? v : (precision == 0 ? dg_cells_per_block<double>(L.n, cells) : dg_cells_per_block<float>(L.n, cells));
   return SIPG_OK;
 }
 
@@ -2367,6 +2390,7 @@ sipg_status sipg_set_tile_shape(sipg_ctx *c, int level, int precision, int pass,
                           : (precision == 0 ? fe_max_cells_per_block<double>(n) : fe_max_cells_per_block<float>(n));
   if (cells_per_block < 0 || cells_per_block > mx) return SIPG_EINVAL;
   c->lv[level].cb[precision][pass] = cells_per_block ? cells_per_block : c->lv[level].cb0[precision][pass];
+  set_box(c->lv[level]);
   // captured V-cycles hold the old launch shapes
   for (int p = 0; p < 2; ++p) {
     if (c->vgraph[p]) cudaGraphExecDestroy(c->vgraph[p]);
@@ -2908,8 +2932,7 @@ std::unique_ptr<BatchCycle<T>> batch_cycle_build(sipg_batch *B) {
     for (int64_t q = 0; q * kBatchNodeThreads < D.ndofs; ++q) nd.push_back({p, (int)q});
     for (int64_t q = 0; q * kBatchNodeThreads < F.ndofs; ++q) ng.push_back({p, (int)q});
   }
-  CK(batch_plan_build<T>(C->dg, a0, nn));
-  C->dg.curved = C->curved;
+  CK(batch_plan_build<T>(C->dg, a0, nn, C->curved));
   CK(prep_fe_cells_batched<T>(C->fe_smem));
   C->n_fe_items = (int)fei.size();
   C->n_d = (int)nd.size();
@@ -2931,7 +2954,7 @@ std::unique_ptr<BatchCycle<T>> batch_cycle_build(sipg_batch *B) {
     for (int p = 0; p < np; ++p) hv.push_back(task(p));
   };
   auto dgapply = [&](auto args) {
-    C->prog.push_back({2, hd.size()});
+    if (C->curved) C->prog.push_back({2, hd.size()});   // axis-aligned cells: one pass
     C->prog.push_back({3, hd.size()});
     for (int p = 0; p < np; ++p) {
       BatchProb<T> q{};
@@ -3107,7 +3130,7 @@ void batch_build_fcg_chunk(sipg_batch *B) {
     }
     for (int i = 0; i < kFcgChunk; ++i) {
       body(add_if_node(s, hA[i]), &B->fcg_kA[i], [&]() {
-        CK(batch_dg_pass<double>(B->plan, B->d_app, false, B->d_segs, s2));
+        if (B->plan.curved) CK(batch_dg_pass<double>(B->plan, B->d_app, false, B->d_segs, s2));
         CK(batch_dg_pass<double>(B->plan, B->d_app, true, B->d_segs, s2));
         CK(seg_dot(B->d_segs, B->sg, 2, B->partials, B->counters, B->sc, st, 2, s2));
         CK(seg_update_xr(B->d_segs, B->sg, B->partials, B->counters, B->sc, st, s2));
@@ -3339,7 +3362,7 @@ void ensure_multi(sipg_ctx *c, int nv) {
     const Level &L = c->lv[l];
     for (int k = 0; k < 4; ++k) M.v[4 * l + k] = dalloc<char>(c, (int64_t)(L.ndofs * nv * es));
     const int64_t n3 = (int64_t)L.n * L.n * L.n;
-    if (L.kind == 0) {
+    if (L.kind == 0 && L.curved) {
       grad = std::max(grad, L.ncells * 3 * n3);
       trace = std::max(trace, L.ncells * 12 * (int64_t)L.n * L.n);
     }
@@ -3493,8 +3516,7 @@ sipg_status sipg_batch_create(int nprob, const sipg_mesh *meshes, const sipg_par
         args.push_back(dg_args<double>(c, c->lv[c->L]));
         ns.push_back(c->lv[c->L].n);
       }
-      CK(batch_plan_build(B->plan, args, ns));
-      B->plan.curved = curved;
+      CK(batch_plan_build(B->plan, args, ns, curved));
       B->segs.assign(nprob, Seg{});
       CK(cudaMalloc(&B->d_segs, nprob * sizeof(Seg)));
       CK(cudaMalloc(&B->sc, (size_t)nprob * kSegSlots * sizeof(double)));
