@@ -315,8 +315,9 @@ sipg_status sipg_time_apply(sipg_ctx *ctx, int precision, const void *u_dev, voi
  * for many right-hand sides.  meshes[i], params[i] describe problem i (all
  * affine or all curved; one precision for all; each needs a Dirichlet side);
  * params[0].stream is the stream of the batched work.  The finest-level
- * operators of all problems run as one persistent launch per pass (a fixed
- * grid walking a work list of (problem, cell block) items, longest first);
+ * operators of all problems run as one launch per degree (affine meshes; a
+ * block per (problem, cell block) item) or one persistent launch per pass
+ * (curved ones; a fixed grid walking a work list, longest first);
  * the flexible-CG iterations run in lockstep with batched inner products and
  * updates (blocks per problem in proportion to its size).  On a non-default
  * stream, when every problem's hierarchy starts with a DG level above a
@@ -335,7 +336,7 @@ sipg_status sipg_batch_destroy(sipg_batch *batch);
 const char *sipg_batch_last_error(const sipg_batch *batch);
 /* The context of problem i (owned by the batch; do not destroy it). */
 sipg_status sipg_batch_context(sipg_batch *batch, int i, sipg_ctx **ctx);
-/* v[i] = A_i u[i] (FP64, finest level) for every problem: two launches total. */
+/* v[i] = A_i u[i] (FP64, finest level) for every problem in shared launches. */
 sipg_status sipg_batch_apply(sipg_batch *batch, const double *const *u_dev, double *const *v_dev);
 /* z[i] = M_i^-1 r[i] (FP64 in and out): one V-cycle (Algorithm 2) of every
  * problem, through the batched cycle where it applies (above).  Each z[i]

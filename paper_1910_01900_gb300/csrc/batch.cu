@@ -1,11 +1,13 @@
 // Many independent SIPG problems (uneven mesh size and degree) or many
 // right-hand sides of one problem, solved together.
 //
-// * The finest-level DG operator of all problems runs as ONE persistent
-//   launch per pass: a fixed grid (SMs x resident blocks) walks a static list
-//   of work items (problem, first cell, cell count), longest first, and
-//   dispatches each item to the sum-factorisation body of that problem's
-//   degree.  The same bodies as the per-problem kernels (dg_kernels.cuh).
+// * The finest-level DG operator of all problems runs as one launch per degree
+//   (axis-aligned cells: a block per item of a static list of problems' blocks,
+//   dg_box.cuh) or, on curved cells, as one persistent launch per pass: a fixed
+//   grid (SMs x resident blocks) walks a static list of work items (problem,
+//   first cell, cell count), longest first, and dispatches each item to the
+//   sum-factorisation body of that problem's degree.  The same bodies as the
+//   per-problem kernels (dg_kernels.cuh).
 // * The flexible-CG iterations of all problems run in lockstep: batched
 //   operator applications, batched inner products and updates (one launch for
 //   all problems, deterministic per-problem reductions), and each problem's
@@ -37,25 +39,11 @@ void upload_tables_batch<float>(const Tables<float> &t, const BoxTables<float> &
   upload_box_tu(bt);
 }
 
-// an item of an axis-aligned problem: block w.cell0 of its mesh, the block's
-// shape packed in w.ncta (the plan's, whatever the problem's own launches use)
-static int pack_shape(const BoxShape &b) { return (b.w[0] - 1) | (b.w[1] - 1) << 1 | (b.w[2] - 1) << 2 | b.bricks << 3; }
-template <typename T, int N>
-__device__ __forceinline__ void dg_box_item(const DGArgs<T> &a, const WorkItem &w, unsigned char *sm) {
-  BoxShape b;
-  b.w[0] = (w.ncta & 1) + 1;
-  b.w[1] = ((w.ncta >> 1) & 1) + 1;
-  b.w[2] = ((w.ncta >> 2) & 1) + 1;
-  b.bricks = w.ncta >> 3;
-  const int wx = b.w[0] * b.bricks, nx = (a.m[0] + wx - 1) / wx, ny = (a.m[1] + b.w[1] - 1) / b.w[1], r = w.cell0 / nx;
-  dg_box_body<T, N>(a, vec_ptrs(a, 0), b, w.cell0 - r * nx, r % ny, r / ny, sm);
-}
-
 // segs (optional): the flexible-CG systems; a problem whose system has left
 // the iteration (segs[p].active == 0, set on the device) is skipped too
 // (register budget as the single-problem passes: FP32, bound by shared
 // memory traffic and latency, keeps 6 blocks of 256 threads resident)
-template <typename T, bool CURVED, bool INTEGRATE>
+template <typename T, bool INTEGRATE>
 __global__ void __launch_bounds__(kBatchThreads, sizeof(T) == 4 ? 6 : 3)
     dg_batched_kernel(const BatchProb<T> *__restrict__ probs, const WorkItem *__restrict__ items, int nitems,
                       const Seg *__restrict__ segs) {
@@ -65,14 +53,12 @@ __global__ void __launch_bounds__(kBatchThreads, sizeof(T) == 4 ? 6 : 3)
     const WorkItem w = items[it];
     const BatchProb<T> &P = probs[w.p];
     if (P.active && (!segs || segs[w.p].active)) {
-#define SIPG_BATCH_CASE(NN)                                                          \
-  case NN:                                                                           \
-    if constexpr (!CURVED)                                                           \
-      dg_box_item<T, NN>(P.a, w, smem_raw);                                          \
-    else if constexpr (INTEGRATE)                                                    \
-      dg_integrate_body<T, NN>(P.a, vec_ptrs(P.a, 0), w.cell0, w.ncta, sm);          \
-    else                                                                             \
-      dg_eval_body<T, NN>(P.a, vec_ptrs(P.a, 0), w.cell0, w.ncta, sm);               \
+#define SIPG_BATCH_CASE(NN)                                                 \
+  case NN:                                                                  \
+    if (INTEGRATE)                                                          \
+      dg_integrate_body<T, NN>(P.a, vec_ptrs(P.a, 0), w.cell0, w.ncta, sm); \
+    else                                                                    \
+      dg_eval_body<T, NN>(P.a, vec_ptrs(P.a, 0), w.cell0, w.ncta, sm);      \
     break;
       switch (P.n) {
         SIPG_BATCH_CASE(2)
@@ -90,6 +76,49 @@ __global__ void __launch_bounds__(kBatchThreads, sizeof(T) == 4 ? 6 : 3)
     }
     __syncthreads();
   }
+}
+
+// Axis-aligned problems: the one pass of all problems of one degree, a block
+// per item (block w.cell0 of problem w.p's mesh, cut by shape, which is the
+// plan's whatever the problem's own launches use).  One kernel per degree: with
+// every degree's body in one kernel the FP32 pass needed 80 registers and 900
+// bytes of stack.
+template <typename T, int N>
+__global__ void __launch_bounds__(kBatchThreads) dg_box_batched_kernel(const BatchProb<T> *__restrict__ probs,
+                                                                       const WorkItem *__restrict__ items,
+                                                                       const Seg *__restrict__ segs) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const WorkItem w = items[blockIdx.x];
+  const BatchProb<T> &P = probs[w.p];
+  if (!P.active || (segs && !segs[w.p].active)) return;
+  BoxShape b;
+  b.w[0] = (w.ncta & 1) + 1;
+  b.w[1] = ((w.ncta >> 1) & 1) + 1;
+  b.w[2] = ((w.ncta >> 2) & 1) + 1;
+  b.bricks = w.ncta >> 3;
+  const int wx = b.w[0] * b.bricks, nx = (P.a.m[0] + wx - 1) / wx, ny = (P.a.m[1] + b.w[1] - 1) / b.w[1],
+            r = w.cell0 / nx;
+  dg_box_body<T, N>(P.a, vec_ptrs(P.a, 0), b, w.cell0 - r * nx, r % ny, r / ny, smem_raw);
+}
+static int pack_shape(const BoxShape &b) { return (b.w[0] - 1) | (b.w[1] - 1) << 1 | (b.w[2] - 1) << 2 | b.bricks << 3; }
+
+template <typename T>
+static cudaError_t prep_box_batched() {
+  cudaError_t e = cudaSuccess;
+#define SIPG_BATCH_PREP(NN)                                                                                     \
+  if (e == cudaSuccess)                                                                                         \
+    e = cudaFuncSetAttribute(dg_box_batched_kernel<T, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize,         \
+                             kBatchThreads / (NN * NN) * box_group_values(NN) * 8);
+  SIPG_BATCH_PREP(2)
+  SIPG_BATCH_PREP(3)
+  SIPG_BATCH_PREP(4)
+  SIPG_BATCH_PREP(5)
+  SIPG_BATCH_PREP(6)
+  SIPG_BATCH_PREP(7)
+  SIPG_BATCH_PREP(8)
+  SIPG_BATCH_PREP(9)
+#undef SIPG_BATCH_PREP
+  return e;
 }
 
 // Blocks of the batched vector kernels: system p gets g.nb[p] blocks (one
@@ -261,35 +290,45 @@ cudaError_t batch_plan_build(BatchPlan<T> &P, const std::vector<DGArgs<T>> &args
   P.curved = curved;
   P.probs.resize(np);
   P.items.clear();
-  size_t smem = 0;
+  P.degrees.clear();
   for (int p = 0; p < np; ++p) {
     P.probs[p].a = args[p];
     P.probs[p].n = ns[p];
     P.probs[p].active = 1;
-    const int n = ns[p], cb = kBatchThreads / (n * n);
-    if (!curved) {   // the block shape of kBatchThreads threads
-      const BoxShape w = dg_box_shape<T>(n, args[p].m, cb * kBoxLanes<T>);
-      int nb = args[p].ncells > 0;
-      for (int d = 0; d < 3; ++d) {
-        const int wd = w.w[d] * (d == 0 ? w.bricks : 1);
-        nb *= (args[p].m[d] + wd - 1) / wd;
-      }
-      smem = std::max(smem, (size_t)box_groups<T>(w) * box_group_values(n) * 8);
-      for (int b = 0; b < nb; ++b) P.items.push_back({p, b, pack_shape(w)});
-      continue;
-    }
-    smem = std::max(smem, (size_t)cb * cell_values(n) * sizeof(T));
-    for (int c = 0; c < args[p].ncells; c += cb) P.items.push_back({p, c, std::min(cb, args[p].ncells - c)});
   }
-  // longest items first (cost ~ cells x n^4), then static striding over the grid
-  std::stable_sort(P.items.begin(), P.items.end(), [&](const WorkItem &x, const WorkItem &y) {
-    auto cost = [&](const WorkItem &w) {
-      const int n = ns[w.p];
-      const double cells = curved ? w.ncta : kBatchThreads / (n * n);
-      return cells * std::pow((double)n, 4);
-    };
-    return cost(x) > cost(y);
-  });
+  size_t smem = 0;
+  if (curved) {
+    for (int p = 0; p < np; ++p) {
+      const int n = ns[p], cb = kBatchThreads / (n * n);
+      smem = std::max(smem, (size_t)cb * cell_values(n) * sizeof(T));
+      for (int c = 0; c < args[p].ncells; c += cb) P.items.push_back({p, c, std::min(cb, args[p].ncells - c)});
+    }
+    // longest items first (cost ~ cells x n^4), then static striding over the grid
+    std::stable_sort(P.items.begin(), P.items.end(), [&](const WorkItem &x, const WorkItem &y) {
+      const double cx = (double)x.ncta * std::pow((double)ns[x.p], 4), cy = (double)y.ncta * std::pow((double)ns[y.p], 4);
+      return cx > cy;
+    });
+  } else {
+    for (int n = kMaxN; n >= 2; --n) {   // the degrees' items one after another
+      typename BatchPlan<T>::Degree d{n, (int)P.items.size(), 0, 0, 0};
+      for (int p = 0; p < np; ++p) {
+        if (ns[p] != n || args[p].ncells == 0) continue;
+        // a default block, as far as kBatchThreads allow
+        const int cb = std::min(dg_cells_per_block<T>(n, false), kBatchThreads / (n * n) * kBoxLanes<T>);
+        const BoxShape w = dg_box_shape<T>(n, args[p].m, cb);
+        int nb = 1;
+        for (int e = 0; e < 3; ++e) {
+          const int we = w.w[e] * (e == 0 ? w.bricks : 1);
+          nb *= (args[p].m[e] + we - 1) / we;
+        }
+        d.groups = std::max(d.groups, box_groups<T>(w));
+        for (int b = 0; b < nb; ++b) P.items.push_back({p, b, pack_shape(w)});
+      }
+      d.count = (int)P.items.size() - d.first;
+      d.smem = (size_t)d.groups * box_group_values(n) * 8;
+      if (d.count) P.degrees.push_back(d);
+    }
+  }
   P.smem = smem;
   cudaError_t e;
   if ((e = cudaMalloc(&P.d_probs, np * sizeof(BatchProb<T>))) != cudaSuccess) return e;
@@ -297,15 +336,15 @@ cudaError_t batch_plan_build(BatchPlan<T> &P, const std::vector<DGArgs<T>> &args
   if ((e = cudaMemcpy(P.d_items, P.items.data(), P.items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice)) !=
       cudaSuccess)
     return e;
-  auto k1 = dg_batched_kernel<T, false, true>;
-  auto k2 = dg_batched_kernel<T, true, false>, k3 = dg_batched_kernel<T, true, true>;
-  for (auto k : {k1, k2, k3})
+  if (!curved) return prep_box_batched<T>();
+  auto k2 = dg_batched_kernel<T, false>, k3 = dg_batched_kernel<T, true>;
+  for (auto k : {k2, k3})
     if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
       return e;
   int dev, nsm, occ = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k1, kBatchThreads, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k3, kBatchThreads, smem);
   P.grid = std::max(1, std::min<int>((int)P.items.size(), nsm * std::max(1, occ)));
   return cudaSuccess;
 }
@@ -318,8 +357,8 @@ void batch_plan_free(BatchPlan<T> &P) {
   P.d_items = nullptr;
 }
 
-// Upload the current descriptors (pointers, modes, active flags) and run both
-// passes as two persistent launches.
+// Upload the current descriptors (pointers, modes, active flags) and run the
+// pass or passes.
 template <typename T>
 cudaError_t batch_dg_pass(const BatchPlan<T> &P, const BatchProb<T> *probs, bool integrate, const Seg *segs,
                           cudaStream_t s);
@@ -341,12 +380,30 @@ cudaError_t batch_dg_pass(const BatchPlan<T> &P, const BatchProb<T> *probs, bool
   const int ni = (int)P.items.size();
   if (ni == 0) return cudaSuccess;
   if (P.curved) {
-    if (integrate) dg_batched_kernel<T, true, true><<<P.grid, kBatchThreads, P.smem, s>>>(probs, P.d_items, ni, segs);
-    else dg_batched_kernel<T, true, false><<<P.grid, kBatchThreads, P.smem, s>>>(probs, P.d_items, ni, segs);
-  } else {
-    dg_batched_kernel<T, false, true><<<P.grid, kBatchThreads, P.smem, s>>>(probs, P.d_items, ni, segs);
+    if (integrate) dg_batched_kernel<T, true><<<P.grid, kBatchThreads, P.smem, s>>>(probs, P.d_items, ni, segs);
+    else dg_batched_kernel<T, false><<<P.grid, kBatchThreads, P.smem, s>>>(probs, P.d_items, ni, segs);
+    note_launch();
+    return cudaGetLastError();
   }
-  note_launch();
+  for (const auto &d : P.degrees) {
+    const WorkItem *it = P.d_items + d.first;
+    switch (d.n) {
+#define SIPG_BATCH_CASE(NN)                                                                             \
+  case NN:                                                                                              \
+    dg_box_batched_kernel<T, NN><<<d.count, d.groups * NN * NN, d.smem, s>>>(probs, it, segs);          \
+    break;
+      SIPG_BATCH_CASE(2)
+      SIPG_BATCH_CASE(3)
+      SIPG_BATCH_CASE(4)
+      SIPG_BATCH_CASE(5)
+      SIPG_BATCH_CASE(6)
+      SIPG_BATCH_CASE(7)
+      SIPG_BATCH_CASE(8)
+      SIPG_BATCH_CASE(9)
+#undef SIPG_BATCH_CASE
+    }
+    note_launch();
+  }
   return cudaGetLastError();
 }
 

@@ -347,23 +347,7 @@ __device__ __forceinline__ void dg_integrate_body(const DGArgs<T> &a, const VecP
     load_line<T, N>(st, base, stride, x);
   }
   apply_mat<T, N, MSt>(x, y);
-  const size_t g0 = (size_t)cell * N3 + l;
-  if (a.mode == 0) {
-#pragma unroll
-    for (int q = 0; q < N; ++q) v.out[g0 + q * N2] = y[q];
-  } else if (a.mode == 2) {
-#pragma unroll
-    for (int q = 0; q < N; ++q) v.out[g0 + q * N2] = v.b[g0 + q * N2] - y[q];
-  } else {
-#pragma unroll
-    for (int q = 0; q < N; ++q) {
-      const size_t i = g0 + q * N2;
-      T z = a.c3 * a.dinv[i] * (v.b[i] - y[q]);
-      if (v.x) z = fma(a.c1, v.x[i], z);
-      if (v.xp) z = fma(a.c2, v.xp[i], z);
-      v.out[i] = z;
-    }
-  }
+  dg_epilogue<T, N>(a, v, (size_t)cell * N3 + l, N2, T(1), y);
 }
 
 // Per-vector pointers of a multi-vector launch: vector r of u, out, x, xp, b

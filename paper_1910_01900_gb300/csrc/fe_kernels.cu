@@ -1,7 +1,8 @@
 // Continuous FE levels of the cph hierarchy (Section 2, Eq. WeakFormFE;
 // Section 3.2 transfers), both precisions.
 //
-// FE operator: a cell pass evaluates (grad v, grad u) on every cell by sum
+// FE operator on axis-aligned cells: one pass (fe_box.cuh).  On curved cells a
+// cell pass evaluates (grad v, grad u) on every cell by sum
 // factorisation (same interpolation/derivative sweeps as the DG cell term)
 // after gathering the cell's nodes from the global grid (constrained
 // Dirichlet nodes read as zero), and writes the cell-local result into an
@@ -14,7 +15,7 @@
 // c-restriction (sum of the duplicated DG nodes, Section 3.2 c-coarsening).
 #include <algorithm>
 
-#include "sumfac.cuh"
+#include "fe_box.cuh"
 
 namespace sipg {
 
@@ -42,7 +43,7 @@ __device__ __forceinline__ bool node_constrained(const int g[3], const int grid[
 // The cell pass on cells cell0 .. cell0 + ncta - 1 of one vector (input ug,
 // element buffer ebv), one line of N points per thread, N^2 threads per cell
 // (threads beyond ncta N^2 only join the barriers).
-template <typename T, int N, bool CURVED>
+template <typename T, int N>
 __device__ __forceinline__ void fe_cell_body(const FEArgs<T> &a, const T *__restrict__ ug, T *__restrict__ ebv,
                                              const int cell0, const int ncta, T *sm) {
   constexpr int N2 = N * N, N3 = N2 * N, TT = Tile<N>::T3;
@@ -65,51 +66,6 @@ __device__ __forceinline__ void fe_cell_body(const FEArgs<T> &a, const T *__rest
       g[2] = cz * P + q;
       xl[q] = node_constrained(g, a.grid, a.bc) ? T(0) : ug[b0 + sz * g[2]];
     }
-  }
-  if constexpr (!CURVED) {
-    // An axis-aligned box cell: its matrix is the sum over d of alpha_d times
-    // the tensor product of the 1D stiffness matrix K1 in direction d and the
-    // 1D mass matrix M1 in the other two (both under the Gauss rule, as the
-    // interpolate / differentiate / weight / transpose sweeps of the general
-    // path compute it), so y = ax K1 M1 M1 u + ay M1 K1 M1 u + az M1 M1 K1 u
-    // takes 7 1D products instead of 12: along z a = M1 u, b = K1 u; along y
-    // c = M1 a, f = ay K1 a + az M1 b; along x y = ax K1 c + M1 f.
-    T *t0 = su, *t1 = su + TT;
-    int base, stride;
-    if (act) {
-      line_of<N>(2, l, base, stride);
-      T y[N];
-      apply_mat<T, N, MK1>(xl, y);
-      store_line<T, N>(t1, base, stride, y);
-      apply_mat<T, N, MM1>(xl, y);
-      store_line<T, N>(t0, base, stride, y);
-    }
-    __syncthreads();
-    if (act) {
-      line_of<N>(1, l, base, stride);
-      T x[N], y[N], k[N];
-      load_line<T, N>(t0, base, stride, x);
-      apply_mat<T, N, MM1>(x, y);
-      store_line<T, N>(t0, base, stride, y);
-      apply_mat<T, N, MK1>(x, k);
-      load_line<T, N>(t1, base, stride, x);
-      apply_mat<T, N, MM1>(x, y);
-#pragma unroll
-      for (int q = 0; q < N; ++q) y[q] = fma(a.alpha[1], k[q], a.alpha[2] * y[q]);
-      store_line<T, N>(t1, base, stride, y);
-    }
-    __syncthreads();
-    if (!act) return;
-    line_of<N>(0, l, base, stride);
-    T x[N], y[N], k[N];
-    load_line<T, N>(t0, base, stride, x);
-    apply_mat<T, N, MK1>(x, k);
-    load_line<T, N>(t1, base, stride, x);
-    apply_mat<T, N, MM1>(x, y);
-    T *eb = ebv + (size_t)(cell0 + cl) * N3 + N * l;   // the x-line of points (q, l % N, l / N)
-#pragma unroll
-    for (int q = 0; q < N; ++q) eb[q] = fma(a.alpha[0], k[q], y[q]);
-    return;
   }
   if (act) {   // interpolation along z from the registers, then x and y in place
     int base, stride;
@@ -140,17 +96,11 @@ __device__ __forceinline__ void fe_cell_body(const FEArgs<T> &a, const T *__rest
     const int c = i / N3, p = i - c * N3;
     T *s = sm + c * Tile<N>::CS + TT + Tile<N>::idx(p);
     const T g0 = s[0], g1 = s[TT], g2 = s[2 * TT];
-    if constexpr (!CURVED) {
-      s[0] = g0 * a.wcart[p];
-      s[TT] = g1 * a.wcart[N3 + p];
-      s[2 * TT] = g2 * a.wcart[2 * N3 + p];
-    } else {
-      const T *M = a.metric + (size_t)(cell0 + c) * 6 * N3 + p;
-      const T xx = M[0], yy = M[N3], zz = M[2 * N3], xy = M[3 * N3], xz = M[4 * N3], yz = M[5 * N3];
-      s[0] = xx * g0 + xy * g1 + xz * g2;
-      s[TT] = xy * g0 + yy * g1 + yz * g2;
-      s[2 * TT] = xz * g0 + yz * g1 + zz * g2;
-    }
+    const T *M = a.metric + (size_t)(cell0 + c) * 6 * N3 + p;
+    const T xx = M[0], yy = M[N3], zz = M[2 * N3], xy = M[3 * N3], xz = M[4 * N3], yz = M[5 * N3];
+    s[0] = xx * g0 + xy * g1 + xz * g2;
+    s[TT] = xy * g0 + yy * g1 + yz * g2;
+    s[2 * TT] = xz * g0 + yz * g1 + zz * g2;
   }
   __syncthreads();
 #pragma unroll 1
@@ -191,14 +141,14 @@ __device__ __forceinline__ void fe_cell_body(const FEArgs<T> &a, const T *__rest
 // cb cells per thread block (a launch parameter, cb N^2 threads); MULTI:
 // several vectors, block b = cell group b / nv of vector b % nv (compiled
 // apart from the single-vector kernel, whose offsets would cost registers)
-template <typename T, int N, bool CURVED, bool MULTI>
+template <typename T, int N, bool MULTI>
 __global__ void __launch_bounds__(kCellThreads) fe_cell_kernel(const FEArgs<T> a, const int cb) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *sm = reinterpret_cast<T *>(smem_raw);
   // block -> (cell group, vector); the vectors of one group are neighbours
   const int grp = MULTI ? blockIdx.x / a.nv : blockIdx.x, vec = MULTI ? blockIdx.x - grp * a.nv : 0;
   const int cell0 = grp * cb;
-  fe_cell_body<T, N, CURVED>(a, MULTI ? a.u + vec * a.vs : a.u, MULTI ? a.ebuf + vec * a.es : a.ebuf, cell0,
+  fe_cell_body<T, N>(a, MULTI ? a.u + vec * a.vs : a.u, MULTI ? a.ebuf + vec * a.es : a.ebuf, cell0,
                              min(cb, a.ncells - cell0), sm);
 }
 
@@ -372,17 +322,7 @@ __global__ void __launch_bounds__(256) fe_stencil_apply_kernel(const FEArgs<T> a
   for (int w = SL / 2; w > 0; w >>= 1) y += __shfl_xor_sync(0xffffffffu, y, w, SL);
   if (gid >= ng || z != 0) return;
   if (node_constrained(g, a.grid, a.bc)) y = u[gid];   // identity row
-  const long gv = vo + gid;
-  if (a.mode == 0) {
-    a.out[gv] = y;
-  } else if (a.mode == 2) {
-    a.out[gv] = a.b[gv] - y;
-  } else {
-    T v = a.c3 * a.dinv[gid] * (a.b[gv] - y);
-    if (a.x) v = fma(a.c1, a.x[gv], v);
-    if (a.xp) v = fma(a.c2, a.xp[gv], v);
-    a.out[gv] = v;
-  }
+  fe_row(a, vo, gid, y);
 }
 
 // Node pass: out[g] = sum over the cells sharing node g of ebuf, then the epilogue.
@@ -435,17 +375,12 @@ __device__ __forceinline__ void fe_gather_node(const FEArgs<T> &a, const long gi
       if ((x || lo[0]) && (yy || lo[1]) && (z || lo[2])) y += e[q];
     }
   }
-  const long gv = vo + gid;
-  if (a.mode == 0 || a.mode >= 3) {
+  if (a.mode >= 3) {
+    const long gv = vo + gid;
     a.out[gv] = y;
     if (a.mode == 5) a.out2[gv] = a.c3 * a.dinv[gid] * y;   // launch_xdb's x = c D^-1 b
-  } else if (a.mode == 2) {
-    a.out[gv] = a.b[gv] - y;
   } else {
-    T v = a.c3 * a.dinv[gid] * (a.b[gv] - y);
-    if (a.x) v = fma(a.c1, a.x[gv], v);
-    if (a.xp) v = fma(a.c2, a.xp[gv], v);
-    a.out[gv] = v;
+    fe_row(a, vo, gid, y);
   }
 }
 
@@ -501,7 +436,7 @@ __global__ void c_prolongate_add_kernel(const FEArgs<T> a, const T *xc, T *xdg, 
 // one its own launch gives.  A problem whose flexible-CG system has left the
 // iteration (segs[p].active == 0) is skipped.
 
-template <typename T, bool CURVED>
+template <typename T>
 __global__ void __launch_bounds__(kBatchCellThreads) fe_cell_batched_kernel(const FETask<T> *__restrict__ tasks,
                                                                           const WorkItem *__restrict__ items,
                                                                           const Seg *__restrict__ segs) {
@@ -513,7 +448,7 @@ __global__ void __launch_bounds__(kBatchCellThreads) fe_cell_batched_kernel(cons
   switch (P.a.deg + 1) {
 #define SIPG_FEB_CASE(NN) \
   case NN:                \
-    fe_cell_body<T, NN, CURVED>(P.a, P.a.u, P.a.ebuf, w.cell0, w.ncta, sm); \
+    fe_cell_body<T, NN>(P.a, P.a.u, P.a.ebuf, w.cell0, w.ncta, sm); \
     break;
     SIPG_FEB_CASE(2)
     SIPG_FEB_CASE(3)
@@ -527,6 +462,19 @@ __global__ void __launch_bounds__(kBatchCellThreads) fe_cell_batched_kernel(cons
     default:
       break;
   }
+}
+
+// Axis-aligned cells: item = brick w.cell0 of problem w.p, the whole operator;
+// one kernel per degree (see dg_box_batched_kernel).
+template <typename T, int N>
+__global__ void __launch_bounds__(fe_box_threads<T>(N), fe_box_blocks<T>(N))
+    fe_box_batched_kernel(const FETask<T> *__restrict__ tasks, const WorkItem *__restrict__ items,
+                          const Seg *__restrict__ segs) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const WorkItem w = items[blockIdx.x];
+  if (segs && !segs[w.p].active) return;
+  const FEArgs<T> &a = tasks[w.p].a;
+  fe_box_body<T, N>(a, 0, a.brick[0], a.brick[1], a.brick[2], w.cell0, reinterpret_cast<T *>(smem_raw));
 }
 
 // node passes (kind 0: gather with the task's mode and epilogue) and the
@@ -833,7 +781,7 @@ __global__ void dg_transfer_kernel(const XferGeom G, const T *__restrict__ P1, c
 }
 
 // ---------------------------------------------------------------- launchers
-template <typename T, int N, bool CURVED>
+template <typename T, int N>
 static cudaError_t run_fe_cells(const FEArgs<T> &a, cudaStream_t s, int cb) {
   if (cb <= 0) cb = default_cb(N);
   if (cb > max_cb(N, sizeof(T))) return cudaErrorInvalidValue;
@@ -842,28 +790,101 @@ static cudaError_t run_fe_cells(const FEArgs<T> &a, cudaStream_t s, int cb) {
   if (grid == 0) return cudaSuccess;
   if (grid > 0x7fffffff) return cudaErrorInvalidValue;
   if (a.nv > 1)
-    fe_cell_kernel<T, N, CURVED, true><<<(unsigned)grid, cb * N * N, smem, s>>>(a, cb);
+    fe_cell_kernel<T, N, true><<<(unsigned)grid, cb * N * N, smem, s>>>(a, cb);
   else
-    fe_cell_kernel<T, N, CURVED, false><<<(unsigned)grid, cb * N * N, smem, s>>>(a, cb);
+    fe_cell_kernel<T, N, false><<<(unsigned)grid, cb * N * N, smem, s>>>(a, cb);
   note_launch();
   return cudaGetLastError();
 }
 
-template <typename T, int N, bool CURVED>
+template <typename T, int N>
 static cudaError_t occ_fe_cells(int cb, int *blocks) {
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fe_cell_kernel<T, N, CURVED, false>, cb * N * N,
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fe_cell_kernel<T, N, false>, cb * N * N,
                                                        (size_t)cb * Tile<N>::CS * sizeof(T));
+}
+
+// Cells per direction of a brick.  kFEBoxBrick[p]: about 16 own nodes along x
+// and y and 8 along z, where a thin brick's tiles leave room for more blocks
+// per SM (FP32 smoothing step on 32^3 cells of degree 4: 27.2 us for 4 x 4 x 2
+// against 36.7 us for 4 x 4 x 4 and 35.3 us for 2 x 2 x 2).  Where that gives
+// fewer bricks than the GPU can use, the side of most cells is halved until it
+// does: FP32 below 140 bricks (16^3 of degree 4: 128 bricks 14.4 us, 256 12.9
+// us), FP64, where the halo's arithmetic costs more, below 100 (50 us against
+// 61 us).  cb > 0: at most cb cells in all.  Sides are evened out over the
+// bricks of a direction.
+constexpr int kFEBoxBrick[kMaxN][3] = {{1, 1, 1}, {16, 8, 4}, {8, 4, 4}, {5, 4, 2}, {4, 4, 2},
+                                       {4, 2, 2}, {3, 2, 2},  {2, 2, 2}, {2, 2, 2}};
+constexpr int kFEBoxSmem = 176 * 1024;   // degree 8 in FP64: 170 KB
+template <typename T>
+void fe_box_brick(int n, const int m[3], int cb, int brick[3]) {
+  const int p = n - 1, least = sizeof(T) == 4 ? 140 : 100;
+  int b[3] = {kFEBoxBrick[p][0], kFEBoxBrick[p][1], kFEBoxBrick[p][2]};
+  for (;;) {
+    int64_t bricks = 1;
+    for (int d = 0; d < 3; ++d) bricks *= (m[d] + b[d] - 1) / b[d];
+    int d = 2;
+    for (int e : {1, 0})
+      if (b[e] > b[d]) d = e;
+    if (b[d] == 1 || (cb > 0 ? b[0] * b[1] * b[2] <= cb : bricks >= least)) break;
+    b[d] = (b[d] + 1) / 2;
+  }
+  for (int d = 0; d < 3; ++d) {
+    const int k = (m[d] + b[d] - 1) / b[d];
+    brick[d] = (m[d] + k - 1) / k;
+  }
+}
+
+template <typename T, int N>
+static cudaError_t run_fe_box(const FEArgs<T> &a, cudaStream_t s) {
+  int64_t blocks = 1;
+  int w[3];
+  for (int d = 0; d < 3; ++d) {
+    blocks *= (a.m[d] + a.brick[d] - 1) / a.brick[d];
+    w[d] = std::min(a.brick[d] + 1, a.m[d]) * (N - 1) + 1;
+  }
+  const int lines = std::max(w[0] * w[1], w[1] * (a.brick[2] * (N - 1) + 1));
+  if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
+  const size_t smem = fe_box_values(N - 1, a.brick) * sizeof(T);
+  if (smem > (size_t)kFEBoxSmem) return cudaErrorInvalidValue;
+  // one round of the widest stage's lines, or two of half its width
+  const int rounds = lines > 256 ? 2 : 1;
+  const int threads = std::min(fe_box_threads<T>(N), ((lines + rounds - 1) / rounds + 31) / 32 * 32);
+  fe_box_kernel<T, N><<<dim3((unsigned)blocks, a.nv), threads, smem, s>>>(a);
+  note_launch();
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_fe_box(const FEArgs<T> &a, cudaStream_t s) {
+  if (a.ncells == 0) return cudaSuccess;
+  if ((int64_t)a.grid[0] * a.grid[1] * a.grid[2] >= (1LL << 32)) return cudaErrorInvalidValue;
+  switch (a.deg) {
+#define SIPG_FEBOX_CASE(NN) \
+  case NN - 1:              \
+    return run_fe_box<T, NN>(a, s);
+    SIPG_FEBOX_CASE(2)
+    SIPG_FEBOX_CASE(3)
+    SIPG_FEBOX_CASE(4)
+    SIPG_FEBOX_CASE(5)
+    SIPG_FEBOX_CASE(6)
+    SIPG_FEBOX_CASE(7)
+    SIPG_FEBOX_CASE(8)
+    SIPG_FEBOX_CASE(9)
+#undef SIPG_FEBOX_CASE
+    default:
+      return cudaErrorInvalidValue;
+  }
 }
 
 template <typename T, int N>
 static cudaError_t prep_fe_n() {
+  constexpr cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
   const int smem = max_cb(N, sizeof(T)) * Tile<N>::CS * (int)sizeof(T);
   cudaError_t e = cudaSuccess;
-  for (cudaError_t r :
-       {cudaFuncSetAttribute(fe_cell_kernel<T, N, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
-        cudaFuncSetAttribute(fe_cell_kernel<T, N, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
-        cudaFuncSetAttribute(fe_cell_kernel<T, N, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
-        cudaFuncSetAttribute(fe_cell_kernel<T, N, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)})
+  for (cudaError_t r : {cudaFuncSetAttribute(fe_cell_kernel<T, N, false>, at, smem),
+                        cudaFuncSetAttribute(fe_cell_kernel<T, N, true>, at, smem),
+                        cudaFuncSetAttribute(fe_box_kernel<T, N>, at, kFEBoxSmem),
+                        cudaFuncSetAttribute(fe_box_batched_kernel<T, N>, at, kFEBoxSmem)})
     if (r != cudaSuccess) e = r;
   return e;
 }
@@ -906,7 +927,7 @@ cudaError_t launch_fe_cells(int n, bool curved, const FEArgs<T> &a, bool diag_on
         return curved ? run_fe_diag<NN, true>(a, s) : run_fe_diag<NN, false>(a, s);          \
       return cudaErrorInvalidValue;                                                          \
     }                                                                                        \
-    return curved ? run_fe_cells<T, NN, true>(a, s, cb) : run_fe_cells<T, NN, false>(a, s, cb);
+    return run_fe_cells<T, NN>(a, s, cb);
   switch (n) {
     SIPG_FE_CASE(2)
     SIPG_FE_CASE(3)
@@ -987,10 +1008,10 @@ int fe_max_cells_per_block(int n) {
 }
 
 template <typename T>
-cudaError_t fe_blocks_per_sm(int n, bool curved, int cb, int *blocks) {
+cudaError_t fe_blocks_per_sm(int n, int cb, int *blocks) {
 #define SIPG_FE_OCC(NN) \
   case NN:              \
-    return curved ? occ_fe_cells<T, NN, true>(cb, blocks) : occ_fe_cells<T, NN, false>(cb, blocks);
+    return occ_fe_cells<T, NN>(cb, blocks);
   switch (n) {
     SIPG_FE_OCC(2)
     SIPG_FE_OCC(3)
@@ -1028,13 +1049,35 @@ cudaError_t launch_fe_gather(const FEArgs<T> &a, cudaStream_t s) {
 }
 
 template <typename T>
-cudaError_t launch_fe_cells_batched(bool curved, const FETask<T> *tasks, const WorkItem *items, int nitems,
-                                    size_t smem, const Seg *segs, cudaStream_t s) {
+cudaError_t launch_fe_cells_batched(const FETask<T> *tasks, const WorkItem *items, int nitems, size_t smem,
+                                    const Seg *segs, cudaStream_t s) {
   if (nitems <= 0) return cudaSuccess;
-  if (curved)
-    fe_cell_batched_kernel<T, true><<<nitems, kBatchCellThreads, smem, s>>>(tasks, items, segs);
-  else
-    fe_cell_batched_kernel<T, false><<<nitems, kBatchCellThreads, smem, s>>>(tasks, items, segs);
+  fe_cell_batched_kernel<T><<<nitems, kBatchCellThreads, smem, s>>>(tasks, items, segs);
+  note_launch();
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_fe_box_batched(int n, const FETask<T> *tasks, const WorkItem *items, int nitems, size_t smem,
+                                  const Seg *segs, cudaStream_t s) {
+  if (nitems <= 0) return cudaSuccess;
+  switch (n) {
+#define SIPG_FEB_CASE(NN)                                                                                   \
+  case NN:                                                                                                  \
+    fe_box_batched_kernel<T, NN><<<nitems, kBatchCellThreads, smem, s>>>(tasks, items, segs);               \
+    break;
+    SIPG_FEB_CASE(2)
+    SIPG_FEB_CASE(3)
+    SIPG_FEB_CASE(4)
+    SIPG_FEB_CASE(5)
+    SIPG_FEB_CASE(6)
+    SIPG_FEB_CASE(7)
+    SIPG_FEB_CASE(8)
+    SIPG_FEB_CASE(9)
+#undef SIPG_FEB_CASE
+    default:
+      return cudaErrorInvalidValue;
+  }
   note_launch();
   return cudaGetLastError();
 }
@@ -1052,11 +1095,7 @@ int tile_values(int n) { return cell_values(n); }
 
 template <typename T>
 cudaError_t prep_fe_cells_batched(size_t smem) {
-  cudaError_t e = cudaFuncSetAttribute(fe_cell_batched_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(fe_cell_batched_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  return e;
+  return cudaFuncSetAttribute(fe_cell_batched_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
 template <typename T>
@@ -1318,12 +1357,16 @@ cudaError_t launch_dg_transfer(const XferGeom &g, const T *P1, const T *in, T *o
 #define SIPG_FE_INST(T)                                                                                   \
   template cudaError_t launch_fe_cells<T>(int, bool, const FEArgs<T> &, bool, cudaStream_t, int);       \
   template int fe_max_cells_per_block<T>(int);                                                          \
-  template cudaError_t fe_blocks_per_sm<T>(int, bool, int, int *);                                      \
+  template cudaError_t fe_blocks_per_sm<T>(int, int, int *);                                            \
+  template void fe_box_brick<T>(int, const int *, int, int *);                                          \
+  template cudaError_t launch_fe_box<T>(const FEArgs<T> &, cudaStream_t);                               \
   template cudaError_t launch_fe_gather<T>(const FEArgs<T> &, cudaStream_t);                            \
   template cudaError_t launch_fe_stencil_apply<T>(const FEArgs<T> &, const T *, cudaStream_t);          \
   template cudaError_t launch_c_prolongate_add<T>(const FEArgs<T> &, const T *, T *, cudaStream_t, int64_t); \
-  template cudaError_t launch_fe_cells_batched<T>(bool, const FETask<T> *, const WorkItem *, int, size_t,      \
+  template cudaError_t launch_fe_cells_batched<T>(const FETask<T> *, const WorkItem *, int, size_t,            \
                                                   const Seg *, cudaStream_t);                                  \
+  template cudaError_t launch_fe_box_batched<T>(int, const FETask<T> *, const WorkItem *, int, size_t,         \
+                                                const Seg *, cudaStream_t);                                    \
   template cudaError_t launch_fe_nodes_batched<T>(const FETask<T> *, const NodeItem *, int, const Seg *, int, \
                                                   cudaStream_t);                                               \
   template cudaError_t prep_fe_cells_batched<T>(size_t);                                                       \

@@ -162,6 +162,7 @@ struct FEArgs {
   const T *x, *xp, *b, *dinv;
   T c1, c2, c3;
   T alpha[3];          // Cartesian: prod(h) / h_d^2, the scale of direction d's term
+  int brick[3] = {1, 1, 1};   // Cartesian: cells of a thread block per direction
   T *out2 = nullptr;   // mode 5
   // nv vectors at once: vector r of u, out, x, xp, b starts at r * vs, its
   // element buffer at r * es
@@ -194,6 +195,7 @@ struct Level {
   int cb[2][3] = {{0, 0, 0}, {0, 0, 0}};
   int cb0[2][3] = {{0, 0, 0}, {0, 0, 0}};
   BoxShape box[2];   // axis-aligned DG level: block shape at cb[precision][1]
+  int brick[2][3] = {{1, 1, 1}, {1, 1, 1}};   // axis-aligned FE level: its brick at cb[precision][2]
   // FE levels of low degree: assembled stencil [(2p+1)^3][nodes] in both
   // precisions (nullptr: matrix-free)
   void *stencil[2] = {nullptr, nullptr};
@@ -235,14 +237,24 @@ cudaError_t dg_blocks_per_sm(int n, bool curved, int pass, int cb, int *blocks);
 
 cudaError_t launch_dg_diag(int n, bool curved, const DGArgs<double> &a, double *diag, cudaStream_t s);
 
-// FE cell pass at cb cells per block (0 = default); diag_only: the cell-local
-// diagonal (setup, FP64)
+// FE cell pass of curved cells at cb cells per block (0 = default); diag_only:
+// the cell-local diagonal (setup, FP64)
 template <typename T>
 cudaError_t launch_fe_cells(int n, bool curved, const FEArgs<T> &a, bool diag_only, cudaStream_t s, int cb = 0);
 template <typename T>
 int fe_max_cells_per_block(int n);
 template <typename T>
-cudaError_t fe_blocks_per_sm(int n, bool curved, int cb, int *blocks);
+cudaError_t fe_blocks_per_sm(int n, int cb, int *blocks);
+// axis-aligned cells: the operator with the epilogue (modes 0-2) in one pass
+template <typename T>
+cudaError_t launch_fe_box(const FEArgs<T> &a, cudaStream_t s);
+// its brick of at most cb cells (0: the default) for a mesh of m cells
+template <typename T>
+void fe_box_brick(int n, const int m[3], int cb, int brick[3]);
+// values of shared memory of a brick of b cells of degree p (two tiles)
+__host__ __device__ inline int64_t fe_box_values(const int p, const int b[3]) {
+  return 2 * (int64_t)(((b[0] + 1) * p + 1) | 1) * ((b[1] + 1) * p + 1) * (b[2] * p + 1);
+}
 template <typename T>
 cudaError_t launch_fe_gather(const FEArgs<T> &a, cudaStream_t s);
 // Assembled stencil of an FE level of degree 1 or 2 (setup, FP64):
@@ -367,7 +379,7 @@ struct BatchProb {
 };
 
 struct WorkItem {
-  int p, cell0, ncta;   // axis-aligned DG cells: block number (x fastest); its shape is in the plan
+  int p, cell0, ncta;   // axis-aligned DG cells: block number (x fastest) and its packed shape
 };
 
 // Per-problem segments for the batched vector kernels.
@@ -379,7 +391,8 @@ struct Seg {
 };
 
 // Batched FE passes (fe_kernels.cu): one task per problem, one thread block
-// per item.  Cell items cover kBatchCellThreads / n^2 cells, node items
+// per item.  Cell items cover kBatchCellThreads / n^2 cells (axis-aligned
+// cells: a brick, the whole operator with its epilogue), node items
 // kBatchNodeThreads nodes (or DG points for the c-prolongation).
 constexpr int kBatchCellThreads = 256;
 constexpr int kBatchNodeThreads = 256;
@@ -393,8 +406,12 @@ struct NodeItem {
   int p, blk;
 };
 template <typename T>
-cudaError_t launch_fe_cells_batched(bool curved, const FETask<T> *tasks, const WorkItem *items, int nitems,
-                                    size_t smem, const Seg *segs, cudaStream_t s);
+cudaError_t launch_fe_cells_batched(const FETask<T> *tasks, const WorkItem *items, int nitems, size_t smem,
+                                    const Seg *segs, cudaStream_t s);
+// axis-aligned cells: the bricks of all problems of one degree
+template <typename T>
+cudaError_t launch_fe_box_batched(int n, const FETask<T> *tasks, const WorkItem *items, int nitems, size_t smem,
+                                  const Seg *segs, cudaStream_t s);
 // kind 0: gather with each task's mode and epilogue; 1: c-prolongation
 template <typename T>
 cudaError_t launch_fe_nodes_batched(const FETask<T> *tasks, const NodeItem *items, int nitems, const Seg *segs,
@@ -422,6 +439,12 @@ cudaError_t launch_batch_fcg_cond(const int *any, cudaGraphConditionalHandle h, 
 
 template <typename T>
 struct BatchPlan {
+  // axis-aligned problems: the items of one degree and their launch
+  struct Degree {
+    int n, first, count, groups;
+    size_t smem;
+  };
+  std::vector<Degree> degrees;
   std::vector<BatchProb<T>> probs;
   std::vector<WorkItem> items;
   BatchProb<T> *d_probs = nullptr;

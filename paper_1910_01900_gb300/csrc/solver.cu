@@ -1,8 +1,10 @@
 // Context, setup, V-cycle, Chebyshev smoother, flexible CG and the C ABI
 // (Section 3 of the paper: Algorithms 1-3, the cph level hierarchy, the
 // coarse solve; Section 4: mixed precision).
+#include <array>
 #include <atomic>
 #include <chrono>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -248,6 +250,7 @@ FEArgs<T> fe_args(sipg_ctx *c, const Level &L) {
   for (int d = 0; d < 3; ++d) {
     a.m[d] = L.m[d];
     a.grid[d] = L.grid[d];
+    a.brick[d] = L.brick[pi][d];
     a.alpha[d] = (T)(L.h[0] * L.h[1] * L.h[2] / (L.h[d] * L.h[d]));
   }
   for (int s = 0; s < 6; ++s) a.bc[s] = c->mesh.bc[s];
@@ -291,8 +294,10 @@ void apply_level(sipg_ctx *c, int l, const T *u, T *out, int mode, const T *x = 
     a.c3 = c3;
     if (L.stencil[pidx<T>()]) {
       CK(launch_fe_stencil_apply<T>(a, (const T *)L.stencil[pidx<T>()], c->stream));
+    } else if (!L.curved) {
+      CK(launch_fe_box<T>(a, c->stream));
     } else {
-      CK(launch_fe_cells<T>(L.n, L.curved, a, false, c->stream, L.cb[pidx<T>()][2]));
+      CK(launch_fe_cells<T>(L.n, true, a, false, c->stream, L.cb[pidx<T>()][2]));
       CK(launch_fe_gather<T>(a, c->stream));
     }
   }
@@ -842,7 +847,7 @@ std::vector<int> tile_candidates(const Level &L, int pass, int keep) {
   std::vector<std::pair<double, int>> score;
   for (int cb = 1; cb <= maxcb; ++cb) {
     int occ = 0;
-    CK(pass < 2 ? dg_blocks_per_sm<T>(L.n, L.curved, pass, cb, &occ) : fe_blocks_per_sm<T>(L.n, L.curved, cb, &occ));
+    CK(pass < 2 ? dg_blocks_per_sm<T>(L.n, L.curved, pass, cb, &occ) : fe_blocks_per_sm<T>(L.n, cb, &occ));
     if (occ <= 0) continue;
     const int threads = cb * L.n * L.n;
     const double lanes = threads / (32.0 * ((threads + 31) / 32));
@@ -900,7 +905,7 @@ void autotune_level(sipg_ctx *c, int l, int pass) {
         CK(launch_dg_box<T>(L.n, a, c->stream));
       } else if (pass == 0) CK(launch_dg_eval<T>(L.n, a, c->stream, cb));
       else if (pass == 1) CK(launch_dg_integrate<T>(L.n, a, c->stream, cb));
-      else CK(launch_fe_cells<T>(L.n, L.curved, f, false, c->stream, cb));
+      else CK(launch_fe_cells<T>(L.n, true, f, false, c->stream, cb));
     };
     if (pass == 1 && L.curved) CK(launch_dg_eval<T>(L.n, a, c->stream, 0));   // valid scratch for the integration
     run();
@@ -949,9 +954,14 @@ void init_device_tables() {
   CK(prepare_fe_kernels());
 }
 
-// the block shapes of an axis-aligned DG level for its widths
+// the block shapes of an axis-aligned level for its widths
 void set_box(Level &L) {
-  if (L.kind != 0 || L.curved) return;
+  if (L.curved) return;
+  if (L.kind == 1) {   // cb0 stands for the rule that fits the mesh
+    fe_box_brick<double>(L.n, L.m, L.cb[0][2] == L.cb0[0][2] ? 0 : L.cb[0][2], L.brick[0]);
+    fe_box_brick<float>(L.n, L.m, L.cb[1][2] == L.cb0[1][2] ? 0 : L.cb[1][2], L.brick[1]);
+    return;
+  }
   L.box[0] = dg_box_shape<double>(L.n, L.m, L.cb[0][1]);
   L.box[1] = dg_box_shape<float>(L.n, L.m, L.cb[1][1]);
 }
@@ -1092,6 +1102,7 @@ void setup(sipg_ctx *c) {
     for (int l = c->solver ? 1 : c->L; l <= c->L; ++l) {
       const int k = c->lv[l].kind;
       if (k == 1 && c->lv[l].deg <= P.fe_assemble) continue;   // assembled stencil: no cell pass to tune
+      if (k == 1 && !c->lv[l].curved) continue;   // its brick follows from the mesh
       // axis-aligned DG levels have one pass (1)
       for (int pass = k == 0 ? (c->lv[l].curved ? 0 : 1) : 2; pass <= (k == 0 ? 1 : 2); ++pass) {
         autotune_level<double>(c, l, pass);
@@ -2578,6 +2589,13 @@ struct BatchCycle {
   WorkItem *fe_items = nullptr;           // FE cell items
   int n_fe_items = 0;
   size_t fe_smem = 0;
+  // axis-aligned cells: each problem's FE brick, and the items of each degree
+  struct FEDegree {
+    int n, first, count;
+    size_t smem;
+  };
+  std::vector<std::array<int, 3>> brick;
+  std::vector<FEDegree> fe_degrees;
   NodeItem *items_d = nullptr, *items_g = nullptr;   // DG points, FE nodes
   int n_d = 0, n_g = 0;
   VecTask *vec = nullptr;
@@ -2853,7 +2871,10 @@ void batch_cycle_emit(sipg_batch *B, BatchCycle<T> &C, cudaStream_t s) {
         CK(batch_dg_pass<T>(C.dg, C.dgt + r.off, r.kind == 3, segs, s));
         break;
       case 4:
-        CK(launch_fe_cells_batched<T>(C.curved, C.fet + r.off, C.fe_items, C.n_fe_items, C.fe_smem, segs, s));
+        if (C.curved)
+          CK(launch_fe_cells_batched<T>(C.fet + r.off, C.fe_items, C.n_fe_items, C.fe_smem, segs, s));
+        for (const auto &d : C.fe_degrees)
+          CK(launch_fe_box_batched<T>(d.n, C.fet + r.off, C.fe_items + d.first, d.count, d.smem, segs, s));
         break;
       case 5:
         CK(launch_fe_nodes_batched<T>(C.fet + r.off, C.items_g, C.n_g, segs, 0, s));
@@ -2926,14 +2947,33 @@ std::unique_ptr<BatchCycle<T>> batch_cycle_build(sipg_batch *B) {
       a0.back().ncells = 0;   // no DG items
       continue;
     }
-    const int cb = kBatchCellThreads / (F.n * F.n);
-    C->fe_smem = std::max(C->fe_smem, (size_t)cb * tile_values(F.n) * sizeof(T));
-    for (int q = 0; q < F.ncells; q += cb) fei.push_back({p, q, (int)std::min<int64_t>(cb, F.ncells - q)});
+    if (C->curved) {
+      const int cb = kBatchCellThreads / (F.n * F.n);
+      C->fe_smem = std::max(C->fe_smem, (size_t)cb * tile_values(F.n) * sizeof(T));
+      for (int q = 0; q < F.ncells; q += cb) fei.push_back({p, q, (int)std::min<int64_t>(cb, F.ncells - q)});
+    }
     for (int64_t q = 0; q * kBatchNodeThreads < D.ndofs; ++q) nd.push_back({p, (int)q});
     for (int64_t q = 0; q * kBatchNodeThreads < F.ndofs; ++q) ng.push_back({p, (int)q});
   }
   CK(batch_plan_build<T>(C->dg, a0, nn, C->curved));
-  CK(prep_fe_cells_batched<T>(C->fe_smem));
+  C->brick.assign(np, {1, 1, 1});
+  if (!C->curved) {   // FE bricks, degree by degree: full ones (the problems together fill the GPU)
+    for (int n = kMaxN; n >= 2; --n) {
+      typename BatchCycle<T>::FEDegree d{n, (int)fei.size(), 0, 0};
+      for (int p = 0; p < np; ++p) {
+        const Level &F = B->ctx[p]->lv[B->ctx[p]->L - 1];
+        if (C->solo[p] || F.n != n) continue;
+        fe_box_brick<T>(n, F.m, INT_MAX, C->brick[p].data());
+        int nb = 1;
+        for (int e = 0; e < 3; ++e) nb *= (F.m[e] + C->brick[p][e] - 1) / C->brick[p][e];
+        for (int q = 0; q < nb; ++q) fei.push_back({p, q, 0});
+        d.smem = std::max(d.smem, (size_t)fe_box_values(F.deg, C->brick[p].data()) * sizeof(T));
+      }
+      d.count = (int)fei.size() - d.first;
+      if (d.count) C->fe_degrees.push_back(d);
+    }
+  }
+  if (C->curved) CK(prep_fe_cells_batched<T>(C->fe_smem));
   C->n_fe_items = (int)fei.size();
   C->n_d = (int)nd.size();
   C->n_g = (int)ng.size();
@@ -2966,7 +3006,8 @@ std::unique_ptr<BatchCycle<T>> batch_cycle_build(sipg_batch *B) {
   };
   auto fetask = [&](int kind, auto args) {   // kind 4: cell and node pass; 5: node pass; 6: c-prolongation
     if (kind == 4) C->prog.push_back({4, hf.size()});
-    C->prog.push_back({kind == 4 ? 5 : kind, hf.size()});
+    // axis-aligned cells: 4 is the whole operator
+    if (kind != 4 || C->curved) C->prog.push_back({kind == 4 ? 5 : kind, hf.size()});
     for (int p = 0; p < np; ++p) hf.push_back(args(p));
   };
   auto dga = [&](int p, const T *u, T *out, int mode, const T *x, const T *xp, const T *b, const ChebStep *q) {
@@ -2982,6 +3023,7 @@ std::unique_ptr<BatchCycle<T>> batch_cycle_build(sipg_batch *B) {
     const Level &F = c->lv[c->L - 1];
     FETask<T> t{};
     t.a = fe_args<T>(c, F);
+    for (int d = 0; d < 3; ++d) t.a.brick[d] = C->brick[p][d];
     t.a.u = u, t.a.out = out, t.a.mode = mode, t.a.x = x, t.a.xp = xp, t.a.b = b;
     if (q) t.a.dinv = (const T *)F.dinv[pi], t.a.c1 = (T)q->c1, t.a.c2 = (T)q->c2, t.a.c3 = (T)q->c3;
     return t;
@@ -3450,10 +3492,10 @@ sipg_status sipg_operator_apply_multi(sipg_ctx *c, int precision, int nv, const 
   if (!c->solver) return SIPG_EINVAL;
   return guarded(c, [&]() -> sipg_status {
     ensure_multi(c, nv);
-    if (precision == 1 && !c->mv.grad[1]) {   // FP32 scratch of a context whose cycle runs in FP64
+    if (precision == 1 && !c->mv.grad[1]) {   // curved cells' FP32 scratch of a context whose cycle runs in FP64
       int64_t grad = 0, trace = 0;
       for (const Level &L : c->lv)
-        if (L.kind == 0) {
+        if (L.kind == 0 && L.curved) {
           grad = std::max(grad, L.ncells * 3 * (int64_t)L.n * L.n * L.n);
           trace = std::max(trace, L.ncells * 12 * (int64_t)L.n * L.n);
         }
