@@ -22,6 +22,7 @@
 #include <vector>
 
 #include "dg_kernels.cuh"
+#include "stride_loop.cuh"
 
 namespace sipg {
 
@@ -41,10 +42,9 @@ void upload_tables_batch<float>(const Tables<float> &t, const BoxTables<float> &
 
 // segs (optional): the flexible-CG systems; a problem whose system has left
 // the iteration (segs[p].active == 0, set on the device) is skipped too
-// (register budget as the single-problem passes: FP32, bound by shared
-// memory traffic and latency, keeps 6 blocks of 256 threads resident)
+// (register budget as the single-problem passes: 64 and 128)
 template <typename T, bool INTEGRATE>
-__global__ void __launch_bounds__(kBatchThreads, sizeof(T) == 4 ? 6 : 3)
+__global__ void __launch_bounds__(kBatchThreads, sizeof(T) == 4 ? 4 : 2)
     dg_batched_kernel(const BatchProb<T> *__restrict__ probs, const WorkItem *__restrict__ items, int nitems,
                       const Seg *__restrict__ segs) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -128,21 +128,25 @@ static cudaError_t prep_box_batched() {
 
 __device__ void seg_reduce2(const SegGrid &g, int p, int j, double a, double b, double *partials, unsigned *counter,
                             double *out) {
-  // per block partial sums; the last block of the system sums them in block
-  // order (deterministic) and resets the system's counter
+  // per block partial sums; the last block of the system sums them (each
+  // thread a strided part in order, then the same tree: deterministic) and
+  // resets the system's counter
   __shared__ double sa[256], sb[256];
   __shared__ bool last;
   const int nb = g.nb[p], off = g.off[p];
+  auto tree = [&] {
+    __syncthreads();
+    for (int w = 128; w > 0; w >>= 1) {
+      if (threadIdx.x < w) {
+        sa[threadIdx.x] += sa[threadIdx.x + w];
+        sb[threadIdx.x] += sb[threadIdx.x + w];
+      }
+      __syncthreads();
+    }
+  };
   sa[threadIdx.x] = a;
   sb[threadIdx.x] = b;
-  __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if (threadIdx.x < w) {
-      sa[threadIdx.x] += sa[threadIdx.x + w];
-      sb[threadIdx.x] += sb[threadIdx.x + w];
-    }
-    __syncthreads();
-  }
+  tree();
   if (threadIdx.x == 0) {
     partials[(off + j) * 2] = sa[0];
     partials[(off + j) * 2 + 1] = sb[0];
@@ -152,14 +156,17 @@ __device__ void seg_reduce2(const SegGrid &g, int p, int j, double a, double b, 
   __syncthreads();
   if (!last) return;
   __threadfence();
+  double ta = 0, tb = 0;
+  for (int q = threadIdx.x; q < nb; q += 256) {
+    ta += ((volatile double *)partials)[(off + q) * 2];
+    tb += ((volatile double *)partials)[(off + q) * 2 + 1];
+  }
+  sa[threadIdx.x] = ta;
+  sb[threadIdx.x] = tb;
+  tree();
   if (threadIdx.x == 0) {
-    double ta = 0, tb = 0;
-    for (int q = 0; q < nb; ++q) {
-      ta += ((volatile double *)partials)[(off + q) * 2];
-      tb += ((volatile double *)partials)[(off + q) * 2 + 1];
-    }
-    out[0] = ta;
-    out[1] = tb;
+    out[0] = sa[0];
+    out[1] = sb[0];
     counter[p] = 0;
   }
 }
@@ -171,19 +178,23 @@ __global__ void seg_dot_kernel(const Seg *segs, const SegGrid g, int which, doub
   const Seg S = segs[p];
   if (!S.active) return;   // whole system inactive: every block of it returns
   double a = 0, b = 0;
-  for (long i = (long)j * blockDim.x + threadIdx.x; i < S.n; i += (long)nb * blockDim.x) {
-    if (which == 0) {
-      a = fma(S.b[i], S.b[i], a);
-      b = fma(S.r[i], S.r[i], b);
-    } else if (which == 1) {
-      a = fma(S.r[i], S.z[i], a);
-    } else if (which == 2) {
-      a = fma(S.p[i], S.v[i], a);
-    } else {
-      a = fma(S.r[i], S.z[i], a);
-      b = fma(S.z[i], S.v[i], b);
-    }
-  }
+  // a = sum u v, b = sum w w' (which 1 and 2: a alone)
+  const double *u = which == 0 ? S.b : (which == 2 ? S.p : S.r), *v = which == 0 ? S.b : (which == 2 ? S.v : S.z);
+  const double *w = which == 0 ? S.r : S.z, *w2 = which == 0 ? S.r : S.v;
+  const bool two = which == 0 || which == 3;
+  double ui[kAhead], vi[kAhead], wi[kAhead], xi[kAhead];
+  stride_loop(
+      (long)j * blockDim.x + threadIdx.x, (long)nb * blockDim.x, S.n,
+      [&](int k, long i) {
+        ui[k] = u[i];
+        vi[k] = v[i];
+        wi[k] = two ? w[i] : 0.0;
+        xi[k] = two ? w2[i] : 0.0;
+      },
+      [&](int k, long) {
+        a = fma(ui[k], vi[k], a);
+        if (two) b = fma(wi[k], xi[k], b);
+      });
   seg_reduce2(g, p, j, a, b, partials, counter, sc + (size_t)p * sc_stride + slot);
 }
 
@@ -196,12 +207,21 @@ __global__ void seg_update_xr_kernel(const Seg *segs, const SegGrid g, double *p
   const double *s = sc + (size_t)p * sc_stride;
   const double alpha = s[0] / s[2];
   double a = 0;
-  for (long i = (long)j * blockDim.x + threadIdx.x; i < S.n; i += (long)nb * blockDim.x) {
-    S.x[i] = fma(alpha, S.p[i], S.x[i]);
-    const double ri = fma(-alpha, S.v[i], S.r[i]);
-    S.r[i] = ri;
-    a = fma(ri, ri, a);
-  }
+  double xi[kAhead], pi[kAhead], vi[kAhead], ri[kAhead];
+  stride_loop(
+      (long)j * blockDim.x + threadIdx.x, (long)nb * blockDim.x, S.n,
+      [&](int k, long i) {
+        xi[k] = S.x[i];
+        pi[k] = S.p[i];
+        vi[k] = S.v[i];
+        ri[k] = S.r[i];
+      },
+      [&](int k, long i) {
+        S.x[i] = fma(alpha, pi[k], xi[k]);
+        const double r = fma(-alpha, vi[k], ri[k]);
+        S.r[i] = r;
+        a = fma(r, r, a);
+      });
   seg_reduce2(g, p, j, a, 0.0, partials, counter, sc + (size_t)p * sc_stride + 3);
 }
 
@@ -212,8 +232,14 @@ __global__ void seg_update_p_kernel(const Seg *segs, const SegGrid g, const doub
   if (!S.active) return;
   const double *s = sc + (size_t)p * sc_stride;
   const double beta = init ? 0.0 : -s[1] / s[2];
-  for (long i = (long)j * blockDim.x + threadIdx.x; i < S.n; i += (long)nb * blockDim.x)
-    S.p[i] = init ? S.z[i] : fma(beta, S.p[i], S.z[i]);
+  double pi[kAhead], zi[kAhead];
+  stride_loop(
+      (long)j * blockDim.x + threadIdx.x, (long)nb * blockDim.x, S.n,
+      [&](int k, long i) {
+        pi[k] = init ? 0.0 : S.p[i];
+        zi[k] = S.z[i];
+      },
+      [&](int k, long i) { S.p[i] = init ? zi[k] : fma(beta, pi[k], zi[k]); });
 }
 
 // ------------------------------------------ lockstep flexible CG gated on the device
@@ -300,7 +326,7 @@ cudaError_t batch_plan_build(BatchPlan<T> &P, const std::vector<DGArgs<T>> &args
   if (curved) {
     for (int p = 0; p < np; ++p) {
       const int n = ns[p], cb = kBatchThreads / (n * n);
-      smem = std::max(smem, (size_t)cb * cell_values(n) * sizeof(T));
+      smem = std::max(smem, (size_t)cb * curved_cell_values(n, true) * sizeof(T));
       for (int c = 0; c < args[p].ncells; c += cb) P.items.push_back({p, c, std::min(cb, args[p].ncells - c)});
     }
     // longest items first (cost ~ cells x n^4), then static striding over the grid

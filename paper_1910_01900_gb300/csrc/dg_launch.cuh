@@ -7,11 +7,19 @@
 
 namespace sipg {
 
+// the width that a setting of cb cells runs at: kCurvedThreads threads and the
+// shared memory at most
+template <typename T, int N>
+static int curved_cb(int cb) {
+  return std::min({cb, kCurvedThreads / (N * N), 232448 / (curved_cell_values(N, true) * (int)sizeof(T))});
+}
+
 template <typename T, int N>
 static cudaError_t run_dg(bool integrate, const DGArgs<T> &a, cudaStream_t s, int cb) {
   if (cb <= 0) cb = default_cb(N);
   if (cb > max_cb(N, sizeof(T))) return cudaErrorInvalidValue;
-  const size_t smem = (size_t)cb * Tile<N>::CS * sizeof(T);
+  cb = curved_cb<T, N>(cb);
+  const size_t smem = (size_t)cb * curved_cell_values(N, integrate) * sizeof(T);
   const int64_t grid = (int64_t)((a.ncells + cb - 1) / cb) * a.nv;
   if (grid == 0) return cudaSuccess;
   if (grid > 0x7fffffff) return cudaErrorInvalidValue;
@@ -81,7 +89,8 @@ static cudaError_t occ_dg(bool curved, bool integrate, int cb, int *blocks) {
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dg_box_kernel<T, N, false>, groups * N * N,
                                                          (size_t)groups * box_group_values(N) * 8);
   }
-  const size_t smem = (size_t)cb * Tile<N>::CS * sizeof(T);
+  cb = curved_cb<T, N>(cb);
+  const size_t smem = (size_t)cb * curved_cell_values(N, integrate) * sizeof(T);
   return integrate ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dg_integrate_kernel<T, N, false>,
                                                                    cb * N * N, smem)
                    : cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dg_eval_kernel<T, N, false>, cb * N * N,
@@ -93,7 +102,7 @@ static cudaError_t occ_dg(bool curved, bool integrate, int cb, int *blocks) {
 template <typename T, int N>
 static cudaError_t prep_dg_n() {
   constexpr cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  const int smem = max_cb(N, sizeof(T)) * Tile<N>::CS * (int)sizeof(T);
+  const int smem = curved_cb<T, N>(max_cb(N, sizeof(T))) * curved_cell_values(N, true) * (int)sizeof(T);
   const int bsmem = std::min(232448, kCellThreads / (N * N) * box_group_values(N) * 8);
   cudaError_t e = cudaSuccess;
   for (cudaError_t r : {cudaFuncSetAttribute(dg_integrate_kernel<T, N, false>, at, smem),

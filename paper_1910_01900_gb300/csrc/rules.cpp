@@ -264,16 +264,22 @@ void build_tables(Tables<T> &t) {
       }
     put(M1, +1, t.M1E[n], t.M1O[n]);
     put(K1, +1, t.K1E[n], t.K1O[n]);
-    for (int q = 0; q < n; ++q) {
-      t.l0[n][q] = (T)r.l0[q];
-      t.l1[n][q] = (T)r.l1[q];
-      double d0 = 0, d1 = 0;   // (D^T l)[q] = sum_j D[j][q] l[j]
-      for (int j = 0; j < n; ++j) {
-        d0 += r.D[j * n + q] * r.l0[j];
-        d1 += r.D[j * n + q] * r.l1[j];
-      }
-      t.dl0[n][q] = (T)d0;
-      t.dl1[n][q] = (T)d1;
+    std::vector<double> d0(n, 0.0);   // (D^T l0)[q] = sum_j D[j][q] l0[j]
+    for (int q = 0; q < n; ++q)
+      for (int j = 0; j < n; ++j) d0[q] += r.D[j * n + q] * r.l0[j];
+    if (n == 2) {   // two points: the vectors themselves
+      t.le[2][0] = (T)r.l0[0];
+      t.lo[2][0] = (T)r.l0[1];
+      t.de[2][0] = (T)d0[0];
+      t.dod[2][0] = (T)d0[1];
+    }
+    for (int j = 0; n > 2 && j < (n + 1) / 2; ++j) {
+      const int k = n - 1 - j;
+      t.le[n][j] = (T)(j == k ? r.l0[j] : 0.5 * (r.l0[j] + r.l0[k]));
+      t.de[n][j] = (T)(j == k ? d0[j] : 0.5 * (d0[j] + d0[k]));
+      if (j == k) continue;
+      t.lo[n][j] = (T)(0.5 * (r.l0[j] - r.l0[k]));
+      t.dod[n][j] = (T)(0.5 * (d0[j] - d0[k]));
     }
   }
 }

@@ -55,11 +55,11 @@ struct Tables {
   // even-odd blocks (n >= 5): E[hc][hc] stride 5, O[hc][h] stride 4
   T SE[kMaxN + 1][25], SO[kMaxN + 1][20], StE[kMaxN + 1][25], StO[kMaxN + 1][20];
   T DE[kMaxN + 1][25], DO[kMaxN + 1][20], DtE[kMaxN + 1][25], DtO[kMaxN + 1][20];
-  T l0[kMaxN + 1][kMaxN], l1[kMaxN + 1][kMaxN];
-  // D^T l0 and D^T l1: the transposed derivative sweep applied to the face
-  // extrapolation vectors (a face's normal-derivative test term enters the
-  // integrated tile through these directly)
-  T dl0[kMaxN + 1][kMaxN], dl1[kMaxN + 1][kMaxN];
+  // the extrapolation l0 to the lower end (l1 is its mirror image) and D^T l0
+  // (D^T l1 minus its mirror image) in even and odd parts: le[j] + lo[j] = l0[j],
+  // le[j] - lo[j] = l0[n-1-j], de + dod = D^T l0 likewise; the middle entry of
+  // an odd n in le and de (n = 2: the two entries of l0 and of D^T l0)
+  T le[kMaxN + 1][5], lo[kMaxN + 1][4], de[kMaxN + 1][5], dod[kMaxN + 1][4];
   // 1D mass and stiffness matrices of the GL basis under the Gauss rule,
   // M1[i][j] = sum_q w_q l_i(x_q) l_j(x_q), K1[i][j] = sum_q w_q l_i'(x_q) l_j'(x_q)
   // (both M[i][j] = M[n-1-i][n-1-j]): the factors of the Cartesian FE cell matrix
@@ -94,7 +94,7 @@ template <typename T>
 struct DGArgs {
   const T *u;          // input vector (cell-major, n^3 per cell)
   T *out;              // output (mode dependent)
-  T *grad;             // scratch: reference gradient at Gauss points, [cell][3][n^3]
+  T *grad;             // scratch (recompute = 0): values at the Gauss points, [cell][n^3]
   T *trace;            // scratch: face traces, [cell][6 faces][2 (value, d_n)][n^2]
   const T *metric;     // curved: [cell][6][n^3] = w|detJ| J^-1 J^-T (xx,yy,zz,xy,xz,yz)
   const T *wcart;      // Cartesian (setup's diagonal): [3][n^3] = w_q * prod(h)/h_d^2
@@ -109,8 +109,9 @@ struct DGArgs {
   int m[3];
   int ncells;
   int bc[6];
-  // 1: the evaluation pass does not store the gradient and the integration
-  // pass recomputes it from u (less traffic, more arithmetic: used in FP32)
+  // 1: the evaluation pass does not store the values at the Gauss points and
+  // the integration pass interpolates them again (less traffic, more
+  // arithmetic: used in FP32)
   int recompute;
   // epilogue: mode 0 out = Au; 1 out = c1 x + c2 xp + c3 dinv (b - Au); 2 out = b - Au
   int mode;
@@ -284,6 +285,13 @@ template <typename T>
 cudaError_t launch_fe_prolongate_add(const XferGeom &g, const T *P1, const T *xc, T *xf, cudaStream_t s);
 template <typename T>
 cudaError_t launch_fe_restrict_cells(const XferGeom &g, const T *P1, const T *rf, T *ebuf_c, cudaStream_t s);
+// the p-transfers of the default sequence by bricks of cells (prolongation:
+// launch_fe_prolongate_add takes them): r_c = P^T r_f and, with x0, the coarse
+// level's first Chebyshev step x0 = c3 D^-1 r_c, in one launch
+bool fe_transfer_box_ok(const XferGeom &g);
+template <typename T>
+cudaError_t launch_fe_restrict_box(const XferGeom &g, const T *P1, const T *rf, T *rc, T *x0, const T *dinv, T c3,
+                                   cudaStream_t s);
 // node-by-node restriction r_c = P^T r_f in one launch, for the transfers
 // degree 2 -> 1 on one mesh and degree 1 across a 2:1 refinement
 inline bool fe_restrict_nodes_ok(const XferGeom &g) {
