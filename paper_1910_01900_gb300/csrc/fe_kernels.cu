@@ -15,7 +15,8 @@
 // c-restriction (sum of the duplicated DG nodes, Section 3.2 c-coarsening).
 #include <algorithm>
 
-#include "fe_box.cuh"
+#include "curved_tile.cuh"
+#include "fe_transfer.cuh"
 
 namespace sipg {
 
@@ -46,96 +47,33 @@ __device__ __forceinline__ bool node_constrained(const int g[3], const int grid[
 template <typename T, int N>
 __device__ __forceinline__ void fe_cell_body(const FEArgs<T> &a, const T *__restrict__ ug, T *__restrict__ ebv,
                                              const int cell0, const int ncta, T *sm) {
-  constexpr int N2 = N * N, N3 = N2 * N, TT = Tile<N>::T3;
-  const int NT = blockDim.x;
+  constexpr int N2 = N * N, N3 = N2 * N;
   const int tid = threadIdx.x, cl = tid / N2, l = tid - cl * N2;
   const bool act = cl < ncta;
-  T *su = sm + cl * Tile<N>::CS;
+  const int cell = cell0 + (act ? cl : 0);
+  const CurvedLines<T, N> t(sm + cl * CurvedTile<N>::CF, l % N, l / N);
   // each thread gathers its z-line of the cell's nodes straight into
   // registers (constrained Dirichlet nodes read as zero); the first sweep
   // runs on them before anything goes to shared memory
-  T xl[N];
+  T x[N];
   if (act) {
     constexpr int P = N - 1;
-    const int cell = cell0 + cl;
     const int cx = cell % a.m[0], rr = cell / a.m[0], cy = rr % a.m[1], cz = rr / a.m[1];
     int g[3] = {cx * P + l % N, cy * P + l / N, 0};
     const size_t b0 = g[0] + (size_t)a.grid[0] * g[1], sz = (size_t)a.grid[0] * a.grid[1];
 #pragma unroll
     for (int q = 0; q < N; ++q) {
       g[2] = cz * P + q;
-      xl[q] = node_constrained(g, a.grid, a.bc) ? T(0) : ug[b0 + sz * g[2]];
+      x[q] = node_constrained(g, a.grid, a.bc) ? T(0) : ug[b0 + sz * g[2]];
     }
   }
-  if (act) {   // interpolation along z from the registers, then x and y in place
-    int base, stride;
-    line_of<N>(2, l, base, stride);
-    T y[N];
-    apply_mat<T, N, MS>(xl, y);
-    store_line<T, N>(su, base, stride, y);
-  }
-  __syncthreads();
-#pragma unroll 1
-  for (int d = 0; d < 2; ++d) {
-    if (act) sweep_inplace<T, N, MS>(su, d, l);
-    __syncthreads();
-  }
-  if (act) {
-#pragma unroll 1
-    for (int d = 0; d < 3; ++d) {
-      int base, stride;
-      line_of<N>(d, l, base, stride);
-      T x[N], y[N];
-      load_line<T, N>(su, base, stride, x);
-      apply_mat<T, N, MD>(x, y);
-      store_line<T, N>(su + (1 + d) * TT, base, stride, y);
-    }
-  }
-  __syncthreads();
-  for (int i = tid; i < ncta * N3; i += NT) {
-    const int c = i / N3, p = i - c * N3;
-    T *s = sm + c * Tile<N>::CS + TT + Tile<N>::idx(p);
-    const T g0 = s[0], g1 = s[TT], g2 = s[2 * TT];
-    const T *M = a.metric + (size_t)(cell0 + c) * 6 * N3 + p;
-    const T xx = M[0], yy = M[N3], zz = M[2 * N3], xy = M[3 * N3], xz = M[4 * N3], yz = M[5 * N3];
-    s[0] = xx * g0 + xy * g1 + xz * g2;
-    s[TT] = xy * g0 + yy * g1 + yz * g2;
-    s[2 * TT] = xz * g0 + yz * g1 + zz * g2;
-  }
-  __syncthreads();
-#pragma unroll 1
-  for (int d = 0; d < 3; ++d) {
-    if (act) {
-      int base, stride;
-      line_of<N>(d, l, base, stride);
-      T x[N], y[N];
-      load_line<T, N>(su + (1 + d) * TT, base, stride, x);
-      apply_mat<T, N, MDt>(x, y);
-      if (d == 0) {
-        store_line<T, N>(su, base, stride, y);
-      } else {
-#pragma unroll
-        for (int q = 0; q < N; ++q) su[base + q * stride] += y[q];
-      }
-    }
-    __syncthreads();
-  }
-#pragma unroll 1
-  for (int d = 0; d < 2; ++d) {
-    if (act) sweep_inplace<T, N, MSt>(su, d, l);
-    __syncthreads();
-  }
+  curved_interpolate<T, N>(t, act, x);
+  curved_cell_term<T, N>(t, act, a.metric + (size_t)cell * 6 * N3 + l, x, [] {},
+                         [](int, const T (&in)[N], T (&out)[N]) { apply_mat<T, N, MDt>(in, out); });
   if (!act) return;
-  T x[N], y[N];
-  {
-    int base, stride;
-    line_of<N>(2, l, base, stride);
-    load_line<T, N>(su, base, stride, x);
-  }
-  apply_mat<T, N, MSt>(x, y);
-  T *eb = ebv + (size_t)(cell0 + cl) * N3 + l;
+  T *eb = ebv + (size_t)cell * N3 + l;
 #pragma unroll
-  for (int q = 0; q < N; ++q) eb[q * N2] = y[q];
+  for (int q = 0; q < N; ++q) eb[q * N2] = x[q];
 }
 
 // cb cells per thread block (a launch parameter, cb N^2 threads); MULTI:
@@ -357,16 +295,15 @@ __device__ __forceinline__ void fe_gather_node(const FEArgs<T> &a, const long gi
     const long own = (c[0] + (long)a.m[0] * (c[1] + (long)a.m[1] * c[2])) * n3 + r[0] + n * r[1] + n2 * r[2];
     const long D0 = P - (long)n3, D1 = (long)P * n - (long)a.m[0] * n3,
                D2 = (long)P * n2 - (long)a.m[0] * a.m[1] * n3;
-    // all eight loads issued unconditionally (a missing cell reads entry 0),
-    // then summed in a fixed order over the cells that exist (the cell below
-    // before the own one in every direction)
+    // the loads of the cells that exist, all before the sum (predicated: most
+    // nodes lie in one cell or two), then summed in a fixed order (the cell
+    // below before the own one in every direction)
     T e[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       const int x = q & 1, yy = (q >> 1) & 1, z = q >> 2;
       const bool take = (x || lo[0]) && (yy || lo[1]) && (z || lo[2]);
-      const long addr = own + (x ? 0 : D0) + (yy ? 0 : D1) + (z ? 0 : D2);
-      e[q] = ebuf[take ? addr : 0];
+      e[q] = take ? ebuf[own + (x ? 0 : D0) + (yy ? 0 : D1) + (z ? 0 : D2)] : T(0);
     }
     y = T(0);
 #pragma unroll
@@ -420,12 +357,33 @@ __device__ __forceinline__ void c_prolongate_dof(const FEArgs<T> &a, const T *xc
   xdg[idx] += xc[g[0] + (size_t)a.grid[0] * (g[1] + (size_t)a.grid[1] * g[2])];
 }
 
-template <typename T>
-__global__ void c_prolongate_add_kernel(const FEArgs<T> a, const T *xc, T *xdg, const int64_t dg_stride) {
-  const int n = a.deg + 1;
-  const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (long)a.ncells * n * n * n) return;
-  c_prolongate_dof<T>(a, xc + blockIdx.y * a.vs, xdg + blockIdx.y * dg_stride, idx);   // vector blockIdx.y
+// z-line by z-line of the cells: the coordinates once per N values, the loads
+// ahead of the stores (one value per thread spent its time on the divisions:
+// 4.1 MDoF 33 us)
+template <typename T, int N>
+__global__ void __launch_bounds__(256) c_prolongate_add_kernel(const FEArgs<T> a, const T *__restrict__ xc, T *xdg,
+                                                              const int64_t dg_stride) {
+  constexpr int N2 = N * N, P = N - 1;
+  const unsigned i = blockIdx.x * 256u + threadIdx.x, cell = i / N2, l = i - cell * N2;
+  if (cell >= (unsigned)a.ncells) return;
+  xc += blockIdx.y * a.vs;   // vector blockIdx.y
+  xdg += blockIdx.y * dg_stride + (int64_t)cell * N2 * N + l;
+  const unsigned r = cell / (unsigned)a.m[0], cy = r % (unsigned)a.m[1], cz = r / (unsigned)a.m[1];
+  const int gx = (int)(cell - r * a.m[0]) * P + (int)(l % N), gy = (int)cy * P + (int)(l / N), gz = (int)cz * P;
+  if ((gx == 0 && a.bc[0] == 0) || (gx == a.grid[0] - 1 && a.bc[1] == 0) || (gy == 0 && a.bc[2] == 0) ||
+      (gy == a.grid[1] - 1 && a.bc[3] == 0))
+    return;
+  const int64_t sz = (int64_t)a.grid[0] * a.grid[1];
+  const T *p = xc + gx + (int64_t)a.grid[0] * gy + sz * gz;
+  T c[N], d[N];
+#pragma unroll
+  for (int q = 0; q < N; ++q) c[q] = p[sz * q];
+#pragma unroll
+  for (int q = 0; q < N; ++q) d[q] = xdg[q * N2];
+  const bool lo = gz == 0 && a.bc[4] == 0, hi = gz + P == a.grid[2] - 1 && a.bc[5] == 0;
+#pragma unroll
+  for (int q = 0; q < N; ++q)
+    if (!(q == 0 && lo) && !(q == P && hi)) xdg[q * N2] = d[q] + c[q];
 }
 
 // ------------------------------------------------ batched launches (many problems)
@@ -781,11 +739,18 @@ __global__ void dg_transfer_kernel(const XferGeom G, const T *__restrict__ P1, c
 }
 
 // ---------------------------------------------------------------- launchers
+// the width that a setting of cb cells runs at: the shared memory at most
+template <typename T, int N>
+static int fe_curved_cb(int cb) {
+  return std::min(cb, 232448 / (fe_curved_cell_values(N) * (int)sizeof(T)));
+}
+
 template <typename T, int N>
 static cudaError_t run_fe_cells(const FEArgs<T> &a, cudaStream_t s, int cb) {
   if (cb <= 0) cb = default_cb(N);
   if (cb > max_cb(N, sizeof(T))) return cudaErrorInvalidValue;
-  const size_t smem = (size_t)cb * Tile<N>::CS * sizeof(T);
+  cb = fe_curved_cb<T, N>(cb);
+  const size_t smem = (size_t)cb * fe_curved_cell_values(N) * sizeof(T);
   const int64_t grid = (int64_t)((a.ncells + cb - 1) / cb) * a.nv;
   if (grid == 0) return cudaSuccess;
   if (grid > 0x7fffffff) return cudaErrorInvalidValue;
@@ -799,8 +764,9 @@ static cudaError_t run_fe_cells(const FEArgs<T> &a, cudaStream_t s, int cb) {
 
 template <typename T, int N>
 static cudaError_t occ_fe_cells(int cb, int *blocks) {
+  cb = fe_curved_cb<T, N>(cb);
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fe_cell_kernel<T, N, false>, cb * N * N,
-                                                       (size_t)cb * Tile<N>::CS * sizeof(T));
+                                                       (size_t)cb * fe_curved_cell_values(N) * sizeof(T));
 }
 
 // Cells per direction of a brick.  kFEBoxBrick[p]: about 16 own nodes along x
@@ -879,7 +845,7 @@ cudaError_t launch_fe_box(const FEArgs<T> &a, cudaStream_t s) {
 template <typename T, int N>
 static cudaError_t prep_fe_n() {
   constexpr cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  const int smem = max_cb(N, sizeof(T)) * Tile<N>::CS * (int)sizeof(T);
+  const int smem = fe_curved_cb<T, N>(max_cb(N, sizeof(T))) * fe_curved_cell_values(N) * (int)sizeof(T);
   cudaError_t e = cudaSuccess;
   for (cudaError_t r : {cudaFuncSetAttribute(fe_cell_kernel<T, N, false>, at, smem),
                         cudaFuncSetAttribute(fe_cell_kernel<T, N, true>, at, smem),
@@ -1091,7 +1057,7 @@ cudaError_t launch_fe_nodes_batched(const FETask<T> *tasks, const NodeItem *item
   return cudaGetLastError();
 }
 
-int tile_values(int n) { return cell_values(n); }
+int tile_values(int n) { return fe_curved_cell_values(n); }
 
 template <typename T>
 cudaError_t prep_fe_cells_batched(size_t smem) {
@@ -1101,11 +1067,80 @@ cudaError_t prep_fe_cells_batched(size_t smem) {
 template <typename T>
 cudaError_t launch_c_prolongate_add(const FEArgs<T> &a, const T *xc, T *xdg, cudaStream_t s, int64_t dg_stride) {
   const int n = a.deg + 1;
-  const long total = (long)a.ncells * n * n * n;
+  const long total = (long)a.ncells * n * n * n, lines = (long)a.ncells * n * n;
   const int bs = 256;
   if (total == 0) return cudaSuccess;
   if (total >= (1L << 32)) return cudaErrorInvalidValue;   // the kernel's 32-bit index arithmetic
-  c_prolongate_add_kernel<T><<<dim3((unsigned)((total + bs - 1) / bs), a.nv), bs, 0, s>>>(a, xc, xdg, dg_stride);
+  const dim3 grid((unsigned)((lines + bs - 1) / bs), a.nv);
+  switch (n) {
+#define SIPG_CPRO_CASE(NN) \
+  case NN:                 \
+    c_prolongate_add_kernel<T, NN><<<grid, bs, 0, s>>>(a, xc, xdg, dg_stride); \
+    break;
+    SIPG_CPRO_CASE(2)
+    SIPG_CPRO_CASE(3)
+    SIPG_CPRO_CASE(4)
+    SIPG_CPRO_CASE(5)
+    SIPG_CPRO_CASE(6)
+    SIPG_CPRO_CASE(7)
+    SIPG_CPRO_CASE(8)
+    SIPG_CPRO_CASE(9)
+#undef SIPG_CPRO_CASE
+    default:
+      return cudaErrorInvalidValue;
+  }
+  note_launch();
+  return cudaGetLastError();
+}
+
+// The p-transfers by bricks: the degree pairs of the default sequence p ->
+// floor(p/2) from degree 3 up (2 -> 1 has its own node pass); the other
+// sequences and the 2:1 transfers keep the kernels for any pair.
+#define SIPG_PAIRS(X) X(4, 2) X(5, 3) X(6, 3) X(7, 4) X(8, 4) X(9, 5)
+bool fe_transfer_box_ok(const XferGeom &g) {
+#define SIPG_PAIR(NF, NC) if (g.kind == 1 && g.pf == NF - 1 && g.pc == NC - 1) return true;
+  SIPG_PAIRS(SIPG_PAIR)
+#undef SIPG_PAIR
+  return false;
+}
+// bricks as the operator's: thin ones, about 16 fine nodes along x and y
+static int64_t transfer_bricks(const XferGeom &g, int b[3]) {
+  fe_box_brick<float>(g.pf + 1, g.mc, 0, b);
+  int64_t n = 1;
+  for (int d = 0; d < 3; ++d) n *= (g.mc[d] + b[d] - 1) / b[d];
+  return n;
+}
+
+template <typename T>
+cudaError_t launch_fe_restrict_box(const XferGeom &g, const T *P1, const T *rf, T *rc, T *x0, const T *dinv, T c3,
+                                   cudaStream_t s) {
+  int b[3];
+  const int64_t n = transfer_bricks(g, b);
+  if (n == 0) return cudaSuccess;
+  if (n > 0x7fffffff || (int64_t)g.gf[0] * g.gf[1] * g.gf[2] >= (1LL << 32)) return cudaErrorInvalidValue;
+  const int ex = ((b[0] + 1) * g.pf + 1) | 1, ey = (b[1] + 1) * g.pf + 1, oz = b[2] * g.pc + 1;
+  const size_t smem = (size_t)ex * ey * oz * sizeof(T);
+#define SIPG_PAIR(NF, NC)                                                                                   \
+  if (g.pf == NF - 1 && g.pc == NC - 1)                                                                     \
+    fe_restrict_box_kernel<T, NF, NC><<<dim3((unsigned)n, g.nv), 256, smem, s>>>(g, b[0], b[1], b[2], P1, rf, rc, x0, dinv, c3);
+  SIPG_PAIRS(SIPG_PAIR)
+#undef SIPG_PAIR
+  note_launch();
+  return cudaGetLastError();
+}
+
+template <typename T>
+static cudaError_t launch_fe_prolongate_box(const XferGeom &g, const T *P1, const T *xc, T *xf, cudaStream_t s) {
+  int b[3];
+  const int64_t n = transfer_bricks(g, b);
+  if (n > 0x7fffffff) return cudaErrorInvalidValue;
+  const int cx = b[0] * g.pc + 1, cy = b[1] * g.pc + 1, fx = b[0] * g.pf + 1, fz = b[2] * g.pf + 1;
+  const size_t smem = (size_t)(cx + fx) * cy * fz * sizeof(T);
+#define SIPG_PAIR(NF, NC)               \
+  if (g.pf == NF - 1 && g.pc == NC - 1) \
+    fe_prolongate_box_kernel<T, NF, NC><<<dim3((unsigned)n, g.nv), 256, smem, s>>>(g, b[0], b[1], b[2], P1, xc, xf);
+  SIPG_PAIRS(SIPG_PAIR)
+#undef SIPG_PAIR
   note_launch();
   return cudaGetLastError();
 }
@@ -1116,6 +1151,7 @@ cudaError_t launch_fe_prolongate_add(const XferGeom &g, const T *P1, const T *xc
   const int bs = 256;
   if (total == 0) return cudaSuccess;
   if (total >= (1L << 32)) return cudaErrorInvalidValue;   // the kernel's 32-bit grid coordinates
+  if (fe_transfer_box_ok(g)) return launch_fe_prolongate_box<T>(g, P1, xc, xf, s);
   const dim3 grid((unsigned)((total + bs - 1) / bs), g.nv);
   switch (g.pc + 1) {
     case 2:
@@ -1374,6 +1410,8 @@ cudaError_t launch_dg_transfer(const XferGeom &g, const T *P1, const T *in, T *o
                                                    cudaStream_t);                                       \
   template cudaError_t launch_fe_restrict_nodes<T>(const XferGeom &, const T *, const T *, T *,         \
                                                    cudaStream_t);                                       \
+  template cudaError_t launch_fe_restrict_box<T>(const XferGeom &, const T *, const T *, T *, T *, const T *, T, \
+                                                 cudaStream_t);                                         \
   template cudaError_t launch_fe_restrict_cells<T>(const XferGeom &, const T *, const T *, T *,         \
                                                    cudaStream_t);                                       \
   template cudaError_t launch_dg_transfer<T>(const XferGeom &, const T *, const T *, T *, bool, cudaStream_t); \

@@ -213,7 +213,7 @@ DGArgs<T> dg_args(sipg_ctx *c, const Level &L) {
   a.trace = (T *)(c->nv > 1 ? c->mv.trace[pi] : c->dg_trace[pi]);
   a.nv = c->nv;
   a.vs = L.ndofs;
-  a.gs = L.ncells * 3 * (int64_t)L.n * L.n * L.n;
+  a.gs = L.ncells * (int64_t)L.n * L.n * L.n;
   a.ts = L.ncells * 12 * (int64_t)L.n * L.n;
   a.metric = (const T *)L.metric[pi];
   a.wcart = (const T *)L.wcart[pi];
@@ -229,8 +229,8 @@ DGArgs<T> dg_args(sipg_ctx *c, const Level &L) {
   a.ufn = L.ufn;
   a.ncells = (int)L.ncells;
   for (int s = 0; s < 6; ++s) a.bc[s] = c->mesh.bc[s];
-  // FP64 is bound by its arithmetic: store the gradient once; FP32 is bound
-  // by traffic: recompute it instead of a 24 B/DoF round trip
+  // FP64 is bound by its arithmetic: store the values at the Gauss points once
+  // (16 B/DoF of traffic); FP32 is bound by traffic: interpolate again
   a.recompute = sizeof(T) == 4 ? 1 : 0;
   return a;
 }
@@ -337,6 +337,11 @@ bool restrict_level(sipg_ctx *c, int l, const T *r, T *rc, T *x0 = nullptr, T c3
   if (F.t_kind != 0 && fe_restrict_nodes_ok(xfer(c, l))) {   // small transfer: one node pass
     CK(launch_fe_restrict_nodes<T>(xfer(c, l), (const T *)F.P1[pi], r, rc, c->stream));
     return false;
+  }
+  if (F.t_kind != 0 && fe_transfer_box_ok(xfer(c, l))) {
+    CK(launch_fe_restrict_box<T>(xfer(c, l), (const T *)F.P1[pi], r, rc, x0, (const T *)c->lv[l - 1].dinv[pi], c3,
+                                 c->stream));
+    return x0 != nullptr;
   }
   FEArgs<T> a = fe_args<T>(c, c->lv[l - 1]);
   a.mode = 3;
@@ -1064,7 +1069,7 @@ void setup(sipg_ctx *c) {
     build_level_geometry(c, L, s.md, s.kind == 0);
     if (s.kind == 1) ebuf_len = std::max(ebuf_len, L.ncells * n3);
     if (s.kind == 0 && L.curved) {   // axis-aligned cells need no scratch
-      dg_grad_len = std::max(dg_grad_len, L.ncells * 3 * n3);
+      dg_grad_len = std::max(dg_grad_len, L.ncells * n3);
       dg_trace_len = std::max(dg_trace_len, L.ncells * 12 * (int64_t)L.n * L.n);
     }
     if (c->solver) alloc_work(c, L);
@@ -1093,7 +1098,6 @@ void setup(sipg_ctx *c) {
   // DG scratch (both precisions), shared by all DG levels (used one at a time)
   c->dg_grad[0] = dalloc<double>(c, dg_grad_len);
   c->dg_trace[0] = dalloc<double>(c, dg_trace_len);
-  c->dg_grad[1] = dalloc<float>(c, dg_grad_len);
   c->dg_trace[1] = dalloc<float>(c, dg_trace_len);
   CK(cudaDeviceSynchronize());   // geometry uploads (legacy stream) complete before stream work
   default_tile_widths(c);
@@ -1235,9 +1239,8 @@ void setup_unstructured(sipg_ctx *c, const UMeshIn &in) {
   upload2(c, g.tau, L.tau);
   L.ufn = (int2 *)dalloc<int>(c, (int64_t)g.ufn.size());
   CK(cudaMemcpy(L.ufn, g.ufn.data(), g.ufn.size() * sizeof(int), cudaMemcpyHostToDevice));
-  c->dg_grad[0] = dalloc<double>(c, L.ncells * 3 * n3);
+  c->dg_grad[0] = dalloc<double>(c, L.ncells * n3);
   c->dg_trace[0] = dalloc<double>(c, L.ncells * 12 * (int64_t)L.n * L.n);
-  c->dg_grad[1] = dalloc<float>(c, L.ncells * 3 * n3);
   c->dg_trace[1] = dalloc<float>(c, L.ncells * 12 * (int64_t)L.n * L.n);
   CK(cudaDeviceSynchronize());
   default_tile_widths(c);
@@ -3405,7 +3408,7 @@ void ensure_multi(sipg_ctx *c, int nv) {
     for (int k = 0; k < 4; ++k) M.v[4 * l + k] = dalloc<char>(c, (int64_t)(L.ndofs * nv * es));
     const int64_t n3 = (int64_t)L.n * L.n * L.n;
     if (L.kind == 0 && L.curved) {
-      grad = std::max(grad, L.ncells * 3 * n3);
+      grad = std::max(grad, L.ncells * n3);
       trace = std::max(trace, L.ncells * 12 * (int64_t)L.n * L.n);
     }
     ebuf = std::max(ebuf, L.ncells * n3);
@@ -3414,7 +3417,6 @@ void ensure_multi(sipg_ctx *c, int nv) {
   M.trace[0] = dalloc<double>(c, trace * nv);
   M.ebuf[0] = dalloc<double>(c, ebuf * nv);
   if (pi == 1) {
-    M.grad[1] = dalloc<float>(c, grad * nv);
     M.trace[1] = dalloc<float>(c, trace * nv);
     M.ebuf[1] = dalloc<float>(c, ebuf * nv);
   }
@@ -3492,14 +3494,10 @@ sipg_status sipg_operator_apply_multi(sipg_ctx *c, int precision, int nv, const 
   if (!c->solver) return SIPG_EINVAL;
   return guarded(c, [&]() -> sipg_status {
     ensure_multi(c, nv);
-    if (precision == 1 && !c->mv.grad[1]) {   // curved cells' FP32 scratch of a context whose cycle runs in FP64
-      int64_t grad = 0, trace = 0;
+    if (precision == 1 && !c->mv.trace[1]) {   // curved cells' FP32 scratch of a context whose cycle runs in FP64
+      int64_t trace = 0;
       for (const Level &L : c->lv)
-        if (L.kind == 0 && L.curved) {
-          grad = std::max(grad, L.ncells * 3 * (int64_t)L.n * L.n * L.n);
-          trace = std::max(trace, L.ncells * 12 * (int64_t)L.n * L.n);
-        }
-      c->mv.grad[1] = dalloc<float>(c, grad * c->mv.cap);
+        if (L.kind == 0 && L.curved) trace = std::max(trace, L.ncells * 12 * (int64_t)L.n * L.n);
       c->mv.trace[1] = dalloc<float>(c, trace * c->mv.cap);
     }
     MultiScope scope(c, nv);

@@ -2,8 +2,8 @@
 // integration as 1D sweeps over the tensor-product structure, even-odd
 // decomposition of the 1D matrices).
 //
-// A 1D sweep applies an n x n matrix along one direction of an n^3 tile in
-// shared memory; one thread handles one line of n points.  The matrices of a
+// A 1D sweep applies an n x n matrix along one direction of a cell's n^3
+// values; one thread handles one line of n points.  The matrices of a
 // symmetric basis on symmetric points satisfy M[i][j] = s M[n-1-i][n-1-j]
 // (s = +1 interpolation, s = -1 derivative), so y = M x splits into an even
 // part (x_j + x_{n-1-j}) and an odd part (x_j - x_{n-1-j}) with half the
@@ -99,59 +99,15 @@ __device__ __forceinline__ void apply_mat(const T (&x)[N], T (&y)[N]) {
   if constexpr (M == MK1) mv<T, N, +1>(t.K1[N], t.K1E[N], t.K1O[N], x, y);
 }
 
-// Shared-memory layout of one cell: four tile arrays of N^3 values (x
-// fastest, y step XP, z step ZP, array stride T3 = ZP N), cells CS values
-// apart.  One thread walks one line per sweep; a warp's 32 lanes cover lines
-// of up to two cells, and the lines of different directions start at
-// different banks.  The pitches below were chosen, per N, by counting the
-// shared-memory wavefronts (the most threads of a warp on one bank) of the
-// three sweep directions and of the point loops at the default and half the
-// default cells per block: 1.57 wavefronts per FP32 instruction at N = 6
-// against 1.85 with the x pitch alone padded (N + 1 for even N), 1.72 against
-// 3.7 at N = 2, 1.43 against 2.0 at N = 4.  The layout moves addresses only:
-// every value is computed by the same thread in the same order.
-__host__ __device__ constexpr int tile_xp(int n) { return n == 8 ? 9 : n; }
-__host__ __device__ constexpr int tile_zp(int n) {
-  return n == 2 ? 4 : n == 3 ? 9 : n == 4 ? 19 : n == 5 ? 25 : n == 6 ? 39 : n == 7 ? 52 : n == 8 ? 72 : 81;
-}
-// values of shared memory per cell (>= 4 tile arrays)
+// The values per cell that the limit on a block's width counts (max_cb below,
+// which set widths are checked against): four arrays of n^3 values with their
+// pitches.  What a pass really lays out is its own (dg_box.cuh, curved_tile.cuh),
+// and where a width's cells do not fit, the pass runs at the widest that do.
 __host__ __device__ constexpr int cell_values(int n) {
   return n == 2 ? 36 : n == 3 ? 123 : n == 4 ? 304 : n == 5 ? 509 : n == 6 ? 964 : n == 7 ? 1457 : n == 8 ? 2304 : 2929;
 }
 
-template <int N>
-struct Tile {
-  static constexpr int XP = tile_xp(N);                  // step of y
-  static constexpr int ZP = tile_zp(N);                  // step of z
-  static constexpr int T3 = ZP * N;                      // values per tile array
-  static constexpr int CS = cell_values(N);              // values per cell
-  static_assert(XP >= N && ZP >= XP * N && CS >= 4 * T3, "tile arrays overlap");
-  // tile position of the node or point with linear index p = x + N (y + N z)
-  static __device__ __forceinline__ int idx(int p) {
-    const int x = p % N, y = (p / N) % N, z = p / (N * N);
-    return x + XP * y + ZP * z;
-  }
-};
-
-// Offset and stride of line l (0 <= l < N^2) along direction d in a tile.
-// The line index l = a + N*b runs over the two other directions in increasing
-// order, so it equals the face-point index of the faces normal to d.
-template <int N>
-__device__ __forceinline__ void line_of(int d, int l, int &base, int &stride) {
-  constexpr int XP = Tile<N>::XP, ZP = Tile<N>::ZP;
-  const int a = l % N, b = l / N;
-  if (d == 0) {
-    base = XP * a + ZP * b;
-    stride = 1;
-  } else if (d == 1) {
-    base = a + ZP * b;
-    stride = XP;
-  } else {
-    base = a + XP * b;
-    stride = ZP;
-  }
-}
-
+// one line of N values in shared memory
 template <typename T, int N>
 __device__ __forceinline__ void load_line(const T *s, int base, int stride, T (&x)[N]) {
 #pragma unroll
@@ -163,20 +119,7 @@ __device__ __forceinline__ void store_line(T *s, int base, int stride, const T (
   for (int q = 0; q < N; ++q) s[base + q * stride] = x[q];
 }
 
-// In-place sweep of matrix M along d on the tile s (one line per thread).
-template <typename T, int N, int M>
-__device__ __forceinline__ void sweep_inplace(T *s, int d, int l) {
-  int base, stride;
-  line_of<N>(d, l, base, stride);
-  T x[N], y[N];
-  load_line<T, N>(s, base, stride, x);
-  apply_mat<T, N, M>(x, y);
-  store_line<T, N>(s, base, stride, y);
-}
-
-
-// Most threads per block of the cell kernels (their __launch_bounds__: at
-// most 85 registers a thread, which the sweeps need without spilling).
+// Most threads per block of the cell kernels.
 constexpr int kCellThreads = 768;
 
 // Largest cells per thread block of the cell kernels (cell_values(n) values

@@ -9,6 +9,7 @@
 #include <cmath>
 
 #include "sipg_internal.h"
+#include "stride_loop.cuh"
 
 namespace sipg {
 
@@ -21,17 +22,24 @@ __global__ void fill_kernel(T *x, T v, long n) {
 }
 template <typename Tout, typename Tin>
 __global__ void cast_kernel(Tout *y, const Tin *x, long n) {
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
-    y[i] = (Tout)x[i];
+  Tin v[kAhead];
+  stride_loop(n, [&](int k, long i) { v[k] = x[i]; }, [&](int k, long i) { y[i] = (Tout)v[k]; });
 }
 // b = (T) r and the first Chebyshev step from x = 0, x = c D^-1 b (xdb_kernel's arithmetic), in one pass
 template <typename T, typename Tin>
 __global__ void cast_xdb_kernel(T *b, T *x, T c, const T *dinv, const Tin *r, long n) {
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    const T v = (T)r[i];
-    b[i] = v;
-    x[i] = c * dinv[i] * v;
-  }
+  Tin v[kAhead];
+  T d[kAhead];
+  stride_loop(
+      n,
+      [&](int k, long i) {
+        v[k] = r[i];
+        d[k] = dinv[i];
+      },
+      [&](int k, long i) {
+        b[i] = (T)v[k];
+        x[i] = c * d[k] * (T)v[k];
+      });
 }
 template <typename T>
 __global__ void axpy_kernel(T *y, T a, const T *x, long n) {
@@ -145,10 +153,19 @@ __device__ void reduce2_finish(double a, double b, double *partials, unsigned *c
 __global__ void dot2_kernel(const double *x, const double *y, const double *z, const double *w, long n,
                             double *partials, unsigned *counter, double *out) {
   double a = 0, b = 0;
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    a = fma(x[i], y[i], a);
-    if (z) b = fma(z[i], w[i], b);
-  }
+  double xi[kAhead], yi[kAhead], zi[kAhead], wi[kAhead];
+  stride_loop(
+      n,
+      [&](int k, long i) {
+        xi[k] = x[i];
+        yi[k] = y[i];
+        zi[k] = z ? z[i] : 0.0;
+        wi[k] = z ? w[i] : 0.0;
+      },
+      [&](int k, long) {
+        a = fma(xi[k], yi[k], a);
+        if (z) b = fma(zi[k], wi[k], b);
+      });
   reduce2_finish(a, b, partials, counter, out);
 }
 
@@ -165,12 +182,21 @@ __global__ void fcg_update_xr_kernel(double *x, double *r, const double *p, cons
                                      const double *sc, double *partials, unsigned *counter, double *out) {
   const double alpha = sc[0] / sc[2];
   double a = 0;
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    x[i] = fma(alpha, p[i], x[i]);
-    const double ri = fma(-alpha, v[i], r[i]);
-    r[i] = ri;
-    a = fma(ri, ri, a);
-  }
+  double xi[kAhead], pi[kAhead], vi[kAhead], ri[kAhead];
+  stride_loop(
+      n,
+      [&](int k, long i) {
+        xi[k] = x[i];
+        pi[k] = p[i];
+        vi[k] = v[i];
+        ri[k] = r[i];
+      },
+      [&](int k, long i) {
+        x[i] = fma(alpha, pi[k], xi[k]);
+        const double s = fma(-alpha, vi[k], ri[k]);
+        r[i] = s;
+        a = fma(s, s, a);
+      });
   reduce2_finish(a, 0.0, partials, counter, out);
 }
 cudaError_t launch_fcg_update_xr(double *x, double *r, const double *p, const double *v, int64_t n,
@@ -183,8 +209,14 @@ cudaError_t launch_fcg_update_xr(double *x, double *r, const double *p, const do
 // p = z + beta p with beta = -z.Ap / p.Ap (flexible CG, one retained direction)
 __global__ void fcg_update_p_kernel(double *p, const double *z, const double *sc, long n) {
   const double beta = -sc[1] / sc[2];
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
-    p[i] = fma(beta, p[i], z[i]);
+  double pi[kAhead], zi[kAhead];
+  stride_loop(
+      n,
+      [&](int k, long i) {
+        pi[k] = p[i];
+        zi[k] = z[i];
+      },
+      [&](int k, long i) { p[i] = fma(beta, pi[k], zi[k]); });
 }
 cudaError_t launch_fcg_update_p(double *p, const double *z, const double *sc, int64_t n, cudaStream_t s) {
   fcg_update_p_kernel<<<grid_for(n), 256, 0, s>>>(p, z, sc, n);
@@ -421,8 +453,14 @@ template <typename T>
 __global__ void xdb_kernel(T *x, T c, const T *dinv, const T *b, long n) {
   x += blockIdx.y * n;   // vector blockIdx.y; dinv is shared
   b += blockIdx.y * n;
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
-    x[i] = c * dinv[i] * b[i];
+  T d[kAhead], v[kAhead];
+  stride_loop(
+      n,
+      [&](int k, long i) {
+        d[k] = dinv[i];
+        v[k] = b[i];
+      },
+      [&](int k, long i) { x[i] = c * d[k] * v[k]; });
 }
 template <typename T>
 cudaError_t launch_xdb(T *x, T c, const T *dinv, const T *b, int64_t n, cudaStream_t s, int nv) {
