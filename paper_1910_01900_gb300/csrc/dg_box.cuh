@@ -34,8 +34,8 @@
 //
 // Measured at 16 MDoF (GB300) against the two-pass scheme with stored traces
 // that axis-aligned cells had before: FP32 k = 3 / 5 / 7 204 / 191 / 165 us ->
-// 68 / 71 / 76 us, FP64 k = 3 / 5 / 7 2440 / 2590 / 2860 us -> 1481 / 1559 /
-// 1802 us; errors against 64 bits no larger (FP32 k = 7: 1.5e-7, before
+// 69 / 71 / 75 us, FP64 k = 3 / 5 / 7 2440 / 2590 / 2860 us -> 1389 / 1495 /
+// 1759 us; errors against 64 bits no larger (FP32 k = 7: 1.5e-7, before
 // 2.5e-7: fewer roundings, end values read instead of extrapolated).  Now
 // FP32 is bound by the L1 data pipe (k = 4: 73% of its wavefronts, 41% shared
 // memory, 32% global lines), FP64 by the FP64 pipe (84% busy).
@@ -105,7 +105,11 @@ __device__ __forceinline__ double vfma(double a, double b, double c) { return fm
 __device__ __forceinline__ double vadd(double a, double b) { return a + b; }
 __device__ __forceinline__ double vsub(double a, double b) { return a - b; }
 __device__ __forceinline__ double vmul(double a, double b) { return a * b; }
-__device__ __forceinline__ double vmax(double a, double b) { return fmax(a, b); }
+// of positive numbers: their order is that of their bits, and integer
+// instructions leave the FP64 pipe alone
+__device__ __forceinline__ double vmax(double a, double b) {
+  return __longlong_as_double(max(__double_as_longlong(a), __double_as_longlong(b)));
+}
 // -a where s is negative (the sign bit alone: no FP64 instruction)
 __device__ __forceinline__ double vsign(double a, bool s) {
   return __longlong_as_double(__double_as_longlong(a) ^ ((long long)s << 63));
@@ -346,6 +350,23 @@ struct BoxEnd {
   V t, u, q;
 };
 
+// The penalty of the thread's cells.  FP64 reads tau_e h_d of the direction
+// (tauh; on the FP64 pipe the products would cost two of its instructions per
+// line: 4.1 MDoF of degree 4 410 us with them, now 384 us), FP32 tau_e once for
+// the three directions and multiplies (its loads are what it is short of: 16.8
+// MDoF of degree 7 74 us, with tauh 80 us).
+template <typename V, typename T>
+__device__ __forceinline__ V box_tau(const DGArgs<T> &a, const int d, const int cell, const int cell1) {
+  if constexpr (BoxLane<V>::pair) return F2{a.tau[cell], a.tau[cell1]};
+  else return a.tauh[(size_t)d * a.ncells + cell];
+}
+// tau_f h_d of the larger of two such penalties
+template <typename V, typename T>
+__device__ __forceinline__ V box_penalty(const DGArgs<T> &a, const int d, const V t0, const V t1) {
+  if constexpr (BoxLane<V>::pair) return vmul(vmax(t0, t1), BoxLane<V>::all(a.hd[d]));
+  else return vmax(t0, t1);
+}
+
 // The end read from memory: the neighbour dc cells away, whose line (start o0,
 // o1 in the two cells, step st) is read towards us, or at an edge the own line.
 template <typename T, int N, typename V>
@@ -357,10 +378,7 @@ __device__ __forceinline__ void box_outside(const DGArgs<T> &a, const T *u0, con
   const int c = edge ? 0 : dc, q = rev ? -st : st;
   const ptrdiff_t w = (ptrdiff_t)c * (N * N * N) + (rev ? (N - 1) * st : 0);
   box_fetch<N>(u0 + (w + o0), q, u1 + (w + o1), q, f);
-  V tn;
-  if constexpr (BoxLane<V>::pair) tn = F2{a.tau[cell + c], a.tau[cell1 + c]};
-  else tn = a.tau[cell + c];
-  b.t = vmul(vmax(tau, tn), BoxLane<V>::all(a.hd[d]));
+  b.t = box_penalty(a, d, tau, box_tau<V>(a, d, cell + c, cell1 + c));
   b.u = vsign(f[N - 1], edge && neg);
   b.q = vsign(box_end<V, N>(f), edge && neg);
 }
@@ -403,14 +421,14 @@ __device__ __forceinline__ void dg_box_body(const DGArgs<T> &a, const VecPtrs<T>
   const int oz = N * at(dy.p, lb) + (dz.p ? (N - 1) * N2 : 0);                    // z-line (x, y) = (la, lb)
   const int oy = N2 * at(dz.p, lb) + (dy.p ? (N - 1) * N : 0);                    // y-line (x, z) = (la, lb)
   const int ox = N * at(dy.p, la) + N2 * at(dz.p, lb);                            // x-line (y, z) = (la, lb)
-  V tau;
-  if constexpr (P2) tau = F2{a.tau[cell], a.tau[cell1]};
-  else tau = a.tau[cell];
+  V tau;   // the own cells' penalty
+  if constexpr (P2) tau = box_tau<V>(a, 0, cell, cell1);
 
   V x[N], y[N];
   BoxEnd<V> ef, en;
   // both ends of a y- or z-line (and an FP64 x-line) as far as they come from memory
   auto outer = [&](const int d, const BoxDir &b, const int o0, const int o1, const int st) {
+    if constexpr (!P2) tau = box_tau<V>(a, d, cell, cell1);
     box_outside<T, N, V>(a, u0, u1, cell, cell1, tau, d, b.far_edge, b.far_dir, -b.cs, b.far_edge, o0, o1, st, ef);
     if (!b.shared)
       box_outside<T, N, V>(a, u0, u1, cell, cell1, tau, d, b.near_edge, b.near_dir, b.cs, !b.near_edge, o0, o1, st, en);
@@ -421,10 +439,7 @@ __device__ __forceinline__ void dg_box_body(const DGArgs<T> &a, const VecPtrs<T>
     en.u = vsign(su[b.gs + end], b.near_edge && b.near_dir);
     en.q = vsign(sq[b.gs + q], b.near_edge && b.near_dir);
     const int c = b.near_edge ? 0 : b.cs;
-    V tn;
-    if constexpr (P2) tn = F2{a.tau[cell + c], a.tau[cell1 + c]};
-    else tn = a.tau[cell + c];
-    en.t = vmul(vmax(tau, tn), L::all(a.hd[d]));
+    en.t = box_penalty(a, d, tau, box_tau<V>(a, d, cell + c, cell1 + c));
   };
   if (act) {
     box_fetch<N>(u0 + oz + bxa, stz, u1 + oz + bxb, stz, x);
@@ -456,7 +471,7 @@ __device__ __forceinline__ void dg_box_body(const DGArgs<T> &a, const VecPtrs<T>
       const bool e0 = cx == 0, e1 = !two || cx + 1 == a.m[0] - 1;
       const T *p0 = u0 + ox - (e0 ? 0 : N3), *p1 = u1 + ox + (e1 ? 0 : N3);
       box_fetch<N>(p0 + (e0 ? N - 1 : 0), e0 ? -1 : 1, p1 + (e1 ? 0 : N - 1), e1 ? 1 : -1, f);
-      ef.t = vmul(vmax(tau, F2{a.tau[cell - !e0], a.tau[cell1 + !e1]}), L::all(a.hd[0]));
+      ef.t = box_penalty(a, 0, tau, box_tau<V>(a, 0, cell - !e0, cell1 + !e1));
       ef.q = box_end<V, N>(f);
       const bool n0 = e0 && a.bc[0] == 0, n1 = e1 && a.bc[1] == 0, nn = !two && a.bc[1] == 0;
       ef.u = F2{n0 ? -f[N - 1].x : f[N - 1].x, n1 ? -f[N - 1].y : f[N - 1].y};

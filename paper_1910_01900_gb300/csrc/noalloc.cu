@@ -23,18 +23,18 @@ namespace {
 
 // Largest problem: what 64 MiB of gradients, traces and tables would hold
 // (about 1.4 million DoF at k = 3), the limit of this entry point.  The one
-// pass of axis-aligned cells needs the penalties alone, 8 of at least 584
-// bytes per cell by that count.
+// pass of axis-aligned cells needs the penalties alone: three values for the at
+// least 584 bytes per cell of that count.
 constexpr size_t kScratchBytes = size_t(64) << 20;
-static __device__ __align__(256) double g_noalloc_tau[kScratchBytes / 584 + 32];
+static __device__ __align__(256) double g_noalloc_tau[3 * (kScratchBytes / 584 + 32)];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 void *g_scratch_addr[kMaxDevices] = {};
 
 // The penalty tau_e (Section 2, same definition as the context path) of every
-// cell, written into the scratch.
-__global__ void noalloc_prep_kernel(double *tau, int n, double h0, double h1, double h2, int m0, int m1, int m2,
+// cell times h_d, written into the scratch.
+__global__ void noalloc_prep_kernel(double *tauh, int n, double h0, double h1, double h2, int m0, int m1, int m2,
                                     double factor) {
   const double h[3] = {h0, h1, h2};
   const int m[3] = {m0, m1, m2};
@@ -52,7 +52,8 @@ __global__ void noalloc_prep_kernel(double *tau, int n, double h0, double h1, do
         else a_int += area;
       }
     }
-    tau[e] = factor * (double)n * n * (0.5 * a_int + a_bd) / vol;
+    const double t = factor * (double)n * n * (0.5 * a_int + a_bd) / vol;
+    for (int d = 0; d < 3; ++d) tauh[d * ncells + e] = t * h[d];
   }
 }
 
@@ -161,7 +162,7 @@ extern "C" sipg_status sipg_operator_apply_noalloc(const sipg_mesh *mesh, int de
   DGArgs<double> a{};
   a.u = u_dev;
   a.out = v_dev;
-  a.tau = tau;
+  a.tauh = tau;
   for (int d = 0; d < 3; ++d) a.m[d] = mesh->m[d];
   dg_box_scales(a, h);
   a.box = dg_box_shape<double>(n, a.m, 0);

@@ -102,6 +102,7 @@ struct DGArgs {
   const T *fc[3];      // curved: [face][2 roles][3][n^2] = J^-1 n_outward (own side)
   const T *fwcart;     // Cartesian (setup's diagonal): [3][n^2] = w_q1 w_q2 h_t1 h_t2
   const T *tau;        // [cell] penalty tau_e
+  const T *tauh;       // Cartesian, FP64: [3][cell] tau_e h_d
   // Cartesian: 1/h_d, h_d, alpha_d / alpha_z of y and x, alpha_z (alpha_d =
   // prod(h) / h_d^2), and the cells a thread block takes
   T ih[3], hd[3], ralpha[2], alphaz;
@@ -186,6 +187,7 @@ struct Level {
   void *fdA[2][3] = {{nullptr}}, *fc[2][3] = {{nullptr}};
   void *fwcart[2] = {nullptr, nullptr};
   void *tau[2] = {nullptr, nullptr};
+  void *tauh = nullptr;   // axis-aligned, FP64: [3][cell] tau h_d
   int2 *ufn = nullptr;   // unstructured face neighbours (DGArgs::ufn)
   void *dinv[2] = {nullptr, nullptr};
   double lambda = 0;

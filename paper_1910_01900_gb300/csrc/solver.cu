@@ -226,6 +226,7 @@ DGArgs<T> dg_args(sipg_ctx *c, const Level &L) {
   dg_box_scales(a, L.h);
   a.fwcart = (const T *)L.fwcart[pi];
   a.tau = (const T *)L.tau[pi];
+  a.tauh = pi == 0 ? (const T *)L.tauh : nullptr;
   a.ufn = L.ufn;
   a.ncells = (int)L.ncells;
   for (int s = 0; s < 6; ++s) a.bc[s] = c->mesh.bc[s];
@@ -816,6 +817,13 @@ void build_level_geometry(sipg_ctx *c, Level &L, const MeshDesc &md, bool faces)
     upload2(c, fw, L.fwcart);
     penalty(map, L.n, c->prm.penalty_factor, tau);
     upload2(c, tau, L.tau);
+    if (!L.curved) {
+      std::vector<double> th;
+      for (int d = 0; d < 3; ++d)
+        for (double t : tau) th.push_back(t * map.h[d]);
+      L.tauh = dalloc<double>(c, (int64_t)th.size());
+      CK(cudaMemcpy(L.tauh, th.data(), th.size() * sizeof(double), cudaMemcpyHostToDevice));
+    }
   }
 }
 
