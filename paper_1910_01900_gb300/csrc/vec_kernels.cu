@@ -1,9 +1,9 @@
 // Vector kernels of the solver (Section 3: Algorithm 1 vector updates and
 // inner products, the coarse solve) and the arithmetic-peak probe.
 //
-// Inner products are deterministic: a fixed grid of blocks writes one partial
-// per block, and the last block to finish (detected with a counter that it
-// resets) sums the partials in block order.  Scalars stay in device memory;
+// Inner products are deterministic: a grid of blocks fixed by the length writes
+// one partial per block, and the last block to finish (detected with a counter
+// that it resets) sums the partials in a fixed order.  Scalars stay in device memory;
 // update kernels read them there, so the host only synchronizes to test
 // convergence.
 #include <cmath>
@@ -104,23 +104,45 @@ template cudaError_t launch_cast<float, float>(float *, const float *, int64_t, 
 template cudaError_t launch_axpy<double>(double *, double, const double *, int64_t, cudaStream_t);
 template cudaError_t launch_axpy<float>(float *, float, const float *, int64_t, cudaStream_t);
 
-// Block reduction of two values; the last block sums the partials in order.
-__device__ void reduce2_finish(double a, double b, double *partials, unsigned *counter, double *out) {
-  __shared__ double sa[kRedThreads], sb[kRedThreads];
-  __shared__ bool last;
-  sa[threadIdx.x] = a;
-  sb[threadIdx.x] = b;
-  __syncthreads();
-  for (int w = kRedThreads / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) {
-      sa[threadIdx.x] += sa[threadIdx.x + w];
-      sb[threadIdx.x] += sb[threadIdx.x + w];
+// (a, b) summed over the block's threads, on thread 0: lanes by shuffles, then
+// the warps' sums in the first warp
+__device__ __forceinline__ void block_sum2(double &a, double &b) {
+  __shared__ double sa[kRedThreads / 32], sb[kRedThreads / 32];
+  auto lanes = [&](const int from) {
+    for (int w = from; w > 0; w >>= 1) {
+      a += __shfl_down_sync(0xffffffffu, a, w);
+      b += __shfl_down_sync(0xffffffffu, b, w);
     }
-    __syncthreads();
+  };
+  lanes(16);
+  __syncthreads();   // the arrays are free again
+  if (threadIdx.x % 32 == 0) {
+    sa[threadIdx.x / 32] = a;
+    sb[threadIdx.x / 32] = b;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    a = threadIdx.x < kRedThreads / 32 ? sa[threadIdx.x] : 0.0;
+    b = threadIdx.x < kRedThreads / 32 ? sb[threadIdx.x] : 0.0;
+    lanes(kRedThreads / 64);
+  }
+}
+
+// Sums of two values over the grid: a partial per block, which the last block
+// to finish sums in a fixed order.
+__device__ void reduce2_finish(double a, double b, double *partials, unsigned *counter, double *out) {
+  __shared__ bool last;
+  block_sum2(a, b);
+  if (gridDim.x == 1) {
+    if (threadIdx.x == 0) {
+      out[0] = a;
+      out[1] = b;
+    }
+    return;
   }
   if (threadIdx.x == 0) {
-    partials[2 * blockIdx.x] = sa[0];
-    partials[2 * blockIdx.x + 1] = sb[0];
+    partials[2 * blockIdx.x] = a;
+    partials[2 * blockIdx.x + 1] = b;
     __threadfence();
     const unsigned done = atomicAdd(counter, 1u);
     last = (done == gridDim.x - 1);
@@ -128,26 +150,25 @@ __device__ void reduce2_finish(double a, double b, double *partials, unsigned *c
   __syncthreads();
   if (!last) return;
   __threadfence();
-  double pa = 0, pb = 0;
+  a = b = 0;
   for (int i = threadIdx.x; i < (int)gridDim.x; i += kRedThreads) {
-    pa += ((volatile double *)partials)[2 * i];
-    pb += ((volatile double *)partials)[2 * i + 1];
+    a += ((volatile double *)partials)[2 * i];
+    b += ((volatile double *)partials)[2 * i + 1];
   }
-  sa[threadIdx.x] = pa;
-  sb[threadIdx.x] = pb;
-  __syncthreads();
-  for (int w = kRedThreads / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) {
-      sa[threadIdx.x] += sa[threadIdx.x + w];
-      sb[threadIdx.x] += sb[threadIdx.x + w];
-    }
-    __syncthreads();
-  }
+  block_sum2(a, b);
   if (threadIdx.x == 0) {
-    out[0] = sa[0];
-    out[1] = sb[0];
+    out[0] = a;
+    out[1] = b;
     *counter = 0;
   }
+}
+
+// blocks of a reduction over n entries: 16 entries a thread, at most kRedBlocks
+// (the partials' array); a small vector's sum then ends in few blocks or one
+// (4096 entries: 304 blocks took 8 us, most of it the counter and the partials)
+static int red_blocks(int64_t n) {
+  const int64_t b = (n + 16 * kRedThreads - 1) / (16 * kRedThreads);
+  return (int)(b < 1 ? 1 : (b > kRedBlocks ? kRedBlocks : b));
 }
 
 __global__ void dot2_kernel(const double *x, const double *y, const double *z, const double *w, long n,
@@ -171,7 +192,7 @@ __global__ void dot2_kernel(const double *x, const double *y, const double *z, c
 
 cudaError_t launch_dot2(const double *x, const double *y, const double *z, const double *w, int64_t n,
                         double *partials, unsigned *counter, double *out, cudaStream_t s) {
-  dot2_kernel<<<kRedBlocks, kRedThreads, 0, s>>>(x, y, z, w, n, partials, counter, out);
+  dot2_kernel<<<red_blocks(n), kRedThreads, 0, s>>>(x, y, z, w, n, partials, counter, out);
   note_launch();
   return cudaGetLastError();
 }
@@ -202,7 +223,7 @@ __global__ void fcg_update_xr_kernel(double *x, double *r, const double *p, cons
 cudaError_t launch_fcg_update_xr(double *x, double *r, const double *p, const double *v, int64_t n,
                                  const double *sc, double *partials, unsigned *counter, double *out,
                                  cudaStream_t s) {
-  fcg_update_xr_kernel<<<kRedBlocks, kRedThreads, 0, s>>>(x, r, p, v, n, sc, partials, counter, out);
+  fcg_update_xr_kernel<<<red_blocks(n), kRedThreads, 0, s>>>(x, r, p, v, n, sc, partials, counter, out);
   note_launch();
   return cudaGetLastError();
 }
