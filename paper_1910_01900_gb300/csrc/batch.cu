@@ -399,6 +399,30 @@ cudaError_t batch_apply(BatchPlan<T> &P, cudaStream_t s) {
   return batch_dg_pass<T>(P, P.d_probs, true, nullptr, s);
 }
 
+// The axis-aligned pass of one degree's items.
+template <typename T>
+cudaError_t batch_dg_degree(const BatchPlan<T> &P, const typename BatchPlan<T>::Degree &d, const BatchProb<T> *probs,
+                            const Seg *segs, cudaStream_t s) {
+  const WorkItem *it = P.d_items + d.first;
+  switch (d.n) {
+#define SIPG_BATCH_CASE(NN)                                                                             \
+  case NN:                                                                                              \
+    dg_box_batched_kernel<T, NN><<<d.count, d.groups * NN * NN, d.smem, s>>>(probs, it, segs);          \
+    break;
+    SIPG_BATCH_CASE(2)
+    SIPG_BATCH_CASE(3)
+    SIPG_BATCH_CASE(4)
+    SIPG_BATCH_CASE(5)
+    SIPG_BATCH_CASE(6)
+    SIPG_BATCH_CASE(7)
+    SIPG_BATCH_CASE(8)
+    SIPG_BATCH_CASE(9)
+#undef SIPG_BATCH_CASE
+  }
+  note_launch();
+  return cudaGetLastError();
+}
+
 // One pass over the plan's work items with the descriptors probs (device).
 template <typename T>
 cudaError_t batch_dg_pass(const BatchPlan<T> &P, const BatchProb<T> *probs, bool integrate, const Seg *segs,
@@ -411,26 +435,10 @@ cudaError_t batch_dg_pass(const BatchPlan<T> &P, const BatchProb<T> *probs, bool
     note_launch();
     return cudaGetLastError();
   }
-  for (const auto &d : P.degrees) {
-    const WorkItem *it = P.d_items + d.first;
-    switch (d.n) {
-#define SIPG_BATCH_CASE(NN)                                                                             \
-  case NN:                                                                                              \
-    dg_box_batched_kernel<T, NN><<<d.count, d.groups * NN * NN, d.smem, s>>>(probs, it, segs);          \
-    break;
-      SIPG_BATCH_CASE(2)
-      SIPG_BATCH_CASE(3)
-      SIPG_BATCH_CASE(4)
-      SIPG_BATCH_CASE(5)
-      SIPG_BATCH_CASE(6)
-      SIPG_BATCH_CASE(7)
-      SIPG_BATCH_CASE(8)
-      SIPG_BATCH_CASE(9)
-#undef SIPG_BATCH_CASE
-    }
-    note_launch();
-  }
-  return cudaGetLastError();
+  cudaError_t e = cudaSuccess;
+  for (const auto &d : P.degrees)
+    if (e == cudaSuccess) e = batch_dg_degree<T>(P, d, probs, segs, s);
+  return e;
 }
 
 // ---------------------------------------------- batched vector steps of the V-cycle
@@ -480,6 +488,10 @@ template void batch_plan_free<double>(BatchPlan<double> &);
 template void batch_plan_free<float>(BatchPlan<float> &);
 template cudaError_t batch_apply<double>(BatchPlan<double> &, cudaStream_t);
 template cudaError_t batch_apply<float>(BatchPlan<float> &, cudaStream_t);
+template cudaError_t batch_dg_degree<double>(const BatchPlan<double> &, const BatchPlan<double>::Degree &,
+                                             const BatchProb<double> *, const Seg *, cudaStream_t);
+template cudaError_t batch_dg_degree<float>(const BatchPlan<float> &, const BatchPlan<float>::Degree &,
+                                            const BatchProb<float> *, const Seg *, cudaStream_t);
 template cudaError_t batch_dg_pass<double>(const BatchPlan<double> &, const BatchProb<double> *, bool, const Seg *,
                                            cudaStream_t);
 template cudaError_t batch_dg_pass<float>(const BatchPlan<float> &, const BatchProb<float> *, bool, const Seg *,

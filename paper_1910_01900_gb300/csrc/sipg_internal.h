@@ -471,6 +471,10 @@ template <typename T>
 void batch_plan_free(BatchPlan<T> &P);
 template <typename T>
 cudaError_t batch_apply(BatchPlan<T> &P, cudaStream_t s);
+// axis-aligned problems: the pass over one degree's items alone
+template <typename T>
+cudaError_t batch_dg_degree(const BatchPlan<T> &P, const typename BatchPlan<T>::Degree &d, const BatchProb<T> *probs,
+                            const Seg *segs, cudaStream_t s);
 // one pass of the batched DG operator with the descriptors probs (device)
 template <typename T>
 cudaError_t batch_dg_pass(const BatchPlan<T> &P, const BatchProb<T> *probs, bool integrate, const Seg *segs,

@@ -2854,6 +2854,41 @@ bool batch_cycle_applicable(const sipg_batch *B) {
   return true;
 }
 
+// Axis-aligned problems have one launch per degree and pass, which depend on
+// nothing of another degree: inside a stream capture on s they go into branches
+// side by side, on s and on the streams of the first problem of each degree,
+// through consecutive passes without a meeting in between.  One after another,
+// launches of 10 us on 50 to 250 blocks left most of the chip idle.
+struct DegreeBranches {
+  sipg_batch *B;
+  cudaStream_t s;
+  std::vector<char> skip;   // problems whose stream is in use otherwise
+  int home = 0;             // the degree that stays on s; 0: not forked
+  std::vector<int> used;    // problems whose streams are branches now
+  cudaStream_t of(int n) {
+    if (!home) {
+      CK(cudaEventRecord(B->ev_branch, s));
+      home = n;
+    }
+    if (n == home) return s;
+    int p = 0;
+    while ((p < (int)skip.size() && skip[p]) || B->ctx[p]->lv[B->ctx[p]->L].n != n) ++p;
+    if (std::find(used.begin(), used.end(), p) == used.end()) {
+      CK(cudaStreamWaitEvent(B->streams[p], B->ev_branch, 0));
+      used.push_back(p);
+    }
+    return B->streams[p];
+  }
+  void join() {
+    for (int p : used) {
+      CK(cudaEventRecord(B->ev_done[p], B->streams[p]));
+      CK(cudaStreamWaitEvent(s, B->ev_done[p], 0));
+    }
+    used.clear();
+    home = 0;
+  }
+};
+
 // Issue the batched cycle's launches on s (inside a stream capture): the
 // problems that fill the GPU alone run their own cycle on their own stream,
 // beside the shared launches of the others.
@@ -2869,7 +2904,10 @@ void batch_cycle_emit(sipg_batch *B, BatchCycle<T> &C, cudaStream_t s) {
     vcycle_body(B->ctx[p], B->ctx[p]->fr, B->ctx[p]->fz);   // on the problem's own stream
     CK(cudaEventRecord(B->ev_done[p], B->streams[p]));
   }
+  DegreeBranches br{B, s, std::vector<char>(C.solo.begin(), C.solo.end())};
   for (const BLaunch &r : C.prog) {
+    const bool by_degree = !C.curved && (r.kind == 3 || r.kind == 4);
+    if (!by_degree) br.join();
     switch (r.kind) {
       case 0:
         CK(launch_vec_batched(C.vec + r.off, C.items_d, C.n_d, segs, s));
@@ -2879,13 +2917,16 @@ void batch_cycle_emit(sipg_batch *B, BatchCycle<T> &C, cudaStream_t s) {
         break;
       case 2:
       case 3:
-        CK(batch_dg_pass<T>(C.dg, C.dgt + r.off, r.kind == 3, segs, s));
+        if (C.curved) CK(batch_dg_pass<T>(C.dg, C.dgt + r.off, r.kind == 3, segs, s));
+        else
+          for (const auto &d : C.dg.degrees) CK(batch_dg_degree<T>(C.dg, d, C.dgt + r.off, segs, br.of(d.n)));
         break;
       case 4:
         if (C.curved)
           CK(launch_fe_cells_batched<T>(C.fet + r.off, C.fe_items, C.n_fe_items, C.fe_smem, segs, s));
         for (const auto &d : C.fe_degrees)
-          CK(launch_fe_box_batched<T>(d.n, C.fet + r.off, C.fe_items + d.first, d.count, d.smem, segs, s));
+          CK(launch_fe_box_batched<T>(d.n, C.fet + r.off, C.fe_items + d.first, d.count, d.smem, segs,
+                                      br.of(d.n)));
         break;
       case 5:
         CK(launch_fe_nodes_batched<T>(C.fet + r.off, C.items_g, C.n_g, segs, 0, s));
@@ -2917,6 +2958,7 @@ void batch_cycle_emit(sipg_batch *B, BatchCycle<T> &C, cudaStream_t s) {
       }
     }
   }
+  br.join();
   for (int p = 0; p < C.np; ++p)
     if (C.solo[p]) CK(cudaStreamWaitEvent(s, B->ev_done[p], 0));
 }
@@ -3183,8 +3225,15 @@ void batch_build_fcg_chunk(sipg_batch *B) {
     }
     for (int i = 0; i < kFcgChunk; ++i) {
       body(add_if_node(s, hA[i]), &B->fcg_kA[i], [&]() {
-        if (B->plan.curved) CK(batch_dg_pass<double>(B->plan, B->d_app, false, B->d_segs, s2));
-        CK(batch_dg_pass<double>(B->plan, B->d_app, true, B->d_segs, s2));
+        if (B->plan.curved) {
+          CK(batch_dg_pass<double>(B->plan, B->d_app, false, B->d_segs, s2));
+          CK(batch_dg_pass<double>(B->plan, B->d_app, true, B->d_segs, s2));
+        } else {
+          DegreeBranches br{B, s2, {}};
+          for (const auto &d : B->plan.degrees)
+            CK(batch_dg_degree<double>(B->plan, d, B->d_app, B->d_segs, br.of(d.n)));
+          br.join();
+        }
         CK(seg_dot(B->d_segs, B->sg, 2, B->partials, B->counters, B->sc, st, 2, s2));
         CK(seg_update_xr(B->d_segs, B->sg, B->partials, B->counters, B->sc, st, s2));
         CK(launch_batch_fcg_check(B->sc, st, B->d_segs, np, B->d_it, B->d_status, B->d_hist, B->d_rn, B->d_r0,
