@@ -115,8 +115,9 @@ typedef struct {
                               (the dense coarse solve works on FE_1)       */
   int autotune;            /* 1: at setup, time a few tile shapes (cells per
                               thread block) of every cell kernel of every
-                              level (both DG passes, the FE cell pass) in
-                              both precisions and keep the fastest; the
+                              level (the DG passes, the curved FE cell
+                              pass) in both precisions and keep the
+                              fastest; the
                               candidates are the widths whose last wave of
                               blocks leaves the fewest cell slots idle;
                               cached per (degree, geometry, cells) for the
@@ -430,10 +431,11 @@ sipg_status sipg_mlp_features(sipg_ctx *ctx, const double *r_dev, float *feat_de
 
 /* Cells per thread block a cell kernel of a level uses in the given
  * precision (pass 0 DG evaluation, 1 DG integration on a DG level; 2 the FE
- * cell pass on an FE level): the autotuned or set value, else the default
- * (about 256 threads per block, fewer cells per block on meshes that would
- * otherwise give fewer blocks than the GPU has SMs).  EINVAL for a pass that
- * does not exist on the level. */
+ * cell pass on an FE level; on axis-aligned cells pass 1 is the whole DG
+ * operator, pass 0 is unused, and the FE pass takes its bricks from the mesh):
+ * the autotuned or set value, else the default (about 256 threads per block,
+ * fewer cells per block on meshes that would otherwise give fewer blocks than
+ * the GPU has SMs).  EINVAL for a pass that does not exist on the level. */
 sipg_status sipg_tile_shape(const sipg_ctx *ctx, int level, int precision, int pass, int *cells_per_block);
 
 /* Sets that width (0 = the default above; at most 768 threads and 227 KB
