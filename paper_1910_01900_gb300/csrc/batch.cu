@@ -3,7 +3,7 @@
 //
 // * The finest-level DG operator of all problems runs as one launch per degree
 //   (axis-aligned cells: a block per item of a static list of problems' blocks,
-//   dg_box.cuh) or, on curved cells, as one persistent launch per pass: a fixed
+//   dg_box.cuh; in the captured graphs the degrees' launches are side by side) or, on curved cells, as one persistent launch per pass: a fixed
 //   grid (SMs x resident blocks) walks a static list of work items (problem,
 //   first cell, cell count), longest first, and dispatches each item to the
 //   sum-factorisation body of that problem's degree.  The same bodies as the

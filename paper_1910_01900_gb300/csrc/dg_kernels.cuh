@@ -64,12 +64,11 @@ template <typename T, int N>
 __device__ __forceinline__ void line_ends(const T (&x)[N], T &v0, T &v1, T &g0, T &g1) {
   constexpr int H = N / 2;
   const Tables<T> &t = tab<T>();
-  if constexpr (N == 2) {   // two points: the plain products are fewer (Tables: le, lo = l_0, de, dod = D^T l_0)
-    const T l0 = t.le[2][0], l1 = t.lo[2][0], d0 = t.de[2][0], d1 = t.dod[2][0];
+  if constexpr (N == 2) {   // two points: plain values, one derivative (Tables: le, lo = l_0)
+    const T l0 = t.le[2][0], l1 = t.lo[2][0];
     v0 = fma(l1, x[1], l0 * x[0]);
     v1 = fma(l0, x[1], l1 * x[0]);
-    g0 = fma(d1, x[1], d0 * x[0]);
-    g1 = -fma(d0, x[1], d1 * x[0]);
+    g0 = g1 = t.D[2][1] * (x[1] - x[0]);
     return;
   }
   T ve = T(0), vo = T(0), ge = T(0), go = T(0);
@@ -99,11 +98,10 @@ __device__ __forceinline__ void sweep_with_ends(const T (&x)[N], const T a0, con
                                                 T (&y)[N]) {
   constexpr int H = N / 2, HC = (N + 1) / 2;
   const Tables<T> &t = tab<T>();
-  if constexpr (N == 2) {
-    const T l0 = t.le[2][0], l1 = t.lo[2][0], d0 = t.de[2][0], d1 = t.dod[2][0];
-    apply_mat<T, N, MDt>(x, y);
-    y[0] = fma(l0, a0, fma(l1, a1, fma(d0, b0, fma(-d1, b1, y[0]))));
-    y[1] = fma(l1, a0, fma(l0, a1, fma(d1, b0, fma(-d0, b1, y[1]))));
+  if constexpr (N == 2) {   // D^T l_0 = D^T l_1 = the rows of D
+    const T l0 = t.le[2][0], l1 = t.lo[2][0], m = t.D[2][1] * ((x[0] + x[1]) + (b0 + b1));
+    y[0] = fma(l0, a0, fma(l1, a1, -m));
+    y[1] = fma(l1, a0, fma(l0, a1, m));
     return;
   }
   const T ap = a0 + a1, am = a0 - a1, bm = b0 - b1, bp = b0 + b1;

@@ -267,11 +267,9 @@ void build_tables(Tables<T> &t) {
     std::vector<double> d0(n, 0.0);   // (D^T l0)[q] = sum_j D[j][q] l0[j]
     for (int q = 0; q < n; ++q)
       for (int j = 0; j < n; ++j) d0[q] += r.D[j * n + q] * r.l0[j];
-    if (n == 2) {   // two points: the vectors themselves
+    if (n == 2) {   // two points: the entries of l0 themselves
       t.le[2][0] = (T)r.l0[0];
       t.lo[2][0] = (T)r.l0[1];
-      t.de[2][0] = (T)d0[0];
-      t.dod[2][0] = (T)d0[1];
     }
     for (int j = 0; n > 2 && j < (n + 1) / 2; ++j) {
       const int k = n - 1 - j;

@@ -58,7 +58,7 @@ struct Tables {
   // the extrapolation l0 to the lower end (l1 is its mirror image) and D^T l0
   // (D^T l1 minus its mirror image) in even and odd parts: le[j] + lo[j] = l0[j],
   // le[j] - lo[j] = l0[n-1-j], de + dod = D^T l0 likewise; the middle entry of
-  // an odd n in le and de (n = 2: the two entries of l0 and of D^T l0)
+  // an odd n in le and de (n = 2: le and lo hold the two entries of l0)
   T le[kMaxN + 1][5], lo[kMaxN + 1][4], de[kMaxN + 1][5], dod[kMaxN + 1][4];
   // 1D mass and stiffness matrices of the GL basis under the Gauss rule,
   // M1[i][j] = sum_q w_q l_i(x_q) l_j(x_q), K1[i][j] = sum_q w_q l_i'(x_q) l_j'(x_q)
