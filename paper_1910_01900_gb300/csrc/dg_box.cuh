@@ -32,6 +32,18 @@
 // product of the same values, so a block may also take single cells (small
 // meshes) with the same result.
 //
+// Up to three points per line M^-1 stays out of it (kBoxDirect): with
+//   v = M_z (M_y a + M_x b) + M_y M_x c,   (a, b, c) = (G_x, G_y, G_z) u,
+// five mass sweeps instead of three and two more tiles.  M^-1 amplifies the
+// parts of a line that M then damps again, by 6 : 2 at two points, and the
+// rounding of w between them with it: FP32 error against 64 bits for random
+// vectors (relative, 2-norm) at degree 1 / 2 1.2e-7 / 1.9e-7 that way and
+// 7.6e-8 / 1.5e-7 this way, where the evaluation at the Gauss points gives
+// 9.7e-8 / 1.54e-7 (time at 12 MDoF 69 / 75 us and 78 / 83 us; at the Gauss
+// points 245 / 185 us).  From four points on the sums of a line's products round more than
+// that, and w is the more accurate form (degree 3 / 5 / 7 1.5e-7 / 1.7e-7 /
+// 1.6e-7, at the Gauss points 1.8e-7 / 2.5e-7 / 2.6e-7).
+//
 // Measured at 16 MDoF (GB300) against the two-pass scheme with stored traces
 // that axis-aligned cells had before: FP32 k = 3 / 5 / 7 204 / 191 / 165 us ->
 // 69 / 71 / 75 us, FP64 k = 3 / 5 / 7 2440 / 2590 / 2860 us -> 1389 / 1495 /
@@ -177,8 +189,8 @@ static void upload_box_tu(const BoxTables<T> &t) {
 }
 
 // Shared memory of one cell (FP32: cell pair), in 8-byte values: the tiles of
-// u and w (x fastest, y step XP, z step ZP) and the near-end derivatives of
-// two phases.  Pitches chosen per N by counting the wavefronts of the three
+// u and w (N <= 3: and two more; x fastest, y step XP, z step ZP) and the
+// near-end derivatives of two phases.  Pitches chosen per N by counting the wavefronts of the three
 // line directions (weighted by their 3, 5 and 3 accesses) over 8 cells: 1.27
 // per half-warp at N = 4 (3.18 unpadded), 1.63 at N = 5, 1.64 at N = 6 (1.79),
 // 1.57 at N = 7 (1.90), 1.27 at N = 8 (3.36), 1.50 at N = 9.
@@ -187,8 +199,11 @@ __host__ __device__ constexpr int box_zp(int n) {
   return n == 2 ? 6 : n == 3 ? 9 : n == 4 ? 20 : n == 5 ? 25 : n == 6 ? 38 : n == 7 ? 55 : n == 8 ? 72 : 81;
 }
 __host__ __device__ constexpr int box_group_values(int n) {
-  return n == 2 ? 36 : n == 3 ? 75 : n == 4 ? 192 : n == 5 ? 301 : n == 6 ? 532 : n == 7 ? 881 : n == 8 ? 1280 : 1633;
+  return n == 2 ? 68 : n == 3 ? 139 : n == 4 ? 192 : n == 5 ? 301 : n == 6 ? 532 : n == 7 ? 881 : n == 8 ? 1280 : 1633;
 }
+// the form without M^-1 (see above; also in the tables, BoxTables)
+template <int N>
+constexpr bool kBoxDirect = box_direct(N);
 // cells that one thread works on
 template <typename T>
 constexpr int kBoxLanes = sizeof(T) == 4 ? 2 : 1;
@@ -210,7 +225,7 @@ __host__ __device__ inline int box_groups(const BoxShape &b) {
 template <int N>
 struct BoxTile {
   static constexpr int XP = box_xp(N), ZP = box_zp(N), T3 = ZP * N, N2 = N * N;
-  static constexpr int Q = 2 * T3;
+  static constexpr int Q = (kBoxDirect<N> ? 4 : 2) * T3;
   static constexpr int GS = box_group_values(N);
   static_assert(XP >= N && ZP >= XP * N && GS >= Q + 2 * N2, "box layout overlaps");
 };
@@ -441,6 +456,13 @@ __device__ __forceinline__ void dg_box_body(const DGArgs<T> &a, const VecPtrs<T>
     const int c = b.near_edge ? 0 : b.cs;
     en.t = box_penalty(a, d, tau, box_tau<V>(a, d, cell + c, cell1 + c));
   };
+  // M along the thread's line of a tile, in place
+  auto mass_along = [&](V *t, const int base, const int step) {
+    V in[N], out[N];
+    box_load<V, N>(t, base, step, in);
+    box_mass<V, N>(in, out);
+    box_store<V, N>(t, base, step, out);
+  };
   if (act) {
     box_fetch<N>(u0 + oz + bxa, stz, u1 + oz + bxb, stz, x);
     box_store<V, N>(su, box_base<N, 2>(l), box_step<N, 2>(), x);
@@ -448,7 +470,7 @@ __device__ __forceinline__ void dg_box_body(const DGArgs<T> &a, const VecPtrs<T>
     outer(2, dz, oz + bxa, oz + bxb, stz);
   }
   __syncthreads();
-  if (act) {   // w = M_z^-1 G_z u / alpha_z
+  if (act) {   // w = M_z^-1 G_z u / alpha_z (N <= 3: G_z u / alpha_z, and so on)
     inner(2, dz, box_base<N, 2>(l) + (N - 1) * box_step<N, 2>(), 0);
     box_flux<V, N>(x, ef, en, y);
     box_store<V, N>(sw, box_base<N, 2>(l), box_step<N, 2>(), y);
@@ -462,8 +484,14 @@ __device__ __forceinline__ void dg_box_body(const DGArgs<T> &a, const VecPtrs<T>
     box_flux<V, N>(x, ef, en, y);
     const V c = L::all(a.ralpha[0]);
     V *p = sw + box_base<N, 1>(l);
+    if constexpr (kBoxDirect<N>) {   // b, and M_y c
 #pragma unroll
-    for (int q = 0; q < N; ++q) p[q * box_step<N, 1>()] = vfma(c, y[q], p[q * box_step<N, 1>()]);
+      for (int q = 0; q < N; ++q) p[T3 + q * box_step<N, 1>()] = vmul(c, y[q]);
+      mass_along(sw, box_base<N, 1>(l), box_step<N, 1>());
+    } else {
+#pragma unroll
+      for (int q = 0; q < N; ++q) p[q * box_step<N, 1>()] = vfma(c, y[q], p[q * box_step<N, 1>()]);
+    }
     box_load<V, N>(su, box_base<N, 0>(l), box_step<N, 0>(), x);
     if constexpr (P2) {
       // the far ends lie on both sides of the pair, the near ends are each other's
@@ -490,22 +518,41 @@ __device__ __forceinline__ void dg_box_body(const DGArgs<T> &a, const VecPtrs<T>
     if constexpr (!P2) inner(0, dx, box_base<N, 0>(l) + N - 1, 0);
     box_flux<V, N>(x, ef, en, y);
     const V c = L::all(a.ralpha[1]);
-    box_load<V, N>(sw, box_base<N, 0>(l), box_step<N, 0>(), x);
+    if constexpr (kBoxDirect<N>) {   // a, M_x b and M_x M_y c
 #pragma unroll
-    for (int q = 0; q < N; ++q) x[q] = vfma(c, y[q], x[q]);
-    box_mass<V, N>(x, y);
-    box_store<V, N>(sw, box_base<N, 0>(l), box_step<N, 0>(), y);
+      for (int q = 0; q < N; ++q) y[q] = vmul(c, y[q]);
+      box_store<V, N>(sw + 2 * T3, box_base<N, 0>(l), box_step<N, 0>(), y);
+      mass_along(sw + T3, box_base<N, 0>(l), box_step<N, 0>());
+      mass_along(sw, box_base<N, 0>(l), box_step<N, 0>());
+    } else {
+      box_load<V, N>(sw, box_base<N, 0>(l), box_step<N, 0>(), x);
+#pragma unroll
+      for (int q = 0; q < N; ++q) x[q] = vfma(c, y[q], x[q]);
+      box_mass<V, N>(x, y);
+      box_store<V, N>(sw, box_base<N, 0>(l), box_step<N, 0>(), y);
+    }
   }
   __syncthreads();
   if (act) {
-    box_load<V, N>(sw, box_base<N, 1>(l), box_step<N, 1>(), x);
-    box_mass<V, N>(x, y);
-    box_store<V, N>(sw, box_base<N, 1>(l), box_step<N, 1>(), y);
+    if constexpr (kBoxDirect<N>) {   // M_y a + M_x b
+      box_load<V, N>(sw + 2 * T3, box_base<N, 1>(l), box_step<N, 1>(), x);
+      box_mass<V, N>(x, y);
+      V *p = sw + T3 + box_base<N, 1>(l);
+#pragma unroll
+      for (int q = 0; q < N; ++q) p[q * box_step<N, 1>()] = vadd(y[q], p[q * box_step<N, 1>()]);
+    } else {
+      mass_along(sw, box_base<N, 1>(l), box_step<N, 1>());
+    }
   }
   __syncthreads();
   if (!act) return;
-  box_load<V, N>(sw, box_base<N, 2>(l), box_step<N, 2>(), x);
+  box_load<V, N>(kBoxDirect<N> ? sw + T3 : sw, box_base<N, 2>(l), box_step<N, 2>(), x);
   box_mass<V, N>(x, y);
+  if constexpr (kBoxDirect<N>) {
+    box_load<V, N>(sw, box_base<N, 2>(l), box_step<N, 2>(), x);
+#pragma unroll
+    for (int q = 0; q < N; ++q) y[q] = vadd(y[q], x[q]);
+  }
   // the epilogue, cell by cell
 #pragma unroll
   for (int k = 0; k < (P2 ? 2 : 1); ++k) {

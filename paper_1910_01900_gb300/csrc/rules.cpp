@@ -141,8 +141,8 @@ void set(double &to, long double v) { to = (double)v; }
 void set(F2 &to, long double v) { to.x = to.y = (float)v; }
 
 // The line operator of axis-aligned cells: M1^-1 applied (in long double, by
-// elimination; M1 is positive definite) to K1 with the own parts of the
-// fluxes and to the end columns; see BoxTables.
+// elimination; M1 is positive definite; up to three points left out) to K1
+// with the own parts of the fluxes and to the end columns; see BoxTables.
 template <typename T>
 void box_tables(const Rules1D &r, const std::vector<double> &M1, const std::vector<double> &K1,
                 BoxTables<T> &t) {
@@ -165,6 +165,9 @@ void box_tables(const Rules1D &r, const std::vector<double> &M1, const std::vect
     B[i * w + n] = i == 0 ? 1.0L : 0.0L;
     B[i * w + n + 1] = 0.5L * q0[i];
   }
+  if (box_direct(n))   // without M1^-1
+    for (int i = 0; i < n; ++i)
+      for (int j = 0; j < n; ++j) A[i * n + j] = i == j;
   for (int k = 0; k < n; ++k)
     for (int i = 0; i < n; ++i) {
       if (i == k) continue;

@@ -74,6 +74,8 @@ void build_tables(Tables<T> &t);
 // e_s, q_s/2], rows of hc + 2 (stride 7) and h + 2 (stride 6): the matrix, then
 // the end columns; ME, MO even-odd blocks of M1 (strides 5, 4); qh = q1/2.
 // e_s: an end's unit vector, q_s: the outward end derivative of the GL basis.
+// Where box_direct(n), HE and HO come without M1^-1.
+__host__ __device__ constexpr bool box_direct(int n) { return n <= 3; }
 template <typename T>
 struct BoxTables {
   using V = typename BoxNum<T>::type;
