@@ -40,9 +40,9 @@
 // vectors (relative, 2-norm) at degree 1 / 2 1.2e-7 / 1.9e-7 that way and
 // 7.6e-8 / 1.5e-7 this way, where the evaluation at the Gauss points gives
 // 9.7e-8 / 1.54e-7 (time at 12 MDoF 69 / 75 us and 78 / 83 us; at the Gauss
-// points 245 / 185 us).  From four points on the sums of a line's products round more than
-// that, and w is the more accurate form (degree 3 / 5 / 7 1.5e-7 / 1.7e-7 /
-// 1.6e-7, at the Gauss points 1.8e-7 / 2.5e-7 / 2.6e-7).
+// points 245 / 185 us).  From four points on the form with w rounds less than
+// the Gauss points do (degree 3 / 5 / 7 1.5e-7 / 1.7e-7 / 1.6e-7, there 1.8e-7 /
+// 2.5e-7 / 2.6e-7) and is kept.
 //
 // Measured at 16 MDoF (GB300) against the two-pass scheme with stored traces
 // that axis-aligned cells had before: FP32 k = 3 / 5 / 7 204 / 191 / 165 us ->
