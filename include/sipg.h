@@ -316,9 +316,9 @@ sipg_status sipg_time_apply(sipg_ctx *ctx, int precision, const void *u_dev, voi
  * for many right-hand sides.  meshes[i], params[i] describe problem i (all
  * affine or all curved; one precision for all; each needs a Dirichlet side);
  * params[0].stream is the stream of the batched work.  The finest-level
- * operators of all problems run as one launch per degree (affine meshes; a
- * block per (problem, cell block) item) or one persistent launch per pass
- * (curved ones; a fixed grid walking a work list, longest first);
+ * operators of all problems run as one launch per degree and pass (one pass
+ * on affine meshes, two on curved ones; a block per (problem, cells) item),
+ * the degrees side by side;
  * the flexible-CG iterations run in lockstep with batched inner products and
  * updates (blocks per problem in proportion to its size).  On a non-default
  * stream, when every problem's hierarchy starts with a DG level above a

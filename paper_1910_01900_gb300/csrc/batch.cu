@@ -2,12 +2,10 @@
 // right-hand sides of one problem, solved together.
 //
 // * The finest-level DG operator of all problems runs as one launch per degree
-//   (axis-aligned cells: a block per item of a static list of problems' blocks,
-//   dg_box.cuh; in the captured graphs the degrees' launches are side by side) or, on curved cells, as one persistent launch per pass: a fixed
-//   grid (SMs x resident blocks) walks a static list of work items (problem,
-//   first cell, cell count), longest first, and dispatches each item to the
-//   sum-factorisation body of that problem's degree.  The same bodies as the
-//   per-problem kernels (dg_kernels.cuh).
+//   and pass, a block per item of a static list (axis-aligned cells: one pass
+//   over the problems' blocks, dg_box.cuh; curved cells: two passes over groups
+//   of cells, dg_kernels.cuh); in the captured graphs the degrees' launches are
+//   side by side.  The same bodies as the per-problem kernels.
 // * The flexible-CG iterations of all problems run in lockstep: batched
 //   operator applications, batched inner products and updates (one launch for
 //   all problems, deterministic per-problem reductions), and each problem's
@@ -41,41 +39,24 @@ void upload_tables_batch<float>(const Tables<float> &t, const BoxTables<float> &
 }
 
 // segs (optional): the flexible-CG systems; a problem whose system has left
-// the iteration (segs[p].active == 0, set on the device) is skipped too
-// (register budget as the single-problem passes: 64 and 128)
-template <typename T, bool INTEGRATE>
-__global__ void __launch_bounds__(kBatchThreads, sizeof(T) == 4 ? 4 : 2)
-    dg_batched_kernel(const BatchProb<T> *__restrict__ probs, const WorkItem *__restrict__ items, int nitems,
+// the iteration (segs[p].active == 0, set on the device) is skipped too.
+// One kernel per degree, with the register budget of the single-problem
+// passes: with every degree's body in one kernel the compiler kept 600 (FP32)
+// and 904 bytes (FP64) of the integration pass in local memory.
+// One V-cycle of 12 curved problems of 8^3 cells of degree 4 in FP32, FP32 cycle
+// of two of 16^3 and 12^3 of degrees 3 and 5: 1006 and 635 us so, now 857 and 551
+// us; operator of 16 problems in FP64 2665 us, now 2542 us.
+template <typename T, int N, bool INTEGRATE>
+__global__ void __launch_bounds__(kBatchThreads, kCurvedThreads / kBatchThreads * kCurvedBlocks<T, N, INTEGRATE>)
+    dg_batched_kernel(const BatchProb<T> *__restrict__ probs, const WorkItem *__restrict__ items,
                       const Seg *__restrict__ segs) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *sm = reinterpret_cast<T *>(smem_raw);
-  for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
-    const WorkItem w = items[it];
-    const BatchProb<T> &P = probs[w.p];
-    if (P.active && (!segs || segs[w.p].active)) {
-#define SIPG_BATCH_CASE(NN)                                                 \
-  case NN:                                                                  \
-    if (INTEGRATE)                                                          \
-      dg_integrate_body<T, NN>(P.a, vec_ptrs(P.a, 0), w.cell0, w.ncta, sm); \
-    else                                                                    \
-      dg_eval_body<T, NN>(P.a, vec_ptrs(P.a, 0), w.cell0, w.ncta, sm);      \
-    break;
-      switch (P.n) {
-        SIPG_BATCH_CASE(2)
-        SIPG_BATCH_CASE(3)
-        SIPG_BATCH_CASE(4)
-        SIPG_BATCH_CASE(5)
-        SIPG_BATCH_CASE(6)
-        SIPG_BATCH_CASE(7)
-        SIPG_BATCH_CASE(8)
-        SIPG_BATCH_CASE(9)
-        default:
-          break;
-      }
-#undef SIPG_BATCH_CASE
-    }
-    __syncthreads();
-  }
+  const WorkItem w = items[blockIdx.x];
+  const BatchProb<T> &P = probs[w.p];
+  if (!P.active || (segs && !segs[w.p].active)) return;
+  if constexpr (INTEGRATE) dg_integrate_body<T, N>(P.a, vec_ptrs(P.a, 0), w.cell0, w.ncta, sm);
+  else dg_eval_body<T, N>(P.a, vec_ptrs(P.a, 0), w.cell0, w.ncta, sm);
 }
 
 // Axis-aligned problems: the one pass of all problems of one degree, a block
@@ -102,13 +83,23 @@ __global__ void __launch_bounds__(kBatchThreads) dg_box_batched_kernel(const Bat
 }
 static int pack_shape(const BoxShape &b) { return (b.w[0] - 1) | (b.w[1] - 1) << 1 | (b.w[2] - 1) << 2 | b.bricks << 3; }
 
+// shared memory of a block of kBatchThreads / n^2 curved cells
 template <typename T>
-static cudaError_t prep_box_batched() {
+static size_t curved_batch_smem(int n, bool integrate) {
+  return (size_t)(kBatchThreads / (n * n)) * curved_cell_values(n, integrate) * sizeof(T);
+}
+template <typename T>
+static cudaError_t prep_batched() {
+  constexpr cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
   cudaError_t e = cudaSuccess;
 #define SIPG_BATCH_PREP(NN)                                                                                     \
-  if (e == cudaSuccess)                                                                                         \
-    e = cudaFuncSetAttribute(dg_box_batched_kernel<T, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize,         \
-                             kBatchThreads / (NN * NN) * box_group_values(NN) * 8);
+  for (cudaError_t r : {cudaFuncSetAttribute(dg_box_batched_kernel<T, NN>, at,                                  \
+                                             kBatchThreads / (NN * NN) * box_group_values(NN) * 8),             \
+                        cudaFuncSetAttribute(dg_batched_kernel<T, NN, false>, at,                               \
+                                             (int)curved_batch_smem<T>(NN, false)),                             \
+                        cudaFuncSetAttribute(dg_batched_kernel<T, NN, true>, at,                                \
+                                             (int)curved_batch_smem<T>(NN, true))})                             \
+    if (r != cudaSuccess) e = r;
   SIPG_BATCH_PREP(2)
   SIPG_BATCH_PREP(3)
   SIPG_BATCH_PREP(4)
@@ -322,57 +313,39 @@ cudaError_t batch_plan_build(BatchPlan<T> &P, const std::vector<DGArgs<T>> &args
     P.probs[p].n = ns[p];
     P.probs[p].active = 1;
   }
-  size_t smem = 0;
-  if (curved) {
+  for (int n = kMaxN; n >= 2; --n) {   // the degrees' items one after another
+    typename BatchPlan<T>::Degree d{n, (int)P.items.size(), 0, 0, {0, 0}};
     for (int p = 0; p < np; ++p) {
-      const int n = ns[p], cb = kBatchThreads / (n * n);
-      smem = std::max(smem, (size_t)cb * curved_cell_values(n, true) * sizeof(T));
-      for (int c = 0; c < args[p].ncells; c += cb) P.items.push_back({p, c, std::min(cb, args[p].ncells - c)});
-    }
-    // longest items first (cost ~ cells x n^4), then static striding over the grid
-    std::stable_sort(P.items.begin(), P.items.end(), [&](const WorkItem &x, const WorkItem &y) {
-      const double cx = (double)x.ncta * std::pow((double)ns[x.p], 4), cy = (double)y.ncta * std::pow((double)ns[y.p], 4);
-      return cx > cy;
-    });
-  } else {
-    for (int n = kMaxN; n >= 2; --n) {   // the degrees' items one after another
-      typename BatchPlan<T>::Degree d{n, (int)P.items.size(), 0, 0, 0};
-      for (int p = 0; p < np; ++p) {
-        if (ns[p] != n || args[p].ncells == 0) continue;
-        // a default block, as far as kBatchThreads allow
-        const int cb = std::min(dg_cells_per_block<T>(n, false), kBatchThreads / (n * n) * kBoxLanes<T>);
-        const BoxShape w = dg_box_shape<T>(n, args[p].m, cb);
-        int nb = 1;
-        for (int e = 0; e < 3; ++e) {
-          const int we = w.w[e] * (e == 0 ? w.bricks : 1);
-          nb *= (args[p].m[e] + we - 1) / we;
-        }
-        d.groups = std::max(d.groups, box_groups<T>(w));
-        for (int b = 0; b < nb; ++b) P.items.push_back({p, b, pack_shape(w)});
+      if (ns[p] != n || args[p].ncells == 0) continue;
+      if (curved) {
+        d.groups = kBatchThreads / (n * n);
+        for (int c = 0; c < args[p].ncells; c += d.groups)
+          P.items.push_back({p, c, std::min(d.groups, args[p].ncells - c)});
+        continue;
       }
-      d.count = (int)P.items.size() - d.first;
-      d.smem = (size_t)d.groups * box_group_values(n) * 8;
-      if (d.count) P.degrees.push_back(d);
+      // a default block, as far as kBatchThreads allow
+      const int cb = std::min(dg_cells_per_block<T>(n, false), kBatchThreads / (n * n) * kBoxLanes<T>);
+      const BoxShape w = dg_box_shape<T>(n, args[p].m, cb);
+      int nb = 1;
+      for (int e = 0; e < 3; ++e) {
+        const int we = w.w[e] * (e == 0 ? w.bricks : 1);
+        nb *= (args[p].m[e] + we - 1) / we;
+      }
+      d.groups = std::max(d.groups, box_groups<T>(w));
+      for (int b = 0; b < nb; ++b) P.items.push_back({p, b, pack_shape(w)});
     }
+    d.count = (int)P.items.size() - d.first;
+    for (int pass = 0; pass < 2; ++pass)
+      d.smem[pass] = curved ? curved_batch_smem<T>(n, pass == 1) : (size_t)d.groups * box_group_values(n) * 8;
+    if (d.count) P.degrees.push_back(d);
   }
-  P.smem = smem;
   cudaError_t e;
   if ((e = cudaMalloc(&P.d_probs, np * sizeof(BatchProb<T>))) != cudaSuccess) return e;
   if ((e = cudaMalloc(&P.d_items, std::max<size_t>(1, P.items.size()) * sizeof(WorkItem))) != cudaSuccess) return e;
   if ((e = cudaMemcpy(P.d_items, P.items.data(), P.items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice)) !=
       cudaSuccess)
     return e;
-  if (!curved) return prep_box_batched<T>();
-  auto k2 = dg_batched_kernel<T, false>, k3 = dg_batched_kernel<T, true>;
-  for (auto k : {k2, k3})
-    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-      return e;
-  int dev, nsm, occ = 1;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k3, kBatchThreads, smem);
-  P.grid = std::max(1, std::min<int>((int)P.items.size(), nsm * std::max(1, occ)));
-  return cudaSuccess;
+  return prep_batched<T>();
 }
 
 template <typename T>
@@ -383,31 +356,21 @@ void batch_plan_free(BatchPlan<T> &P) {
   P.d_items = nullptr;
 }
 
-// Upload the current descriptors (pointers, modes, active flags) and run the
-// pass or passes.
-template <typename T>
-cudaError_t batch_dg_pass(const BatchPlan<T> &P, const BatchProb<T> *probs, bool integrate, const Seg *segs,
-                          cudaStream_t s);
-
-template <typename T>
-cudaError_t batch_apply(BatchPlan<T> &P, cudaStream_t s) {
-  cudaError_t e = cudaMemcpyAsync(P.d_probs, P.probs.data(), P.probs.size() * sizeof(BatchProb<T>),
-                                  cudaMemcpyHostToDevice, s);
-  if (e != cudaSuccess) return e;
-  if (P.items.empty()) return cudaSuccess;
-  if (P.curved && (e = batch_dg_pass<T>(P, P.d_probs, false, nullptr, s)) != cudaSuccess) return e;
-  return batch_dg_pass<T>(P, P.d_probs, true, nullptr, s);
-}
-
-// The axis-aligned pass of one degree's items.
+// One degree's items with the descriptors probs (device): the evaluation (pass
+// 0) or the integration pass of curved cells, or the one pass of axis-aligned
+// cells (1).
 template <typename T>
 cudaError_t batch_dg_degree(const BatchPlan<T> &P, const typename BatchPlan<T>::Degree &d, const BatchProb<T> *probs,
-                            const Seg *segs, cudaStream_t s) {
+                            int pass, const Seg *segs, cudaStream_t s) {
   const WorkItem *it = P.d_items + d.first;
+  const int threads = d.groups * d.n * d.n;
   switch (d.n) {
-#define SIPG_BATCH_CASE(NN)                                                                             \
-  case NN:                                                                                              \
-    dg_box_batched_kernel<T, NN><<<d.count, d.groups * NN * NN, d.smem, s>>>(probs, it, segs);          \
+#define SIPG_BATCH_CASE(NN)                                                                            \
+  case NN:                                                                                             \
+    if (!P.curved) dg_box_batched_kernel<T, NN><<<d.count, threads, d.smem[1], s>>>(probs, it, segs);  \
+    else if (pass == 0)                                                                                \
+      dg_batched_kernel<T, NN, false><<<d.count, threads, d.smem[0], s>>>(probs, it, segs);            \
+    else dg_batched_kernel<T, NN, true><<<d.count, threads, d.smem[1], s>>>(probs, it, segs);          \
     break;
     SIPG_BATCH_CASE(2)
     SIPG_BATCH_CASE(3)
@@ -421,24 +384,6 @@ cudaError_t batch_dg_degree(const BatchPlan<T> &P, const typename BatchPlan<T>::
   }
   note_launch();
   return cudaGetLastError();
-}
-
-// One pass over the plan's work items with the descriptors probs (device).
-template <typename T>
-cudaError_t batch_dg_pass(const BatchPlan<T> &P, const BatchProb<T> *probs, bool integrate, const Seg *segs,
-                          cudaStream_t s) {
-  const int ni = (int)P.items.size();
-  if (ni == 0) return cudaSuccess;
-  if (P.curved) {
-    if (integrate) dg_batched_kernel<T, true><<<P.grid, kBatchThreads, P.smem, s>>>(probs, P.d_items, ni, segs);
-    else dg_batched_kernel<T, false><<<P.grid, kBatchThreads, P.smem, s>>>(probs, P.d_items, ni, segs);
-    note_launch();
-    return cudaGetLastError();
-  }
-  cudaError_t e = cudaSuccess;
-  for (const auto &d : P.degrees)
-    if (e == cudaSuccess) e = batch_dg_degree<T>(P, d, probs, segs, s);
-  return e;
 }
 
 // ---------------------------------------------- batched vector steps of the V-cycle
@@ -486,16 +431,10 @@ template cudaError_t batch_plan_build<float>(BatchPlan<float> &, const std::vect
                                              const std::vector<int> &, bool);
 template void batch_plan_free<double>(BatchPlan<double> &);
 template void batch_plan_free<float>(BatchPlan<float> &);
-template cudaError_t batch_apply<double>(BatchPlan<double> &, cudaStream_t);
-template cudaError_t batch_apply<float>(BatchPlan<float> &, cudaStream_t);
 template cudaError_t batch_dg_degree<double>(const BatchPlan<double> &, const BatchPlan<double>::Degree &,
-                                             const BatchProb<double> *, const Seg *, cudaStream_t);
+                                             const BatchProb<double> *, int, const Seg *, cudaStream_t);
 template cudaError_t batch_dg_degree<float>(const BatchPlan<float> &, const BatchPlan<float>::Degree &,
-                                            const BatchProb<float> *, const Seg *, cudaStream_t);
-template cudaError_t batch_dg_pass<double>(const BatchPlan<double> &, const BatchProb<double> *, bool, const Seg *,
-                                           cudaStream_t);
-template cudaError_t batch_dg_pass<float>(const BatchPlan<float> &, const BatchProb<float> *, bool, const Seg *,
-                                          cudaStream_t);
+                                            const BatchProb<float> *, int, const Seg *, cudaStream_t);
 
 cudaError_t seg_dot(const Seg *segs, const SegGrid &g, int which, double *partials, unsigned *counter, double *sc,
                     int sc_stride, int slot, cudaStream_t s) {

@@ -394,32 +394,16 @@ __global__ void __launch_bounds__(256) c_prolongate_add_kernel(const FEArgs<T> a
 // one its own launch gives.  A problem whose flexible-CG system has left the
 // iteration (segs[p].active == 0) is skipped.
 
-template <typename T>
+// One kernel per degree (see dg_batched_kernel).
+template <typename T, int N>
 __global__ void __launch_bounds__(kBatchCellThreads) fe_cell_batched_kernel(const FETask<T> *__restrict__ tasks,
                                                                           const WorkItem *__restrict__ items,
                                                                           const Seg *__restrict__ segs) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T *sm = reinterpret_cast<T *>(smem_raw);
   const WorkItem w = items[blockIdx.x];
   if (segs && !segs[w.p].active) return;
-  const FETask<T> &P = tasks[w.p];
-  switch (P.a.deg + 1) {
-#define SIPG_FEB_CASE(NN) \
-  case NN:                \
-    fe_cell_body<T, NN>(P.a, P.a.u, P.a.ebuf, w.cell0, w.ncta, sm); \
-    break;
-    SIPG_FEB_CASE(2)
-    SIPG_FEB_CASE(3)
-    SIPG_FEB_CASE(4)
-    SIPG_FEB_CASE(5)
-    SIPG_FEB_CASE(6)
-    SIPG_FEB_CASE(7)
-    SIPG_FEB_CASE(8)
-    SIPG_FEB_CASE(9)
-#undef SIPG_FEB_CASE
-    default:
-      break;
-  }
+  const FEArgs<T> &a = tasks[w.p].a;
+  fe_cell_body<T, N>(a, a.u, a.ebuf, w.cell0, w.ncta, reinterpret_cast<T *>(smem_raw));
 }
 
 // Axis-aligned cells: item = brick w.cell0 of problem w.p, the whole operator;
@@ -842,6 +826,12 @@ cudaError_t launch_fe_box(const FEArgs<T> &a, cudaStream_t s) {
   }
 }
 
+// shared memory of a block of kBatchCellThreads / n^2 curved cells
+template <typename T>
+static size_t fe_batch_smem(int n) {
+  return (size_t)(kBatchCellThreads / (n * n)) * fe_curved_cell_values(n) * sizeof(T);
+}
+
 template <typename T, int N>
 static cudaError_t prep_fe_n() {
   constexpr cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
@@ -849,6 +839,7 @@ static cudaError_t prep_fe_n() {
   cudaError_t e = cudaSuccess;
   for (cudaError_t r : {cudaFuncSetAttribute(fe_cell_kernel<T, N, false>, at, smem),
                         cudaFuncSetAttribute(fe_cell_kernel<T, N, true>, at, smem),
+                        cudaFuncSetAttribute(fe_cell_batched_kernel<T, N>, at, (int)fe_batch_smem<T>(N)),
                         cudaFuncSetAttribute(fe_box_kernel<T, N>, at, kFEBoxSmem),
                         cudaFuncSetAttribute(fe_box_batched_kernel<T, N>, at, kFEBoxSmem)})
     if (r != cudaSuccess) e = r;
@@ -1015,10 +1006,27 @@ cudaError_t launch_fe_gather(const FEArgs<T> &a, cudaStream_t s) {
 }
 
 template <typename T>
-cudaError_t launch_fe_cells_batched(const FETask<T> *tasks, const WorkItem *items, int nitems, size_t smem,
-                                    const Seg *segs, cudaStream_t s) {
+cudaError_t launch_fe_cells_batched(int n, const FETask<T> *tasks, const WorkItem *items, int nitems, const Seg *segs,
+                                    cudaStream_t s) {
   if (nitems <= 0) return cudaSuccess;
-  fe_cell_batched_kernel<T><<<nitems, kBatchCellThreads, smem, s>>>(tasks, items, segs);
+  const int threads = kBatchCellThreads / (n * n) * n * n;
+  switch (n) {
+#define SIPG_FEB_CASE(NN)                                                                                 \
+  case NN:                                                                                                \
+    fe_cell_batched_kernel<T, NN><<<nitems, threads, fe_batch_smem<T>(NN), s>>>(tasks, items, segs);      \
+    break;
+    SIPG_FEB_CASE(2)
+    SIPG_FEB_CASE(3)
+    SIPG_FEB_CASE(4)
+    SIPG_FEB_CASE(5)
+    SIPG_FEB_CASE(6)
+    SIPG_FEB_CASE(7)
+    SIPG_FEB_CASE(8)
+    SIPG_FEB_CASE(9)
+#undef SIPG_FEB_CASE
+    default:
+      return cudaErrorInvalidValue;
+  }
   note_launch();
   return cudaGetLastError();
 }
@@ -1055,13 +1063,6 @@ cudaError_t launch_fe_nodes_batched(const FETask<T> *tasks, const NodeItem *item
   fe_nodes_batched_kernel<T><<<nitems, kBatchNodeThreads, 0, s>>>(tasks, items, segs, kind);
   note_launch();
   return cudaGetLastError();
-}
-
-int tile_values(int n) { return fe_curved_cell_values(n); }
-
-template <typename T>
-cudaError_t prep_fe_cells_batched(size_t smem) {
-  return cudaFuncSetAttribute(fe_cell_batched_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
 template <typename T>
@@ -1399,13 +1400,12 @@ cudaError_t launch_dg_transfer(const XferGeom &g, const T *P1, const T *in, T *o
   template cudaError_t launch_fe_gather<T>(const FEArgs<T> &, cudaStream_t);                            \
   template cudaError_t launch_fe_stencil_apply<T>(const FEArgs<T> &, const T *, cudaStream_t);          \
   template cudaError_t launch_c_prolongate_add<T>(const FEArgs<T> &, const T *, T *, cudaStream_t, int64_t); \
-  template cudaError_t launch_fe_cells_batched<T>(const FETask<T> *, const WorkItem *, int, size_t,            \
-                                                  const Seg *, cudaStream_t);                                  \
+  template cudaError_t launch_fe_cells_batched<T>(int, const FETask<T> *, const WorkItem *, int, const Seg *,  \
+                                                  cudaStream_t);                                               \
   template cudaError_t launch_fe_box_batched<T>(int, const FETask<T> *, const WorkItem *, int, size_t,         \
                                                 const Seg *, cudaStream_t);                                    \
   template cudaError_t launch_fe_nodes_batched<T>(const FETask<T> *, const NodeItem *, int, const Seg *, int, \
                                                   cudaStream_t);                                               \
-  template cudaError_t prep_fe_cells_batched<T>(size_t);                                                       \
   template cudaError_t launch_fe_prolongate_add<T>(const XferGeom &, const T *, const T *, T *,         \
                                                    cudaStream_t);                                       \
   template cudaError_t launch_fe_restrict_nodes<T>(const XferGeom &, const T *, const T *, T *,         \

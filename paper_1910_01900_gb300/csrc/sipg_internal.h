@@ -418,8 +418,8 @@ struct NodeItem {
   int p, blk;
 };
 template <typename T>
-cudaError_t launch_fe_cells_batched(const FETask<T> *tasks, const WorkItem *items, int nitems, size_t smem,
-                                    const Seg *segs, cudaStream_t s);
+cudaError_t launch_fe_cells_batched(int n, const FETask<T> *tasks, const WorkItem *items, int nitems, const Seg *segs,
+                                    cudaStream_t s);
 // axis-aligned cells: the bricks of all problems of one degree
 template <typename T>
 cudaError_t launch_fe_box_batched(int n, const FETask<T> *tasks, const WorkItem *items, int nitems, size_t smem,
@@ -428,9 +428,6 @@ cudaError_t launch_fe_box_batched(int n, const FETask<T> *tasks, const WorkItem 
 template <typename T>
 cudaError_t launch_fe_nodes_batched(const FETask<T> *tasks, const NodeItem *items, int nitems, const Seg *segs,
                                     int kind, cudaStream_t s);
-template <typename T>
-cudaError_t prep_fe_cells_batched(size_t smem);
-int tile_values(int n);   // shared-memory values per cell of the cell passes (sumfac.cuh)
 // batched vector steps (batch.cu); op as in vec_batched_kernel
 struct VecTask {
   int op = 0;
@@ -451,18 +448,17 @@ cudaError_t launch_batch_fcg_cond(const int *any, cudaGraphConditionalHandle h, 
 
 template <typename T>
 struct BatchPlan {
-  // axis-aligned problems: the items of one degree and their launch
+  // the items of one degree and their launch: thread groups (of n^2 threads) and
+  // shared memory (evaluation, integration or the one pass)
   struct Degree {
     int n, first, count, groups;
-    size_t smem;
+    size_t smem[2];
   };
   std::vector<Degree> degrees;
   std::vector<BatchProb<T>> probs;
   std::vector<WorkItem> items;
   BatchProb<T> *d_probs = nullptr;
   WorkItem *d_items = nullptr;
-  size_t smem = 0;
-  int grid = 0;
   bool curved = false;
 };
 
@@ -471,16 +467,11 @@ cudaError_t batch_plan_build(BatchPlan<T> &P, const std::vector<DGArgs<T>> &args
                              bool curved);
 template <typename T>
 void batch_plan_free(BatchPlan<T> &P);
-template <typename T>
-cudaError_t batch_apply(BatchPlan<T> &P, cudaStream_t s);
-// axis-aligned problems: the pass over one degree's items alone
+// one pass over one degree's items with the descriptors probs (device): 0 the
+// evaluation, 1 the integration or the one pass of axis-aligned cells
 template <typename T>
 cudaError_t batch_dg_degree(const BatchPlan<T> &P, const typename BatchPlan<T>::Degree &d, const BatchProb<T> *probs,
-                            const Seg *segs, cudaStream_t s);
-// one pass of the batched DG operator with the descriptors probs (device)
-template <typename T>
-cudaError_t batch_dg_pass(const BatchPlan<T> &P, const BatchProb<T> *probs, bool integrate, const Seg *segs,
-                          cudaStream_t s);
+                            int pass, const Seg *segs, cudaStream_t s);
 constexpr int kSegSlots = 8;   // scalar slots per problem (FCG layout of solver.cu, 4: b.b, 5: r0.r0)
 // Block map of the batched vector kernels (batch.cu): g.nb[p] blocks for
 // system p, one per kSegChunk entries (at least one), its partial sums at

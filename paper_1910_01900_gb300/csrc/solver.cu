@@ -2597,13 +2597,12 @@ struct BatchCycle {
   int np = 0;
   bool curved = false;
   BatchPlan<T> dg;                        // DG work items of the finest levels
-  WorkItem *fe_items = nullptr;           // FE cell items
-  int n_fe_items = 0;
-  size_t fe_smem = 0;
-  // axis-aligned cells: each problem's FE brick, and the items of each degree
+  // FE items, degree by degree: groups of cells, or (axis-aligned cells) bricks,
+  // each problem's own
+  WorkItem *fe_items = nullptr;
   struct FEDegree {
     int n, first, count;
-    size_t smem;
+    size_t smem;   // bricks
   };
   std::vector<std::array<int, 3>> brick;
   std::vector<FEDegree> fe_degrees;
@@ -2854,11 +2853,12 @@ bool batch_cycle_applicable(const sipg_batch *B) {
   return true;
 }
 
-// Axis-aligned problems have one launch per degree and pass, which depend on
-// nothing of another degree: inside a stream capture on s they go into branches
-// side by side, on s and on the streams of the first problem of each degree,
-// through consecutive passes without a meeting in between.  One after another,
-// launches of 10 us on 50 to 250 blocks left most of the chip idle.
+// The cell passes have one launch per degree, which depends on nothing of
+// another degree: they go into branches side by side, on s and on the streams
+// of the first problem of each degree, through consecutive passes without a
+// meeting in between.  One after another, launches of 10 us on 50 to 250 blocks
+// left most of the chip idle (operator of eight small curved problems of five
+// degrees 296 us, side by side 136 us).
 struct DegreeBranches {
   sipg_batch *B;
   cudaStream_t s;
@@ -2889,6 +2889,19 @@ struct DegreeBranches {
   }
 };
 
+// The finest-level operator of all problems with the plan's descriptors
+// (pointers, modes, active flags), on the batch's stream.
+void batch_apply(sipg_batch *B) {
+  const BatchPlan<double> &P = B->plan;
+  CK(cudaMemcpyAsync(P.d_probs, P.probs.data(), P.probs.size() * sizeof(BatchProb<double>), cudaMemcpyHostToDevice,
+                     B->stream));
+  DegreeBranches br{B, B->stream, {}};
+  for (int pass = P.curved ? 0 : 1; pass < 2; ++pass)
+    for (const auto &d : P.degrees)
+      CK(batch_dg_degree<double>(P, d, P.d_probs, pass, nullptr, P.degrees.size() > 1 ? br.of(d.n) : B->stream));
+  br.join();
+}
+
 // Issue the batched cycle's launches on s (inside a stream capture): the
 // problems that fill the GPU alone run their own cycle on their own stream,
 // beside the shared launches of the others.
@@ -2906,7 +2919,7 @@ void batch_cycle_emit(sipg_batch *B, BatchCycle<T> &C, cudaStream_t s) {
   }
   DegreeBranches br{B, s, std::vector<char>(C.solo.begin(), C.solo.end())};
   for (const BLaunch &r : C.prog) {
-    const bool by_degree = !C.curved && (r.kind == 3 || r.kind == 4);
+    const bool by_degree = r.kind >= 2 && r.kind <= 4;
     if (!by_degree) br.join();
     switch (r.kind) {
       case 0:
@@ -2917,16 +2930,15 @@ void batch_cycle_emit(sipg_batch *B, BatchCycle<T> &C, cudaStream_t s) {
         break;
       case 2:
       case 3:
-        if (C.curved) CK(batch_dg_pass<T>(C.dg, C.dgt + r.off, r.kind == 3, segs, s));
-        else
-          for (const auto &d : C.dg.degrees) CK(batch_dg_degree<T>(C.dg, d, C.dgt + r.off, segs, br.of(d.n)));
+        for (const auto &d : C.dg.degrees)
+          CK(batch_dg_degree<T>(C.dg, d, C.dgt + r.off, r.kind - 2, segs, br.of(d.n)));
         break;
       case 4:
-        if (C.curved)
-          CK(launch_fe_cells_batched<T>(C.fet + r.off, C.fe_items, C.n_fe_items, C.fe_smem, segs, s));
-        for (const auto &d : C.fe_degrees)
-          CK(launch_fe_box_batched<T>(d.n, C.fet + r.off, C.fe_items + d.first, d.count, d.smem, segs,
-                                      br.of(d.n)));
+        for (const auto &d : C.fe_degrees) {
+          const WorkItem *it = C.fe_items + d.first;
+          if (C.curved) CK(launch_fe_cells_batched<T>(d.n, C.fet + r.off, it, d.count, segs, br.of(d.n)));
+          else CK(launch_fe_box_batched<T>(d.n, C.fet + r.off, it, d.count, d.smem, segs, br.of(d.n)));
+        }
         break;
       case 5:
         CK(launch_fe_nodes_batched<T>(C.fet + r.off, C.items_g, C.n_g, segs, 0, s));
@@ -3000,34 +3012,30 @@ std::unique_ptr<BatchCycle<T>> batch_cycle_build(sipg_batch *B) {
       a0.back().ncells = 0;   // no DG items
       continue;
     }
-    if (C->curved) {
-      const int cb = kBatchCellThreads / (F.n * F.n);
-      C->fe_smem = std::max(C->fe_smem, (size_t)cb * tile_values(F.n) * sizeof(T));
-      for (int q = 0; q < F.ncells; q += cb) fei.push_back({p, q, (int)std::min<int64_t>(cb, F.ncells - q)});
-    }
     for (int64_t q = 0; q * kBatchNodeThreads < D.ndofs; ++q) nd.push_back({p, (int)q});
     for (int64_t q = 0; q * kBatchNodeThreads < F.ndofs; ++q) ng.push_back({p, (int)q});
   }
   CK(batch_plan_build<T>(C->dg, a0, nn, C->curved));
   C->brick.assign(np, {1, 1, 1});
-  if (!C->curved) {   // FE bricks, degree by degree: full ones (the problems together fill the GPU)
-    for (int n = kMaxN; n >= 2; --n) {
-      typename BatchCycle<T>::FEDegree d{n, (int)fei.size(), 0, 0};
-      for (int p = 0; p < np; ++p) {
-        const Level &F = B->ctx[p]->lv[B->ctx[p]->L - 1];
-        if (C->solo[p] || F.n != n) continue;
-        fe_box_brick<T>(n, F.m, INT_MAX, C->brick[p].data());
-        int nb = 1;
-        for (int e = 0; e < 3; ++e) nb *= (F.m[e] + C->brick[p][e] - 1) / C->brick[p][e];
-        for (int q = 0; q < nb; ++q) fei.push_back({p, q, 0});
-        d.smem = std::max(d.smem, (size_t)fe_box_values(F.deg, C->brick[p].data()) * sizeof(T));
+  for (int n = kMaxN; n >= 2; --n) {   // bricks: full ones (the problems together fill the GPU)
+    typename BatchCycle<T>::FEDegree d{n, (int)fei.size(), 0, 0};
+    for (int p = 0; p < np; ++p) {
+      const Level &F = B->ctx[p]->lv[B->ctx[p]->L - 1];
+      if (C->solo[p] || F.n != n) continue;
+      if (C->curved) {
+        const int cb = kBatchCellThreads / (n * n);
+        for (int q = 0; q < F.ncells; q += cb) fei.push_back({p, q, (int)std::min<int64_t>(cb, F.ncells - q)});
+        continue;
       }
-      d.count = (int)fei.size() - d.first;
-      if (d.count) C->fe_degrees.push_back(d);
+      fe_box_brick<T>(n, F.m, INT_MAX, C->brick[p].data());
+      int nb = 1;
+      for (int e = 0; e < 3; ++e) nb *= (F.m[e] + C->brick[p][e] - 1) / C->brick[p][e];
+      for (int q = 0; q < nb; ++q) fei.push_back({p, q, 0});
+      d.smem = std::max(d.smem, (size_t)fe_box_values(F.deg, C->brick[p].data()) * sizeof(T));
     }
+    d.count = (int)fei.size() - d.first;
+    if (d.count) C->fe_degrees.push_back(d);
   }
-  if (C->curved) CK(prep_fe_cells_batched<T>(C->fe_smem));
-  C->n_fe_items = (int)fei.size();
   C->n_d = (int)nd.size();
   C->n_g = (int)ng.size();
   // the program, task by task
@@ -3225,15 +3233,11 @@ void batch_build_fcg_chunk(sipg_batch *B) {
     }
     for (int i = 0; i < kFcgChunk; ++i) {
       body(add_if_node(s, hA[i]), &B->fcg_kA[i], [&]() {
-        if (B->plan.curved) {
-          CK(batch_dg_pass<double>(B->plan, B->d_app, false, B->d_segs, s2));
-          CK(batch_dg_pass<double>(B->plan, B->d_app, true, B->d_segs, s2));
-        } else {
-          DegreeBranches br{B, s2, {}};
+        DegreeBranches br{B, s2, {}};
+        for (int pass = B->plan.curved ? 0 : 1; pass < 2; ++pass)
           for (const auto &d : B->plan.degrees)
-            CK(batch_dg_degree<double>(B->plan, d, B->d_app, B->d_segs, br.of(d.n)));
-          br.join();
-        }
+            CK(batch_dg_degree<double>(B->plan, d, B->d_app, pass, B->d_segs, br.of(d.n)));
+        br.join();
         CK(seg_dot(B->d_segs, B->sg, 2, B->partials, B->counters, B->sc, st, 2, s2));
         CK(seg_update_xr(B->d_segs, B->sg, B->partials, B->counters, B->sc, st, s2));
         CK(launch_batch_fcg_check(B->sc, st, B->d_segs, np, B->d_it, B->d_status, B->d_hist, B->d_rn, B->d_r0,
@@ -3313,7 +3317,7 @@ sipg_status batch_solve_device(sipg_batch *B, const double *const *b, double *co
   CK(cudaEventRecord(e0, s));
   CK(cudaMemcpyAsync(B->d_segs, B->segs.data(), np * sizeof(Seg), cudaMemcpyHostToDevice, s));
   batch_set_plan(B, 2, xu.data(), rout.data());   // r = b - A x
-  CK(batch_apply(B->plan, s));
+  batch_apply(B);
   CK(seg_dot(B->d_segs, B->sg, 0, B->partials, B->counters, B->sc, st, 4, s));
   batch_precondition(B);
   CK(seg_dot(B->d_segs, B->sg, 1, B->partials, B->counters, B->sc, st, 0, s));
@@ -3419,11 +3423,11 @@ sipg_status batch_solve_impl(sipg_batch *B, const double *const *b, double *cons
       K,
       [&]() {   // r = b - A x
         batch_set_plan(B, 2, xu.data(), rout.data());
-        CK(batch_apply(B->plan, B->stream));
+        batch_apply(B);
       },
       [&]() {   // v = A p
         batch_set_plan(B, 0, pu.data(), vout.data());
-        CK(batch_apply(B->plan, B->stream));
+        batch_apply(B);
       },
       [&]() { batch_precondition(B); }, rtol, maxit, infos);
 }
@@ -3659,7 +3663,7 @@ sipg_status sipg_batch_apply(sipg_batch *B, const double *const *u, double *cons
   return bguarded(B, [&]() -> sipg_status {
     for (size_t p = 0; p < B->ctx.size(); ++p) B->segs[p].active = 1;
     batch_set_plan(B, 0, u, v);
-    CK(batch_apply(B->plan, B->stream));
+    batch_apply(B);
     return SIPG_OK;
   });
 }
