@@ -14,6 +14,7 @@
 // The same node pass, fed with a DG vector as the element buffer, is the
 // c-restriction (sum of the duplicated DG nodes, Section 3.2 c-coarsening).
 #include <algorithm>
+#include <climits>
 
 #include "curved_tile.cuh"
 #include "fe_transfer.cuh"
@@ -355,6 +356,16 @@ __device__ __forceinline__ void c_prolongate_dof(const FEArgs<T> &a, const T *xc
                     (cell / (a.m[0] * a.m[1])) * a.deg + p / n2};
   if (node_constrained(g, a.grid, a.bc)) return;
   xdg[idx] += xc[g[0] + (size_t)a.grid[0] * (g[1] + (size_t)a.grid[1] * g[2])];
+}
+
+// one value per thread (small meshes, see launch_c_prolongate_add)
+template <typename T>
+__global__ void __launch_bounds__(256) c_prolongate_values_kernel(const FEArgs<T> a, const T *__restrict__ xc, T *xdg,
+                                                                 const int64_t dg_stride) {
+  const int n = a.deg + 1;
+  const long idx = (long)blockIdx.x * 256 + threadIdx.x;
+  if (idx >= (long)a.ncells * n * n * n) return;
+  c_prolongate_dof<T>(a, xc + blockIdx.y * a.vs, xdg + blockIdx.y * dg_stride, idx);   // vector blockIdx.y
 }
 
 // z-line by z-line of the cells: the coordinates once per N values, the loads
@@ -1072,6 +1083,14 @@ cudaError_t launch_c_prolongate_add(const FEArgs<T> &a, const T *xc, T *xdg, cud
   const int bs = 256;
   if (total == 0) return cudaSuccess;
   if (total >= (1L << 32)) return cudaErrorInvalidValue;   // the kernel's 32-bit index arithmetic
+  // FP64 on small meshes: a line of n values in one thread waits longer than the
+  // divisions of one value take (degree 8, 4^3 cells 2.9 us against 2.3 us; 6^3
+  // 3.1 / 3.2; degree 5, 6^3 2.4 / 2.4; in FP32 the lines are never slower)
+  if (sizeof(T) == 8 && n >= 6 && total < 100000) {
+    c_prolongate_values_kernel<T><<<dim3((unsigned)((total + bs - 1) / bs), a.nv), bs, 0, s>>>(a, xc, xdg, dg_stride);
+    note_launch();
+    return cudaGetLastError();
+  }
   const dim3 grid((unsigned)((lines + bs - 1) / bs), a.nv);
   switch (n) {
 #define SIPG_CPRO_CASE(NN) \
@@ -1096,13 +1115,28 @@ cudaError_t launch_c_prolongate_add(const FEArgs<T> &a, const T *xc, T *xdg, cud
 
 // The p-transfers by bricks: the degree pairs of the default sequence p ->
 // floor(p/2) from degree 3 up (2 -> 1 has its own node pass); the other
-// sequences and the 2:1 transfers keep the kernels for any pair.
+// sequences and the 2:1 transfers keep the kernels for any pair, and so do these
+// pairs where those are the faster ones: below the mesh cells here, by fine
+// degree 3..8 (INT_MAX: always).  Prolongation: few coarse nodes per fine node, or a mesh
+// that leaves most SMs without a brick (FP32 3 -> 1 16^3 cells 2.7 us against 6.4
+// us by bricks, 28^3 6.8 / 7.3, 32^3 9.1 / 8.2; 4 -> 2 12^3 3.6 / 4.0, 16^3 5.5 /
+// 4.3; FP64 3 -> 1 16^3 5.2 / 7.5, 20^3 8.3 / 8.2).  Restriction: in FP64 the
+// halo's arithmetic (6 -> 3 16^3 36.3 / 38.8, 20^3 65.6 / 64.7; 7 -> 3 20^3 82.1
+// / 93.8; 8 -> 4 16^3 77.3 / 92.5).
 #define SIPG_PAIRS(X) X(4, 2) X(5, 3) X(6, 3) X(7, 4) X(8, 4) X(9, 5)
-bool fe_transfer_box_ok(const XferGeom &g) {
-#define SIPG_PAIR(NF, NC) if (g.kind == 1 && g.pf == NF - 1 && g.pc == NC - 1) return true;
+constexpr int kProlongLeast[2][6] = {{8000, 600, 0, 0, 0, 0}, {29000, 3000, 512, 0, 512, 0}};
+constexpr int kRestrictLeast[2][6] = {{0, 0, 0, 8000, INT_MAX, INT_MAX}, {0, 0, 0, 0, 0, 0}};
+static bool transfer_by_bricks(const XferGeom &g, const int (&least)[6]) {
+  const int64_t cells = (int64_t)g.mc[0] * g.mc[1] * g.mc[2];
+#define SIPG_PAIR(NF, NC) \
+  if (g.kind == 1 && g.pf == NF - 1 && g.pc == NC - 1) return cells >= least[NF - 4] && least[NF - 4] < INT_MAX;
   SIPG_PAIRS(SIPG_PAIR)
 #undef SIPG_PAIR
   return false;
+}
+template <typename T>
+bool fe_restrict_box_ok(const XferGeom &g) {
+  return transfer_by_bricks(g, kRestrictLeast[sizeof(T) == 4]);
 }
 // bricks as the operator's: thin ones, about 16 fine nodes along x and y
 static int64_t transfer_bricks(const XferGeom &g, int b[3]) {
@@ -1122,8 +1156,9 @@ cudaError_t launch_fe_restrict_box(const XferGeom &g, const T *P1, const T *rf, 
   const int ex = ((b[0] + 1) * g.pf + 1) | 1, ey = (b[1] + 1) * g.pf + 1, oz = b[2] * g.pc + 1;
   const size_t smem = (size_t)ex * ey * oz * sizeof(T);
 #define SIPG_PAIR(NF, NC)                                                                                   \
-  if (g.pf == NF - 1 && g.pc == NC - 1)                                                                     \
-    fe_restrict_box_kernel<T, NF, NC><<<dim3((unsigned)n, g.nv), 256, smem, s>>>(g, b[0], b[1], b[2], P1, rf, rc, x0, dinv, c3);
+  if constexpr (kRestrictLeast[sizeof(T) == 4][NF - 4] < INT_MAX)                                           \
+    if (g.pf == NF - 1 && g.pc == NC - 1)                                                                   \
+      fe_restrict_box_kernel<T, NF, NC><<<dim3((unsigned)n, g.nv), 256, smem, s>>>(g, b[0], b[1], b[2], P1, rf, rc, x0, dinv, c3);
   SIPG_PAIRS(SIPG_PAIR)
 #undef SIPG_PAIR
   note_launch();
@@ -1152,7 +1187,7 @@ cudaError_t launch_fe_prolongate_add(const XferGeom &g, const T *P1, const T *xc
   const int bs = 256;
   if (total == 0) return cudaSuccess;
   if (total >= (1L << 32)) return cudaErrorInvalidValue;   // the kernel's 32-bit grid coordinates
-  if (fe_transfer_box_ok(g)) return launch_fe_prolongate_box<T>(g, P1, xc, xf, s);
+  if (transfer_by_bricks(g, kProlongLeast[sizeof(T) == 4])) return launch_fe_prolongate_box<T>(g, P1, xc, xf, s);
   const dim3 grid((unsigned)((total + bs - 1) / bs), g.nv);
   switch (g.pc + 1) {
     case 2:
@@ -1410,6 +1445,7 @@ cudaError_t launch_dg_transfer(const XferGeom &g, const T *P1, const T *in, T *o
                                                    cudaStream_t);                                       \
   template cudaError_t launch_fe_restrict_nodes<T>(const XferGeom &, const T *, const T *, T *,         \
                                                    cudaStream_t);                                       \
+  template bool fe_restrict_box_ok<T>(const XferGeom &);                                                \
   template cudaError_t launch_fe_restrict_box<T>(const XferGeom &, const T *, const T *, T *, T *, const T *, T, \
                                                  cudaStream_t);                                         \
   template cudaError_t launch_fe_restrict_cells<T>(const XferGeom &, const T *, const T *, T *,         \

@@ -289,10 +289,11 @@ template <typename T>
 cudaError_t launch_fe_prolongate_add(const XferGeom &g, const T *P1, const T *xc, T *xf, cudaStream_t s);
 template <typename T>
 cudaError_t launch_fe_restrict_cells(const XferGeom &g, const T *P1, const T *rf, T *ebuf_c, cudaStream_t s);
-// the p-transfers of the default sequence by bricks of cells (prolongation:
-// launch_fe_prolongate_add takes them): r_c = P^T r_f and, with x0, the coarse
+// the p-restrictions of the default sequence by bricks of cells, where that is
+// the faster way (the prolongations: launch_fe_prolongate_add takes them): r_c = P^T r_f and, with x0, the coarse
 // level's first Chebyshev step x0 = c3 D^-1 r_c, in one launch
-bool fe_transfer_box_ok(const XferGeom &g);
+template <typename T>
+bool fe_restrict_box_ok(const XferGeom &g);
 template <typename T>
 cudaError_t launch_fe_restrict_box(const XferGeom &g, const T *P1, const T *rf, T *rc, T *x0, const T *dinv, T c3,
                                    cudaStream_t s);

@@ -339,7 +339,7 @@ bool restrict_level(sipg_ctx *c, int l, const T *r, T *rc, T *x0 = nullptr, T c3
     CK(launch_fe_restrict_nodes<T>(xfer(c, l), (const T *)F.P1[pi], r, rc, c->stream));
     return false;
   }
-  if (F.t_kind != 0 && fe_transfer_box_ok(xfer(c, l))) {
+  if (F.t_kind != 0 && fe_restrict_box_ok<T>(xfer(c, l))) {
     CK(launch_fe_restrict_box<T>(xfer(c, l), (const T *)F.P1[pi], r, rc, x0, (const T *)c->lv[l - 1].dinv[pi], c3,
                                  c->stream));
     return x0 != nullptr;
