@@ -20,7 +20,8 @@
 // products whatever the brick, so its size changes no bit.  Measured (GB300),
 // one smoothing step with its launch: FP32 32^3 cells of degree 4 45 -> 29 us,
 // degree 2 13 us, 16^3 cells of degree 4 13 us; FP64 32^3 of degree 4 290 -> 273
-// us (FP64 pipe).  FP32 is bound by latency and occupancy: three stages with a
+// us (FP64 pipe); FP64 levels where the halo costs more than that saves take the
+// two passes (fe_two_pass).  FP32 is bound by latency and occupancy: three stages with a
 // barrier between them, 4 blocks of 256 threads per SM.
 #pragma once
 #include "sumfac.cuh"
@@ -256,10 +257,10 @@ __device__ __forceinline__ void fe_box_body(const FEArgs<T> &a, const int64_t vo
 }
 
 // Most threads of a block (the widest stage of the default bricks in two
-// rounds), and blocks per SM to leave registers for: FP64 at the highest
-// degrees takes what a cell's lines need.
+// rounds), and blocks per SM to leave registers for: FP64 takes what a cell's
+// lines need.
 template <typename T>
-__host__ __device__ constexpr int fe_box_threads(int n) { return sizeof(T) == 8 && n <= 7 ? 384 : 256; }
+__host__ __device__ constexpr int fe_box_threads(int) { return sizeof(T) == 8 ? 384 : 256; }
 template <typename T>
 __host__ __device__ constexpr int fe_box_blocks(int n) { return sizeof(T) == 8 ? 1 : (n <= 5 ? 4 : 3); }
 

@@ -1,7 +1,8 @@
 // Continuous FE levels of the cph hierarchy (Section 2, Eq. WeakFormFE;
 // Section 3.2 transfers), both precisions.
 //
-// FE operator on axis-aligned cells: one pass (fe_box.cuh).  On curved cells a
+// FE operator on axis-aligned cells: one pass (fe_box.cuh; fe_two_pass says
+// where not).  On curved cells a
 // cell pass evaluates (grad v, grad u) on every cell by sum
 // factorisation (same interpolation/derivative sweeps as the DG cell term)
 // after gathering the cell's nodes from the global grid (constrained
@@ -42,17 +43,68 @@ __device__ __forceinline__ bool node_constrained(const int g[3], const int grid[
          (g[2] == 0 && bc[4] == 0) || (g[2] == grid[2] - 1 && bc[5] == 0);
 }
 
+// Shared memory of one axis-aligned cell of the cell pass: two tiles (x
+// fastest, y step XP, z step ZP), cells CS values apart; pitches counted for the
+// fewest wavefronts of the three line directions.
+template <int N>
+struct BoxCellTile {
+  static constexpr int XP = N == 8 ? 9 : N;
+  static constexpr int ZP = N == 2 ? 4 : N == 3 ? 9 : N == 4 ? 19 : N == 5 ? 25 : N == 6 ? 39 : N == 7 ? 52 : N == 8 ? 72 : 81;
+  static constexpr int T3 = ZP * N, CS = 2 * T3 + (cell_values(N) - 2 * T3) % 16;
+};
+// shared-memory values per cell of the cell pass
+template <int N, bool CURVED>
+constexpr int kFECellValues = CURVED ? fe_curved_cell_values(N) : BoxCellTile<N>::CS;
+
+// An axis-aligned cell: its matrix is the sum over d of alpha_d times the
+// tensor product of K1 in direction d and M1 in the other two, 7 1D products:
+// along z a = M1 u, b = K1 u; along y c = M1 a, f = ay K1 a + az M1 b; along x
+// ax K1 c + M1 f.  x: the thread's z-line of u; the result goes to its x-line
+// of the cell's n^3 values at eb.
+template <typename T, int N>
+__device__ __forceinline__ void fe_box_cell_term(const FEArgs<T> &a, const int l, const bool act, T (&x)[N], T *t0,
+                                                 T *eb) {
+  using C = BoxCellTile<N>;
+  T *t1 = t0 + C::T3, y[N], k[N];
+  const int la = l % N, lb = l / N;
+  if (act) {
+    apply_mat<T, N, MK1>(x, y);
+    store_line<T, N>(t1, la + C::XP * lb, C::ZP, y);
+    apply_mat<T, N, MM1>(x, y);
+    store_line<T, N>(t0, la + C::XP * lb, C::ZP, y);
+  }
+  __syncthreads();
+  if (act) {
+    load_line<T, N>(t0, la + C::ZP * lb, C::XP, x);
+    apply_mat<T, N, MM1>(x, y);
+    store_line<T, N>(t0, la + C::ZP * lb, C::XP, y);
+    apply_mat<T, N, MK1>(x, k);
+    load_line<T, N>(t1, la + C::ZP * lb, C::XP, x);
+    apply_mat<T, N, MM1>(x, y);
+#pragma unroll
+    for (int q = 0; q < N; ++q) y[q] = fma(a.alpha[1], k[q], a.alpha[2] * y[q]);
+    store_line<T, N>(t1, la + C::ZP * lb, C::XP, y);
+  }
+  __syncthreads();
+  if (!act) return;
+  load_line<T, N>(t0, C::XP * la + C::ZP * lb, 1, x);
+  apply_mat<T, N, MK1>(x, k);
+  load_line<T, N>(t1, C::XP * la + C::ZP * lb, 1, x);
+  apply_mat<T, N, MM1>(x, y);
+#pragma unroll
+  for (int q = 0; q < N; ++q) eb[N * l + q] = fma(a.alpha[0], k[q], y[q]);
+}
+
 // The cell pass on cells cell0 .. cell0 + ncta - 1 of one vector (input ug,
 // element buffer ebv), one line of N points per thread, N^2 threads per cell
 // (threads beyond ncta N^2 only join the barriers).
-template <typename T, int N>
+template <typename T, int N, bool CURVED>
 __device__ __forceinline__ void fe_cell_body(const FEArgs<T> &a, const T *__restrict__ ug, T *__restrict__ ebv,
                                              const int cell0, const int ncta, T *sm) {
   constexpr int N2 = N * N, N3 = N2 * N;
   const int tid = threadIdx.x, cl = tid / N2, l = tid - cl * N2;
   const bool act = cl < ncta;
   const int cell = cell0 + (act ? cl : 0);
-  const CurvedLines<T, N> t(sm + cl * CurvedTile<N>::CF, l % N, l / N);
   // each thread gathers its z-line of the cell's nodes straight into
   // registers (constrained Dirichlet nodes read as zero); the first sweep
   // runs on them before anything goes to shared memory
@@ -68,6 +120,11 @@ __device__ __forceinline__ void fe_cell_body(const FEArgs<T> &a, const T *__rest
       x[q] = node_constrained(g, a.grid, a.bc) ? T(0) : ug[b0 + sz * g[2]];
     }
   }
+  if constexpr (!CURVED) {
+    fe_box_cell_term<T, N>(a, l, act, x, sm + cl * BoxCellTile<N>::CS, ebv + (size_t)cell * N3);
+    return;
+  }
+  const CurvedLines<T, N> t(sm + cl * CurvedTile<N>::CF, l % N, l / N);
   curved_interpolate<T, N>(t, act, x);
   curved_cell_term<T, N>(t, act, a.metric + (size_t)cell * 6 * N3 + l, x, [] {},
                          [](int, const T (&in)[N], T (&out)[N]) { apply_mat<T, N, MDt>(in, out); });
@@ -80,14 +137,14 @@ __device__ __forceinline__ void fe_cell_body(const FEArgs<T> &a, const T *__rest
 // cb cells per thread block (a launch parameter, cb N^2 threads); MULTI:
 // several vectors, block b = cell group b / nv of vector b % nv (compiled
 // apart from the single-vector kernel, whose offsets would cost registers)
-template <typename T, int N, bool MULTI>
+template <typename T, int N, bool CURVED, bool MULTI>
 __global__ void __launch_bounds__(kCellThreads) fe_cell_kernel(const FEArgs<T> a, const int cb) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *sm = reinterpret_cast<T *>(smem_raw);
   // block -> (cell group, vector); the vectors of one group are neighbours
   const int grp = MULTI ? blockIdx.x / a.nv : blockIdx.x, vec = MULTI ? blockIdx.x - grp * a.nv : 0;
   const int cell0 = grp * cb;
-  fe_cell_body<T, N>(a, MULTI ? a.u + vec * a.vs : a.u, MULTI ? a.ebuf + vec * a.es : a.ebuf, cell0,
+  fe_cell_body<T, N, CURVED>(a, MULTI ? a.u + vec * a.vs : a.u, MULTI ? a.ebuf + vec * a.es : a.ebuf, cell0,
                              min(cb, a.ncells - cell0), sm);
 }
 
@@ -406,7 +463,7 @@ __global__ void __launch_bounds__(256) c_prolongate_add_kernel(const FEArgs<T> a
 // iteration (segs[p].active == 0) is skipped.
 
 // One kernel per degree (see dg_batched_kernel).
-template <typename T, int N>
+template <typename T, int N, bool CURVED>
 __global__ void __launch_bounds__(kBatchCellThreads) fe_cell_batched_kernel(const FETask<T> *__restrict__ tasks,
                                                                           const WorkItem *__restrict__ items,
                                                                           const Seg *__restrict__ segs) {
@@ -414,7 +471,7 @@ __global__ void __launch_bounds__(kBatchCellThreads) fe_cell_batched_kernel(cons
   const WorkItem w = items[blockIdx.x];
   if (segs && !segs[w.p].active) return;
   const FEArgs<T> &a = tasks[w.p].a;
-  fe_cell_body<T, N>(a, a.u, a.ebuf, w.cell0, w.ncta, reinterpret_cast<T *>(smem_raw));
+  fe_cell_body<T, N, CURVED>(a, a.u, a.ebuf, w.cell0, w.ncta, reinterpret_cast<T *>(smem_raw));
 }
 
 // Axis-aligned cells: item = brick w.cell0 of problem w.p, the whole operator;
@@ -734,34 +791,56 @@ __global__ void dg_transfer_kernel(const XferGeom G, const T *__restrict__ P1, c
 }
 
 // ---------------------------------------------------------------- launchers
-// the width that a setting of cb cells runs at: the shared memory at most
+// Axis-aligned levels whose operator takes the cell and node passes all the
+// same: FP64 levels of degree p from kFETwoPass[p][0] to below [1] cells.  The one
+// pass is the faster one where two launches and the element buffer's way through
+// memory count, on small and on large meshes; between, and from degree 5 on,
+// FP64 pays for the arithmetic of the halo layer.  Two passes / one, us: degree
+// 2 6^3 10.4 / 8.5, 12^3 10.5 / 12.6, 16^3 12.9 / 14.7, 18^3 20.6 / 16.6; degree 3
+// 4^3 12.4 / 10.3, 10^3 12.5 / 18.6, 14^3 28.8 / 22.7; degree 4 4^3 13.4 / 12.6,
+// 10^3 17.6 / 20.8, 14^3 34 / 47, 20^3 84.4 / 86.4, 24^3 136 / 125; degree 5 16^3
+// 80 / 109; degree 7 12^3 94 / 176; degree 8 12^3 144 / 256.  In FP32, bound by
+// latency and memory, the one pass is never slower.
+constexpr int kFETwoPass[kMaxN][2] = {{0, 0},       {0, 0},       {1000, 5000}, {300, 2000}, {200, 12000},
+                                      {0, INT_MAX}, {0, INT_MAX}, {0, INT_MAX}, {0, INT_MAX}};
+template <typename T>
+bool fe_two_pass(int n, int64_t cells) {
+  return sizeof(T) == 8 && cells >= kFETwoPass[n - 1][0] && cells < kFETwoPass[n - 1][1];
+}
+// what is compiled: the cell pass on axis-aligned cells, and the one pass
 template <typename T, int N>
-static int fe_curved_cb(int cb) {
-  return std::min(cb, 232448 / (fe_curved_cell_values(N) * (int)sizeof(T)));
+constexpr bool kBoxCells = sizeof(T) == 8 && kFETwoPass[N - 1][1] > 0;
+template <typename T, int N>
+constexpr bool kOnePass = sizeof(T) == 4 || kFETwoPass[N - 1][1] < INT_MAX;
+
+// the width that a setting of cb cells runs at: the shared memory at most
+template <typename T, int N, bool CURVED>
+static int fe_cells_cb(int cb) {
+  return std::min(cb, 232448 / (kFECellValues<N, CURVED> * (int)sizeof(T)));
 }
 
-template <typename T, int N>
+template <typename T, int N, bool CURVED>
 static cudaError_t run_fe_cells(const FEArgs<T> &a, cudaStream_t s, int cb) {
   if (cb <= 0) cb = default_cb(N);
   if (cb > max_cb(N, sizeof(T))) return cudaErrorInvalidValue;
-  cb = fe_curved_cb<T, N>(cb);
-  const size_t smem = (size_t)cb * fe_curved_cell_values(N) * sizeof(T);
+  cb = fe_cells_cb<T, N, CURVED>(cb);
+  const size_t smem = (size_t)cb * kFECellValues<N, CURVED> * sizeof(T);
   const int64_t grid = (int64_t)((a.ncells + cb - 1) / cb) * a.nv;
   if (grid == 0) return cudaSuccess;
   if (grid > 0x7fffffff) return cudaErrorInvalidValue;
   if (a.nv > 1)
-    fe_cell_kernel<T, N, true><<<(unsigned)grid, cb * N * N, smem, s>>>(a, cb);
+    fe_cell_kernel<T, N, CURVED, true><<<(unsigned)grid, cb * N * N, smem, s>>>(a, cb);
   else
-    fe_cell_kernel<T, N, false><<<(unsigned)grid, cb * N * N, smem, s>>>(a, cb);
+    fe_cell_kernel<T, N, CURVED, false><<<(unsigned)grid, cb * N * N, smem, s>>>(a, cb);
   note_launch();
   return cudaGetLastError();
 }
 
-template <typename T, int N>
+template <typename T, int N, bool CURVED>
 static cudaError_t occ_fe_cells(int cb, int *blocks) {
-  cb = fe_curved_cb<T, N>(cb);
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fe_cell_kernel<T, N, false>, cb * N * N,
-                                                       (size_t)cb * fe_curved_cell_values(N) * sizeof(T));
+  cb = fe_cells_cb<T, N, CURVED>(cb);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fe_cell_kernel<T, N, CURVED, false>, cb * N * N,
+                                                       (size_t)cb * kFECellValues<N, CURVED> * sizeof(T));
 }
 
 // Cells per direction of a brick.  kFEBoxBrick[p]: about 16 own nodes along x
@@ -771,14 +850,15 @@ static cudaError_t occ_fe_cells(int cb, int *blocks) {
 // fewer bricks than the GPU can use, the side of most cells is halved until it
 // does: FP32 below 140 bricks (16^3 of degree 4: 128 bricks 14.4 us, 256 12.9
 // us), FP64, where the halo's arithmetic costs more, below 100 (50 us against
-// 61 us).  cb > 0: at most cb cells in all.  Sides are evened out over the
+// 61 us) and at degree 1, where it costs little, below 200 (16^3: 128 bricks 10.3
+// us, 256 8.5 us, in two passes 9.5 us).  cb > 0: at most cb cells in all.  Sides are evened out over the
 // bricks of a direction.
 constexpr int kFEBoxBrick[kMaxN][3] = {{1, 1, 1}, {16, 8, 4}, {8, 4, 4}, {5, 4, 2}, {4, 4, 2},
                                        {4, 2, 2}, {3, 2, 2},  {2, 2, 2}, {2, 2, 2}};
-constexpr int kFEBoxSmem = 176 * 1024;   // degree 8 in FP64: 170 KB
+constexpr int kFEBoxSmem = 96 * 1024;   // degree 8 in FP32: 85 KB
 template <typename T>
 void fe_box_brick(int n, const int m[3], int cb, int brick[3]) {
-  const int p = n - 1, least = sizeof(T) == 4 ? 140 : 100;
+  const int p = n - 1, least = sizeof(T) == 4 ? 140 : (p == 1 ? 200 : 100);
   int b[3] = {kFEBoxBrick[p][0], kFEBoxBrick[p][1], kFEBoxBrick[p][2]};
   for (;;) {
     int64_t bricks = 1;
@@ -820,9 +900,10 @@ cudaError_t launch_fe_box(const FEArgs<T> &a, cudaStream_t s) {
   if (a.ncells == 0) return cudaSuccess;
   if ((int64_t)a.grid[0] * a.grid[1] * a.grid[2] >= (1LL << 32)) return cudaErrorInvalidValue;
   switch (a.deg) {
-#define SIPG_FEBOX_CASE(NN) \
-  case NN - 1:              \
-    return run_fe_box<T, NN>(a, s);
+#define SIPG_FEBOX_CASE(NN)                                             \
+  case NN - 1:                                                          \
+    if constexpr (kOnePass<T, NN>) return run_fe_box<T, NN>(a, s);      \
+    return cudaErrorInvalidValue;
     SIPG_FEBOX_CASE(2)
     SIPG_FEBOX_CASE(3)
     SIPG_FEBOX_CASE(4)
@@ -837,23 +918,31 @@ cudaError_t launch_fe_box(const FEArgs<T> &a, cudaStream_t s) {
   }
 }
 
-// shared memory of a block of kBatchCellThreads / n^2 curved cells
-template <typename T>
-static size_t fe_batch_smem(int n) {
-  return (size_t)(kBatchCellThreads / (n * n)) * fe_curved_cell_values(n) * sizeof(T);
-}
+// shared memory of a block of kBatchCellThreads / n^2 cells
+template <typename T, int N, bool CURVED>
+constexpr int kFEBatchSmem = kBatchCellThreads / (N * N) * kFECellValues<N, CURVED> * (int)sizeof(T);
 
+template <typename T, int N, bool CURVED>
+static cudaError_t prep_fe_cells() {
+  constexpr cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  const int smem = fe_cells_cb<T, N, CURVED>(max_cb(N, sizeof(T))) * kFECellValues<N, CURVED> * (int)sizeof(T);
+  cudaError_t e = cudaSuccess;
+  for (cudaError_t r : {cudaFuncSetAttribute(fe_cell_kernel<T, N, CURVED, false>, at, smem),
+                        cudaFuncSetAttribute(fe_cell_kernel<T, N, CURVED, true>, at, smem),
+                        cudaFuncSetAttribute(fe_cell_batched_kernel<T, N, CURVED>, at, kFEBatchSmem<T, N, CURVED>)})
+    if (r != cudaSuccess) e = r;
+  return e;
+}
 template <typename T, int N>
 static cudaError_t prep_fe_n() {
   constexpr cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  const int smem = fe_curved_cb<T, N>(max_cb(N, sizeof(T))) * fe_curved_cell_values(N) * (int)sizeof(T);
-  cudaError_t e = cudaSuccess;
-  for (cudaError_t r : {cudaFuncSetAttribute(fe_cell_kernel<T, N, false>, at, smem),
-                        cudaFuncSetAttribute(fe_cell_kernel<T, N, true>, at, smem),
-                        cudaFuncSetAttribute(fe_cell_batched_kernel<T, N>, at, (int)fe_batch_smem<T>(N)),
-                        cudaFuncSetAttribute(fe_box_kernel<T, N>, at, kFEBoxSmem),
-                        cudaFuncSetAttribute(fe_box_batched_kernel<T, N>, at, kFEBoxSmem)})
-    if (r != cudaSuccess) e = r;
+  cudaError_t e = prep_fe_cells<T, N, true>();
+  if constexpr (kBoxCells<T, N>)
+    if (e == cudaSuccess) e = prep_fe_cells<T, N, false>();
+  if constexpr (kOnePass<T, N>)
+    for (cudaError_t r : {cudaFuncSetAttribute(fe_box_kernel<T, N>, at, kFEBoxSmem),
+                          cudaFuncSetAttribute(fe_box_batched_kernel<T, N>, at, kFEBoxSmem)})
+      if (r != cudaSuccess) e = r;
   return e;
 }
 
@@ -895,7 +984,9 @@ cudaError_t launch_fe_cells(int n, bool curved, const FEArgs<T> &a, bool diag_on
         return curved ? run_fe_diag<NN, true>(a, s) : run_fe_diag<NN, false>(a, s);          \
       return cudaErrorInvalidValue;                                                          \
     }                                                                                        \
-    return run_fe_cells<T, NN>(a, s, cb);
+    if (curved) return run_fe_cells<T, NN, true>(a, s, cb);                                  \
+    if constexpr (kBoxCells<T, NN>) return run_fe_cells<T, NN, false>(a, s, cb);             \
+    return cudaErrorInvalidValue;
   switch (n) {
     SIPG_FE_CASE(2)
     SIPG_FE_CASE(3)
@@ -976,10 +1067,12 @@ int fe_max_cells_per_block(int n) {
 }
 
 template <typename T>
-cudaError_t fe_blocks_per_sm(int n, int cb, int *blocks) {
-#define SIPG_FE_OCC(NN) \
-  case NN:              \
-    return occ_fe_cells<T, NN>(cb, blocks);
+cudaError_t fe_blocks_per_sm(int n, bool curved, int cb, int *blocks) {
+#define SIPG_FE_OCC(NN)                                                                 \
+  case NN:                                                                              \
+    if (curved) return occ_fe_cells<T, NN, true>(cb, blocks);                           \
+    if constexpr (kBoxCells<T, NN>) return occ_fe_cells<T, NN, false>(cb, blocks);      \
+    return cudaErrorInvalidValue;
   switch (n) {
     SIPG_FE_OCC(2)
     SIPG_FE_OCC(3)
@@ -1017,14 +1110,20 @@ cudaError_t launch_fe_gather(const FEArgs<T> &a, cudaStream_t s) {
 }
 
 template <typename T>
-cudaError_t launch_fe_cells_batched(int n, const FETask<T> *tasks, const WorkItem *items, int nitems, const Seg *segs,
-                                    cudaStream_t s) {
+cudaError_t launch_fe_cells_batched(int n, bool curved, const FETask<T> *tasks, const WorkItem *items, int nitems,
+                                    const Seg *segs, cudaStream_t s) {
   if (nitems <= 0) return cudaSuccess;
   const int threads = kBatchCellThreads / (n * n) * n * n;
   switch (n) {
-#define SIPG_FEB_CASE(NN)                                                                                 \
-  case NN:                                                                                                \
-    fe_cell_batched_kernel<T, NN><<<nitems, threads, fe_batch_smem<T>(NN), s>>>(tasks, items, segs);      \
+#define SIPG_FEB_CASE(NN)                                                                                     \
+  case NN:                                                                                                    \
+    if (curved) {                                                                                             \
+      constexpr int smem = kFEBatchSmem<T, NN, true>;                                                         \
+      fe_cell_batched_kernel<T, NN, true><<<nitems, threads, smem, s>>>(tasks, items, segs);                  \
+    } else if constexpr (kBoxCells<T, NN>) {                                                                  \
+      constexpr int smem = kFEBatchSmem<T, NN, false>;                                                        \
+      fe_cell_batched_kernel<T, NN, false><<<nitems, threads, smem, s>>>(tasks, items, segs);                 \
+    }                                                                                                         \
     break;
     SIPG_FEB_CASE(2)
     SIPG_FEB_CASE(3)
@@ -1049,7 +1148,8 @@ cudaError_t launch_fe_box_batched(int n, const FETask<T> *tasks, const WorkItem 
   switch (n) {
 #define SIPG_FEB_CASE(NN)                                                                                   \
   case NN:                                                                                                  \
-    fe_box_batched_kernel<T, NN><<<nitems, kBatchCellThreads, smem, s>>>(tasks, items, segs);               \
+    if constexpr (kOnePass<T, NN>)                                                                          \
+      fe_box_batched_kernel<T, NN><<<nitems, kBatchCellThreads, smem, s>>>(tasks, items, segs);             \
     break;
     SIPG_FEB_CASE(2)
     SIPG_FEB_CASE(3)
@@ -1429,14 +1529,15 @@ cudaError_t launch_dg_transfer(const XferGeom &g, const T *P1, const T *in, T *o
 #define SIPG_FE_INST(T)                                                                                   \
   template cudaError_t launch_fe_cells<T>(int, bool, const FEArgs<T> &, bool, cudaStream_t, int);       \
   template int fe_max_cells_per_block<T>(int);                                                          \
-  template cudaError_t fe_blocks_per_sm<T>(int, int, int *);                                            \
+  template cudaError_t fe_blocks_per_sm<T>(int, bool, int, int *);                                      \
+  template bool fe_two_pass<T>(int, int64_t);                                                           \
   template void fe_box_brick<T>(int, const int *, int, int *);                                          \
   template cudaError_t launch_fe_box<T>(const FEArgs<T> &, cudaStream_t);                               \
   template cudaError_t launch_fe_gather<T>(const FEArgs<T> &, cudaStream_t);                            \
   template cudaError_t launch_fe_stencil_apply<T>(const FEArgs<T> &, const T *, cudaStream_t);          \
   template cudaError_t launch_c_prolongate_add<T>(const FEArgs<T> &, const T *, T *, cudaStream_t, int64_t); \
-  template cudaError_t launch_fe_cells_batched<T>(int, const FETask<T> *, const WorkItem *, int, const Seg *,  \
-                                                  cudaStream_t);                                               \
+  template cudaError_t launch_fe_cells_batched<T>(int, bool, const FETask<T> *, const WorkItem *, int,         \
+                                                  const Seg *, cudaStream_t);                                  \
   template cudaError_t launch_fe_box_batched<T>(int, const FETask<T> *, const WorkItem *, int, size_t,         \
                                                 const Seg *, cudaStream_t);                                    \
   template cudaError_t launch_fe_nodes_batched<T>(const FETask<T> *, const NodeItem *, int, const Seg *, int, \

@@ -242,14 +242,17 @@ cudaError_t dg_blocks_per_sm(int n, bool curved, int pass, int cb, int *blocks);
 
 cudaError_t launch_dg_diag(int n, bool curved, const DGArgs<double> &a, double *diag, cudaStream_t s);
 
-// FE cell pass of curved cells at cb cells per block (0 = default); diag_only:
+// FE cell pass at cb cells per block (0 = default); diag_only:
 // the cell-local diagonal (setup, FP64)
 template <typename T>
 cudaError_t launch_fe_cells(int n, bool curved, const FEArgs<T> &a, bool diag_only, cudaStream_t s, int cb = 0);
 template <typename T>
 int fe_max_cells_per_block(int n);
 template <typename T>
-cudaError_t fe_blocks_per_sm(int n, int cb, int *blocks);
+cudaError_t fe_blocks_per_sm(int n, bool curved, int cb, int *blocks);
+// whether an axis-aligned level takes the cell and node passes (else the one pass)
+template <typename T>
+bool fe_two_pass(int n, int64_t cells);
 // axis-aligned cells: the operator with the epilogue (modes 0-2) in one pass
 template <typename T>
 cudaError_t launch_fe_box(const FEArgs<T> &a, cudaStream_t s);
@@ -419,8 +422,8 @@ struct NodeItem {
   int p, blk;
 };
 template <typename T>
-cudaError_t launch_fe_cells_batched(int n, const FETask<T> *tasks, const WorkItem *items, int nitems, const Seg *segs,
-                                    cudaStream_t s);
+cudaError_t launch_fe_cells_batched(int n, bool curved, const FETask<T> *tasks, const WorkItem *items, int nitems,
+                                    const Seg *segs, cudaStream_t s);
 // axis-aligned cells: the bricks of all problems of one degree
 template <typename T>
 cudaError_t launch_fe_box_batched(int n, const FETask<T> *tasks, const WorkItem *items, int nitems, size_t smem,

@@ -258,6 +258,12 @@ FEArgs<T> fe_args(sipg_ctx *c, const Level &L) {
   return a;
 }
 
+// whether an FE level's operator is the one pass of axis-aligned cells (else the cell and node passes)
+template <typename T>
+bool one_pass_fe(const Level &L) {
+  return !L.curved && !fe_two_pass<T>(L.n, L.ncells);
+}
+
 // out = epilogue(A_l u): mode 0 Au, 1 c1 x + c2 xp + c3 dinv (b - Au), 2 b - Au
 template <typename T>
 void apply_level(sipg_ctx *c, int l, const T *u, T *out, int mode, const T *x = nullptr, const T *xp = nullptr,
@@ -295,10 +301,10 @@ void apply_level(sipg_ctx *c, int l, const T *u, T *out, int mode, const T *x = 
     a.c3 = c3;
     if (L.stencil[pidx<T>()]) {
       CK(launch_fe_stencil_apply<T>(a, (const T *)L.stencil[pidx<T>()], c->stream));
-    } else if (!L.curved) {
+    } else if (one_pass_fe<T>(L)) {
       CK(launch_fe_box<T>(a, c->stream));
     } else {
-      CK(launch_fe_cells<T>(L.n, true, a, false, c->stream, L.cb[pidx<T>()][2]));
+      CK(launch_fe_cells<T>(L.n, L.curved, a, false, c->stream, L.cb[pidx<T>()][2]));
       CK(launch_fe_gather<T>(a, c->stream));
     }
   }
@@ -860,7 +866,7 @@ std::vector<int> tile_candidates(const Level &L, int pass, int keep) {
   std::vector<std::pair<double, int>> score;
   for (int cb = 1; cb <= maxcb; ++cb) {
     int occ = 0;
-    CK(pass < 2 ? dg_blocks_per_sm<T>(L.n, L.curved, pass, cb, &occ) : fe_blocks_per_sm<T>(L.n, cb, &occ));
+    CK(pass < 2 ? dg_blocks_per_sm<T>(L.n, L.curved, pass, cb, &occ) : fe_blocks_per_sm<T>(L.n, L.curved, cb, &occ));
     if (occ <= 0) continue;
     const int threads = cb * L.n * L.n;
     const double lanes = threads / (32.0 * ((threads + 31) / 32));
@@ -918,7 +924,7 @@ void autotune_level(sipg_ctx *c, int l, int pass) {
         CK(launch_dg_box<T>(L.n, a, c->stream));
       } else if (pass == 0) CK(launch_dg_eval<T>(L.n, a, c->stream, cb));
       else if (pass == 1) CK(launch_dg_integrate<T>(L.n, a, c->stream, cb));
-      else CK(launch_fe_cells<T>(L.n, true, f, false, c->stream, cb));
+      else CK(launch_fe_cells<T>(L.n, L.curved, f, false, c->stream, cb));
     };
     if (pass == 1 && L.curved) CK(launch_dg_eval<T>(L.n, a, c->stream, 0));   // valid scratch for the integration
     run();
@@ -1114,11 +1120,10 @@ void setup(sipg_ctx *c) {
     for (int l = c->solver ? 1 : c->L; l <= c->L; ++l) {
       const int k = c->lv[l].kind;
       if (k == 1 && c->lv[l].deg <= P.fe_assemble) continue;   // assembled stencil: no cell pass to tune
-      if (k == 1 && !c->lv[l].curved) continue;   // its brick follows from the mesh
-      // axis-aligned DG levels have one pass (1)
+      // axis-aligned DG levels have one pass (1); an FE level's brick follows from the mesh
       for (int pass = k == 0 ? (c->lv[l].curved ? 0 : 1) : 2; pass <= (k == 0 ? 1 : 2); ++pass) {
-        autotune_level<double>(c, l, pass);
-        autotune_level<float>(c, l, pass);
+        if (k == 0 || !one_pass_fe<double>(c->lv[l])) autotune_level<double>(c, l, pass);
+        if (k == 0 || !one_pass_fe<float>(c->lv[l])) autotune_level<float>(c, l, pass);
       }
       set_box(c->lv[l]);
     }
@@ -2588,7 +2593,8 @@ sipg_status sipg_fma_peak(int precision, void *stream, double *flops) {
 // graph, the branches of different problems side by side.
 struct BLaunch {
   int kind;     // 0 vector op over DG points, 1 over FE nodes, 2 DG evaluation, 3 DG integration,
-                // 4 FE cell pass, 5 FE node pass, 6 c-prolongation, 7 the per-problem branches
+                // 4 FE cell pass (or the one pass), 5 FE node pass, 6 c-prolongation, 7 the per-problem branches,
+                // 8 FE node pass of the problems whose operator takes two passes
   size_t off;   // the launch's first task in its task array (one task per problem)
 };
 
@@ -2597,17 +2603,18 @@ struct BatchCycle {
   int np = 0;
   bool curved = false;
   BatchPlan<T> dg;                        // DG work items of the finest levels
-  // FE items, degree by degree: groups of cells, or (axis-aligned cells) bricks,
-  // each problem's own
+  // FE items, degree by degree: bricks of the problems whose operator is one
+  // pass, groups of cells of the others
   WorkItem *fe_items = nullptr;
   struct FEDegree {
     int n, first, count;
+    bool bricks;
     size_t smem;   // bricks
   };
   std::vector<std::array<int, 3>> brick;
   std::vector<FEDegree> fe_degrees;
-  NodeItem *items_d = nullptr, *items_g = nullptr;   // DG points, FE nodes
-  int n_d = 0, n_g = 0;
+  NodeItem *items_d = nullptr, *items_g = nullptr, *items_n = nullptr;   // DG points, FE nodes, those of kind 8
+  int n_d = 0, n_g = 0, n_n = 0;
   VecTask *vec = nullptr;
   BatchProb<T> *dgt = nullptr;
   FETask<T> *fet = nullptr;
@@ -2619,7 +2626,7 @@ struct BatchCycle {
   ~BatchCycle() {
     if (graph) cudaGraphExecDestroy(graph);
     batch_plan_free(dg);
-    for (void *q : {(void *)fe_items, (void *)items_d, (void *)items_g, (void *)vec, (void *)dgt, (void *)fet})
+    for (void *q : {(void *)fe_items, (void *)items_d, (void *)items_g, (void *)items_n, (void *)vec, (void *)dgt, (void *)fet})
       cudaFree(q);
   }
 };
@@ -2936,12 +2943,15 @@ void batch_cycle_emit(sipg_batch *B, BatchCycle<T> &C, cudaStream_t s) {
       case 4:
         for (const auto &d : C.fe_degrees) {
           const WorkItem *it = C.fe_items + d.first;
-          if (C.curved) CK(launch_fe_cells_batched<T>(d.n, C.fet + r.off, it, d.count, segs, br.of(d.n)));
-          else CK(launch_fe_box_batched<T>(d.n, C.fet + r.off, it, d.count, d.smem, segs, br.of(d.n)));
+          if (d.bricks) CK(launch_fe_box_batched<T>(d.n, C.fet + r.off, it, d.count, d.smem, segs, br.of(d.n)));
+          else CK(launch_fe_cells_batched<T>(d.n, C.curved, C.fet + r.off, it, d.count, segs, br.of(d.n)));
         }
         break;
       case 5:
         CK(launch_fe_nodes_batched<T>(C.fet + r.off, C.items_g, C.n_g, segs, 0, s));
+        break;
+      case 8:
+        CK(launch_fe_nodes_batched<T>(C.fet + r.off, C.items_n, C.n_n, segs, 0, s));
         break;
       case 6:
         CK(launch_fe_nodes_batched<T>(C.fet + r.off, C.items_d, C.n_d, segs, 1, s));
@@ -2996,7 +3006,7 @@ std::unique_ptr<BatchCycle<T>> batch_cycle_build(sipg_batch *B) {
   std::vector<DGArgs<T>> a0;
   std::vector<int> nn;
   std::vector<WorkItem> fei;
-  std::vector<NodeItem> nd, ng;
+  std::vector<NodeItem> nd, ng, nn8;
   // a problem of at least kSoloDofs DoF keeps its own cycle (its launches
   // fill the GPU; in lockstep with small problems it would wait for their
   // lower levels at every shared step)
@@ -3013,16 +3023,20 @@ std::unique_ptr<BatchCycle<T>> batch_cycle_build(sipg_batch *B) {
       continue;
     }
     for (int64_t q = 0; q * kBatchNodeThreads < D.ndofs; ++q) nd.push_back({p, (int)q});
-    for (int64_t q = 0; q * kBatchNodeThreads < F.ndofs; ++q) ng.push_back({p, (int)q});
+    for (int64_t q = 0; q * kBatchNodeThreads < F.ndofs; ++q) {
+      ng.push_back({p, (int)q});
+      if (!one_pass_fe<T>(F)) nn8.push_back(ng.back());
+    }
   }
   CK(batch_plan_build<T>(C->dg, a0, nn, C->curved));
   C->brick.assign(np, {1, 1, 1});
-  for (int n = kMaxN; n >= 2; --n) {   // bricks: full ones (the problems together fill the GPU)
-    typename BatchCycle<T>::FEDegree d{n, (int)fei.size(), 0, 0};
+  for (int k = 0; k < 2 * (kMaxN - 1); ++k) {   // bricks: full ones (the problems together fill the GPU)
+    const int n = kMaxN - k / 2;
+    typename BatchCycle<T>::FEDegree d{n, (int)fei.size(), 0, k % 2 == 1, 0};
     for (int p = 0; p < np; ++p) {
       const Level &F = B->ctx[p]->lv[B->ctx[p]->L - 1];
-      if (C->solo[p] || F.n != n) continue;
-      if (C->curved) {
+      if (C->solo[p] || F.n != n || one_pass_fe<T>(F) != d.bricks) continue;
+      if (!d.bricks) {
         const int cb = kBatchCellThreads / (n * n);
         for (int q = 0; q < F.ncells; q += cb) fei.push_back({p, q, (int)std::min<int64_t>(cb, F.ncells - q)});
         continue;
@@ -3038,6 +3052,7 @@ std::unique_ptr<BatchCycle<T>> batch_cycle_build(sipg_batch *B) {
   }
   C->n_d = (int)nd.size();
   C->n_g = (int)ng.size();
+  C->n_n = (int)nn8.size();
   // the program, task by task
   std::vector<VecTask> hv;
   std::vector<BatchProb<T>> hd;
@@ -3065,10 +3080,9 @@ std::unique_ptr<BatchCycle<T>> batch_cycle_build(sipg_batch *B) {
       hd.push_back(q);
     }
   };
-  auto fetask = [&](int kind, auto args) {   // kind 4: cell and node pass; 5: node pass; 6: c-prolongation
-    if (kind == 4) C->prog.push_back({4, hf.size()});
-    // axis-aligned cells: 4 is the whole operator
-    if (kind != 4 || C->curved) C->prog.push_back({kind == 4 ? 5 : kind, hf.size()});
+  auto fetask = [&](int kind, auto args) {   // kind 4: the operator; 5: node pass; 6: c-prolongation
+    C->prog.push_back({kind, hf.size()});
+    if (kind == 4 && C->n_n) C->prog.push_back({8, hf.size()});
     for (int p = 0; p < np; ++p) hf.push_back(args(p));
   };
   auto dga = [&](int p, const T *u, T *out, int mode, const T *x, const T *xp, const T *b, const ChebStep *q) {
@@ -3155,6 +3169,7 @@ std::unique_ptr<BatchCycle<T>> batch_cycle_build(sipg_batch *B) {
   C->fe_items = upload_vec(fei);
   C->items_d = upload_vec(nd);
   C->items_g = upload_vec(ng);
+  C->items_n = upload_vec(nn8);
   C->vec = upload_vec(hv);
   C->dgt = upload_vec(hd);
   C->fet = upload_vec(hf);
