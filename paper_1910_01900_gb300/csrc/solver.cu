@@ -4,7 +4,6 @@
 #include <array>
 #include <atomic>
 #include <chrono>
-#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -3030,7 +3029,30 @@ std::unique_ptr<BatchCycle<T>> batch_cycle_build(sipg_batch *B) {
   }
   CK(batch_plan_build<T>(C->dg, a0, nn, C->curved));
   C->brick.assign(np, {1, 1, 1});
-  for (int k = 0; k < 2 * (kMaxN - 1); ++k) {   // bricks: full ones (the problems together fill the GPU)
+  // Bricks as large as leave kFEBatchBricks of them to all problems together (the
+  // degrees run side by side), down to single cells: with the full bricks
+  // always, four problems of 4^3 to 8^3 cells of degrees 7 and 8 had 126 and took
+  // 772 us a cycle (FP32), with at least 140 674 us, 256 612 us; 8^3 of degree 8
+  // 635 / 442 / 440 us; more bricks cost halo arithmetic (16^3 and 12^3 of degrees
+  // 3 and 5 377 / 377 / 404, with 1200 411 us).
+  constexpr int64_t kFEBatchBricks = 256;
+  auto bricks = [&](int p) {
+    const Level &F = B->ctx[p]->lv[B->ctx[p]->L - 1];
+    int64_t nb = 1;
+    for (int e = 0; e < 3; ++e) nb *= (F.m[e] + C->brick[p][e] - 1) / C->brick[p][e];
+    return nb;
+  };
+  for (int most = 512; most >= 1; most /= 2) {
+    int64_t total = 0;
+    for (int p = 0; p < np; ++p) {
+      const Level &F = B->ctx[p]->lv[B->ctx[p]->L - 1];
+      if (C->solo[p] || !one_pass_fe<T>(F)) continue;
+      fe_box_brick<T>(F.n, F.m, most, C->brick[p].data());
+      total += bricks(p);
+    }
+    if (total >= kFEBatchBricks) break;
+  }
+  for (int k = 0; k < 2 * (kMaxN - 1); ++k) {
     const int n = kMaxN - k / 2;
     typename BatchCycle<T>::FEDegree d{n, (int)fei.size(), 0, k % 2 == 1, 0};
     for (int p = 0; p < np; ++p) {
@@ -3041,10 +3063,7 @@ std::unique_ptr<BatchCycle<T>> batch_cycle_build(sipg_batch *B) {
         for (int q = 0; q < F.ncells; q += cb) fei.push_back({p, q, (int)std::min<int64_t>(cb, F.ncells - q)});
         continue;
       }
-      fe_box_brick<T>(n, F.m, INT_MAX, C->brick[p].data());
-      int nb = 1;
-      for (int e = 0; e < 3; ++e) nb *= (F.m[e] + C->brick[p][e] - 1) / C->brick[p][e];
-      for (int q = 0; q < nb; ++q) fei.push_back({p, q, 0});
+      for (int q = 0; q < bricks(p); ++q) fei.push_back({p, q, 0});
       d.smem = std::max(d.smem, (size_t)fe_box_values(F.deg, C->brick[p].data()) * sizeof(T));
     }
     d.count = (int)fei.size() - d.first;
