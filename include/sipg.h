@@ -229,7 +229,7 @@ sipg_status sipg_l2_error(sipg_ctx *ctx, int kind, const double *x_dev, double *
 sipg_status sipg_operator_apply(sipg_ctx *ctx, int precision, const void *u_dev, void *v_dev);
 
 /* v = A_l u on any level (FE levels: Eq. WeakFormFE with constrained rows set
- * to the identity, Section 2), in either precision. */
+ * to the identity, Section 2), in either precision.  u and v must not overlap. */
 sipg_status sipg_level_apply(sipg_ctx *ctx, int level, int precision, const void *u_dev, void *v_dev);
 
 /* Inverse diagonal D^-1 of level l (Section 3.1), written in the level's

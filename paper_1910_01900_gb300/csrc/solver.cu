@@ -177,6 +177,13 @@ thread_local std::string *t_err = nullptr;
   throw Fail{SIPG_EINVAL};
 }
 
+// whether na bytes at a and nb bytes at b share memory.  The one-pass kernels
+// read cells (nodes) that another block writes the result of, so where a caller's
+// input may lie in the output, it is copied aside first.
+bool overlap(const void *a, int64_t na, const void *b, int64_t nb) {
+  return (const char *)a < (const char *)b + nb && (const char *)b < (const char *)a + na;
+}
+
 template <typename T>
 T *dalloc(sipg_ctx *c, int64_t n) {
   void *p = nullptr;
@@ -2275,6 +2282,12 @@ sipg_status sipg_smooth(sipg_ctx *c, int level, const void *b, void *x, int nste
 sipg_status sipg_restrict(sipg_ctx *c, int level, const void *r, void *rc) {
   if (!level_ok(c, level) || level == 0 || !r || !rc || !c->solver) return SIPG_EINVAL;
   return guarded(c, [&]() -> sipg_status {
+    const int pi = c->prm.precision, es = pi ? 4 : 8;
+    const int64_t bytes = c->lv[level].ndofs * es;
+    if (overlap(r, bytes, rc, c->lv[level - 1].ndofs * es)) {
+      CK(cudaMemcpyAsync(c->lv[level].vx[pi], r, bytes, cudaMemcpyDeviceToDevice, c->stream));
+      r = c->lv[level].vx[pi];
+    }
     if (c->prm.precision == 0)
       restrict_level<double>(c, level, (const double *)r, (double *)rc);
     else
@@ -2366,10 +2379,20 @@ sipg_status sipg_time_apply(sipg_ctx *c, int precision, const void *u, void *v, 
     cudaEvent_t ev[3];
     for (auto &e : ev) CK(cudaEventCreate(&e));
     float te = 0, ti = 0;
+    const int64_t bytes = L.ndofs * (precision ? 4 : 8);
+    struct Aside {   // u, where it lies in v (the one pass)
+      void *p = nullptr;
+      ~Aside() { cudaFree(p); }
+    } aside;
+    const void *in = u;
+    if (!L.curved && overlap(u, bytes, v, bytes)) {
+      CK(cudaMalloc(&aside.p, bytes));
+      in = aside.p;
+    }
     auto timed = [&](auto a) {
       using T = std::remove_const_t<std::remove_pointer_t<decltype(a.u)>>;
       constexpr int pi = pidx<T>();
-      a.u = (const T *)u;
+      a.u = (const T *)in;
       a.out = (T *)v;
       if (L.curved) CK(launch_dg_eval<T>(L.n, a, c->stream, L.cb[pi][0]));
       CK(cudaEventRecord(ev[1], c->stream));
@@ -2377,6 +2400,7 @@ sipg_status sipg_time_apply(sipg_ctx *c, int precision, const void *u, void *v, 
       else CK(launch_dg_box<T>(L.n, a, c->stream));
     };
     for (int r = 0; r < repeats; ++r) {
+      if (in != u) CK(cudaMemcpyAsync(aside.p, u, bytes, cudaMemcpyDeviceToDevice, c->stream));
       CK(cudaEventRecord(ev[0], c->stream));
       if (precision == 0) timed(dg_args<double>(c, L));
       else timed(dg_args<float>(c, L));
@@ -3595,6 +3619,11 @@ sipg_status sipg_operator_apply_multi(sipg_ctx *c, int precision, int nv, const 
         if (L.kind == 0 && L.curved) trace = std::max(trace, L.ncells * 12 * (int64_t)L.n * L.n);
       c->mv.trace[1] = dalloc<float>(c, trace * c->mv.cap);
     }
+    const int64_t bytes = c->lv[c->L].ndofs * nv * (precision ? 4 : 8);
+    if (!c->lv[c->L].curved && overlap(U, bytes, V, bytes)) {
+      CK(cudaMemcpyAsync(c->mv.p, U, bytes, cudaMemcpyDeviceToDevice, c->stream));
+      U = c->mv.p;
+    }
     MultiScope scope(c, nv);
     if (precision == 0)
       apply_level<double>(c, c->L, (const double *)U, (double *)V, 0);
@@ -3695,8 +3724,24 @@ sipg_status sipg_batch_apply(sipg_batch *B, const double *const *u, double *cons
   for (size_t p = 0; p < B->ctx.size(); ++p)
     if (!u[p] || !v[p] || u[p] == v[p]) return SIPG_EINVAL;
   return bguarded(B, [&]() -> sipg_status {
-    for (size_t p = 0; p < B->ctx.size(); ++p) B->segs[p].active = 1;
-    batch_set_plan(B, 0, u, v);
+    const size_t np = B->ctx.size();
+    for (size_t p = 0; p < np; ++p) B->segs[p].active = 1;
+    std::vector<const double *> in(u, u + np);
+    if (!B->plan.curved) {   // an input inside any problem's output
+      std::vector<std::pair<const double *, const double *>> out(np);
+      for (size_t p = 0; p < np; ++p) out[p] = {v[p], v[p] + B->ctx[p]->lv[B->ctx[p]->L].ndofs};
+      std::sort(out.begin(), out.end());
+      for (size_t p = 0; p < np; ++p) {
+        sipg_ctx *c = B->ctx[p];
+        const int64_t n = c->lv[c->L].ndofs;
+        // of disjoint outputs, the last that starts below u's end reaches furthest
+        auto it = std::lower_bound(out.begin(), out.end(), std::make_pair(u[p] + n, (const double *)nullptr));
+        if (it == out.begin() || !((--it)->second > u[p])) continue;
+        CK(cudaMemcpyAsync(c->fp, u[p], n * sizeof(double), cudaMemcpyDeviceToDevice, B->stream));
+        in[p] = c->fp;
+      }
+    }
+    batch_set_plan(B, 0, in.data(), v);
     batch_apply(B);
     return SIPG_OK;
   });
