@@ -9,16 +9,16 @@ namespace sipg {
 
 // the width that a setting of cb cells runs at: kCurvedThreads threads and the
 // shared memory at most
-template <typename T, int N>
-static int curved_cb(int cb) {
-  return std::min({cb, kCurvedThreads / (N * N), 232448 / (curved_cell_values(N, true) * (int)sizeof(T))});
+template <typename T>
+static int curved_cb(int n, int cb) {
+  return std::min({cb, kCurvedThreads / (n * n), 232448 / (curved_cell_values(n, true) * (int)sizeof(T))});
 }
 
 template <typename T, int N>
 static cudaError_t run_dg(bool integrate, const DGArgs<T> &a, cudaStream_t s, int cb) {
   if (cb <= 0) cb = default_cb(N);
   if (cb > max_cb(N, sizeof(T))) return cudaErrorInvalidValue;
-  cb = curved_cb<T, N>(cb);
+  cb = curved_cb<T>(N, cb);
   const size_t smem = (size_t)cb * curved_cell_values(N, integrate) * sizeof(T);
   const int64_t grid = (int64_t)((a.ncells + cb - 1) / cb) * a.nv;
   if (grid == 0) return cudaSuccess;
@@ -80,21 +80,17 @@ static cudaError_t run_dg_box(const DGArgs<T> &a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// Resident thread blocks per SM of one pass at cb cells per block.
+// Resident thread blocks per SM of one pass in blocks of groups x N^2 threads.
 template <typename T, int N>
-static cudaError_t occ_dg(bool curved, bool integrate, int cb, int *blocks) {
-  if (!curved) {
-    const int big[3] = {1 << 20, 1 << 20, 1 << 20};
-    const int groups = box_groups<T>(dg_box_shape<T>(N, big, cb));
+static cudaError_t occ_dg(bool curved, bool integrate, int groups, int *blocks) {
+  if (!curved)
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dg_box_kernel<T, N, false>, groups * N * N,
                                                          (size_t)groups * box_group_values(N) * 8);
-  }
-  cb = curved_cb<T, N>(cb);
-  const size_t smem = (size_t)cb * curved_cell_values(N, integrate) * sizeof(T);
+  const size_t smem = (size_t)groups * curved_cell_values(N, integrate) * sizeof(T);
   return integrate ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dg_integrate_kernel<T, N, false>,
-                                                                   cb * N * N, smem)
-                   : cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dg_eval_kernel<T, N, false>, cb * N * N,
-                                                                   smem);
+                                                                   groups * N * N, smem)
+                   : cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dg_eval_kernel<T, N, false>,
+                                                                   groups * N * N, smem);
 }
 
 // Opt every kernel into the shared memory of its widest block (once per
@@ -102,7 +98,7 @@ static cudaError_t occ_dg(bool curved, bool integrate, int cb, int *blocks) {
 template <typename T, int N>
 static cudaError_t prep_dg_n() {
   constexpr cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  const int smem = curved_cb<T, N>(max_cb(N, sizeof(T))) * curved_cell_values(N, true) * (int)sizeof(T);
+  const int smem = curved_cb<T>(N, max_cb(N, sizeof(T))) * curved_cell_values(N, true) * (int)sizeof(T);
   const int bsmem = std::min(232448, kCellThreads / (N * N) * box_group_values(N) * 8);
   cudaError_t e = cudaSuccess;
   for (cudaError_t r : {cudaFuncSetAttribute(dg_integrate_kernel<T, N, false>, at, smem),
@@ -148,8 +144,24 @@ static BoxShape box_shape(int n, const int m[3], int cb) {
   return b;
 }
 
+// what a width setting of cb cells (0 = default) launches on a mesh of m cells
+template <typename T>
+static TileLaunch dg_tile_launch(int n, bool curved, const int m[3], int64_t ncells, int cb) {
+  if (curved) {
+    const int c = curved_cb<T>(n, cb > 0 ? cb : default_cb(n));
+    return {c, c * n * n, (ncells + c - 1) / c};
+  }
+  const BoxShape b = box_shape<T>(n, m, cb);
+  TileLaunch t{b.bricks * b.w[0] * b.w[1] * b.w[2], box_groups<T>(b) * n * n, 1};
+  for (int d = 0; d < 3; ++d) {
+    const int w = b.w[d] * (d == 0 ? b.bricks : 1);
+    t.blocks *= (m[d] + w - 1) / w;
+  }
+  return t;
+}
+
 // op 0 evaluation, 1 integration, 2 the one pass of axis-aligned cells; 3 an
-// occupancy query of the given pass into *blocks
+// occupancy query of the given pass in blocks of cb n^2 threads into *blocks
 template <typename T>
 static cudaError_t dispatch_dg(int op, int n, const DGArgs<T> *a, cudaStream_t s, int cb, bool curved = true,
                                bool integrate = true, int *blocks = nullptr) {

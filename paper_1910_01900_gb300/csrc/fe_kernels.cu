@@ -838,7 +838,6 @@ static cudaError_t run_fe_cells(const FEArgs<T> &a, cudaStream_t s, int cb) {
 
 template <typename T, int N, bool CURVED>
 static cudaError_t occ_fe_cells(int cb, int *blocks) {
-  cb = fe_cells_cb<T, N, CURVED>(cb);
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fe_cell_kernel<T, N, CURVED, false>, cb * N * N,
                                                        (size_t)cb * kFECellValues<N, CURVED> * sizeof(T));
 }
@@ -1074,11 +1073,32 @@ int fe_max_cells_per_block(int n) {
 }
 
 template <typename T>
-cudaError_t fe_blocks_per_sm(int n, bool curved, int cb, int *blocks) {
+TileLaunch fe_tile(int n, bool curved, int64_t ncells, int cb) {
+  int c = cb > 0 ? cb : default_cb(n);
+  switch (n) {
+#define SIPG_FE_TILE(NN)                                                             \
+  case NN:                                                                           \
+    c = curved ? fe_cells_cb<T, NN, true>(c) : fe_cells_cb<T, NN, false>(c);         \
+    break;
+    SIPG_FE_TILE(2)
+    SIPG_FE_TILE(3)
+    SIPG_FE_TILE(4)
+    SIPG_FE_TILE(5)
+    SIPG_FE_TILE(6)
+    SIPG_FE_TILE(7)
+    SIPG_FE_TILE(8)
+    SIPG_FE_TILE(9)
+#undef SIPG_FE_TILE
+  }
+  return {c, c * n * n, (ncells + c - 1) / c};
+}
+
+template <typename T>
+cudaError_t fe_blocks_per_sm(int n, bool curved, int cells, int *blocks) {
 #define SIPG_FE_OCC(NN)                                                                 \
   case NN:                                                                              \
-    if (curved) return occ_fe_cells<T, NN, true>(cb, blocks);                           \
-    if constexpr (kBoxCells<T, NN>) return occ_fe_cells<T, NN, false>(cb, blocks);      \
+    if (curved) return occ_fe_cells<T, NN, true>(cells, blocks);                        \
+    if constexpr (kBoxCells<T, NN>) return occ_fe_cells<T, NN, false>(cells, blocks);   \
     return cudaErrorInvalidValue;
   switch (n) {
     SIPG_FE_OCC(2)
@@ -1536,6 +1556,7 @@ cudaError_t launch_dg_transfer(const XferGeom &g, const T *P1, const T *in, T *o
 #define SIPG_FE_INST(T)                                                                                   \
   template cudaError_t launch_fe_cells<T>(int, bool, const FEArgs<T> &, bool, cudaStream_t, int);       \
   template int fe_max_cells_per_block<T>(int);                                                          \
+  template TileLaunch fe_tile<T>(int, bool, int64_t, int);                                              \
   template cudaError_t fe_blocks_per_sm<T>(int, bool, int, int *);                                      \
   template bool fe_two_pass<T>(int, int64_t);                                                           \
   template void fe_box_brick<T>(int, const int *, int, int *);                                          \

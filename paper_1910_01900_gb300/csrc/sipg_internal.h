@@ -9,6 +9,8 @@
 
 #include "../../include/sipg.h"
 
+#include "tile_rules.h"
+
 namespace sipg {
 
 constexpr int kMaxN = 9;   // points per direction, k = 1..8
@@ -235,10 +237,13 @@ template <typename T>
 int dg_cells_per_block(int n, bool curved = true);   // curved: the cell passes' default (FE too)
 template <typename T>
 int dg_max_cells_per_block(int n);
-// resident blocks per SM of a DG pass (0 evaluation, 1 integration; on
-// axis-aligned cells 1 is the one pass) at cb cells per block
+// what a width setting (0 = default) launches on a level of ncells cells (axis-aligned: m)
 template <typename T>
-cudaError_t dg_blocks_per_sm(int n, bool curved, int pass, int cb, int *blocks);
+TileLaunch dg_tile(int n, bool curved, const int m[3], int64_t ncells, int cb);
+// resident blocks per SM of a DG pass (0 evaluation, 1 integration; on
+// axis-aligned cells 1 is the one pass) in blocks of groups n^2 threads
+template <typename T>
+cudaError_t dg_blocks_per_sm(int n, bool curved, int pass, int groups, int *blocks);
 
 cudaError_t launch_dg_diag(int n, bool curved, const DGArgs<double> &a, double *diag, cudaStream_t s);
 
@@ -249,7 +254,9 @@ cudaError_t launch_fe_cells(int n, bool curved, const FEArgs<T> &a, bool diag_on
 template <typename T>
 int fe_max_cells_per_block(int n);
 template <typename T>
-cudaError_t fe_blocks_per_sm(int n, bool curved, int cb, int *blocks);
+TileLaunch fe_tile(int n, bool curved, int64_t ncells, int cb);
+template <typename T>
+cudaError_t fe_blocks_per_sm(int n, bool curved, int cells, int *blocks);
 // whether an axis-aligned level takes the cell and node passes (else the one pass)
 template <typename T>
 bool fe_two_pass(int n, int64_t cells);

@@ -855,9 +855,7 @@ void alloc_work(sipg_ctx *c, Level &L) {
 // Tile-shape autotuner.  A cell kernel's block width cb (cells per block)
 // fixes how many cells an SM holds at once (the occupancy calculator's
 // resident blocks times cb) and hence how full the last wave of blocks is.
-// The candidates are the widths whose waves leave the fewest cell slots
-// idle (weighted by the share of live lanes in the block's last warp), plus
-// the compiled default; each is timed on the level and the fastest kept.
+// The candidates (pick_widths) are each timed on the level and the fastest kept.
 // Results are cached per (n, geometry, precision, pass, cells) for the
 // process, so contexts and batch members of equal shape tune once.
 std::mutex g_tune_mu;
@@ -868,25 +866,19 @@ std::vector<int> tile_candidates(const Level &L, int pass, int keep) {
   int dev = 0, nsm = 0;
   CK(cudaGetDevice(&dev));
   CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  const int maxcb = pass < 2 ? dg_max_cells_per_block<T>(L.n) : fe_max_cells_per_block<T>(L.n);
-  std::vector<std::pair<double, int>> score;
-  for (int cb = 1; cb <= maxcb; ++cb) {
-    int occ = 0;
-    CK(pass < 2 ? dg_blocks_per_sm<T>(L.n, L.curved, pass, cb, &occ) : fe_blocks_per_sm<T>(L.n, L.curved, cb, &occ));
-    if (occ <= 0) continue;
-    const int threads = cb * L.n * L.n;
-    const double lanes = threads / (32.0 * ((threads + 31) / 32));
-    const int64_t slots = (int64_t)occ * nsm, groups = (L.ncells + cb - 1) / cb;
-    const int64_t waves = (groups + slots - 1) / slots;
-    score.push_back({(double)L.ncells / ((double)waves * slots * cb) * lanes, cb});
-  }
-  std::stable_sort(score.begin(), score.end(), [](const auto &x, const auto &y) { return x.first > y.first; });
-  std::vector<int> out{dg_cells_per_block<T>(L.n, L.kind != 0 || L.curved)};
-  for (const auto &sc : score) {
-    if ((int)out.size() > keep) break;
-    if (std::find(out.begin(), out.end(), sc.second) == out.end()) out.push_back(sc.second);
-  }
-  return out;
+  const int most = pass < 2 ? dg_max_cells_per_block<T>(L.n) : fe_max_cells_per_block<T>(L.n);
+  return pick_widths(
+      L.cb0[pidx<T>()][pass], most, L.ncells, nsm, keep,
+      [&](int cb) {
+        return pass < 2 ? dg_tile<T>(L.n, L.curved, L.m, L.ncells, cb) : fe_tile<T>(L.n, L.curved, L.ncells, cb);
+      },
+      [&](const TileLaunch &t) {
+        int occ = 0;
+        const int groups = t.threads / (L.n * L.n);
+        CK(pass < 2 ? dg_blocks_per_sm<T>(L.n, L.curved, pass, groups, &occ)
+                    : fe_blocks_per_sm<T>(L.n, L.curved, groups, &occ));
+        return occ;
+      });
 }
 
 template <typename T>
@@ -1005,6 +997,8 @@ void default_tile_widths(sipg_ctx *c) {
         const bool box = L.kind == 0 && !L.curved;
         int cb = pi ? dg_cells_per_block<float>(L.n, !box) : dg_cells_per_block<double>(L.n, !box);
         if (nsm > 0 && (L.ncells + cb - 1) / cb < nsm) cb = (int)std::max<int64_t>(1, (L.ncells + nsm - 1) / nsm);
+        if (box)   // the cells of the block that this gives
+          cb = (pi ? dg_tile<float>(L.n, false, L.m, L.ncells, cb) : dg_tile<double>(L.n, false, L.m, L.ncells, cb)).cells;
         L.cb[pi][pass] = L.cb0[pi][pass] = cb;
       }
   for (Level &L : c->lv) set_box(L);

@@ -1,0 +1,45 @@
+// Which widths (cells per thread block) of a cell kernel are worth timing.
+#pragma once
+#include <algorithm>
+#include <cstdint>
+#include <utility>
+#include <vector>
+
+namespace sipg {
+
+// What a width setting launches on a level: the kernels round it to what they
+// lay out (a thread limit, bricks of cells), so several settings are one launch.
+struct TileLaunch {
+  int cells, threads;   // of a block
+  int64_t blocks;       // of the level
+  bool operator==(const TileLaunch &o) const {
+    return cells == o.cells && threads == o.threads && blocks == o.blocks;
+  }
+};
+
+// The launch of the level's default setting, then up to keep others among the
+// settings 1 .. most whose waves of blocks leave the fewest cell slots idle,
+// weighted by the share of live lanes in the block's last warp; each launch once,
+// named by the cells its blocks take (which as a setting gives it again).
+// launch(cb): the TileLaunch of a setting; resident(t): its blocks per SM.
+template <typename Launch, typename Resident>
+std::vector<int> pick_widths(int standard, int most, int64_t ncells, int nsm, int keep, Launch launch, Resident resident) {
+  std::vector<TileLaunch> seen{launch(standard)};
+  std::vector<std::pair<double, int>> score;
+  for (int cb = 1; cb <= most; ++cb) {
+    const TileLaunch t = launch(cb);
+    if (std::find(seen.begin(), seen.end(), t) != seen.end()) continue;
+    seen.push_back(t);
+    const int64_t slots = (int64_t)resident(t) * nsm;
+    if (slots <= 0) continue;
+    const int64_t waves = (t.blocks + slots - 1) / slots;
+    const double lanes = t.threads / (32.0 * ((t.threads + 31) / 32));
+    score.push_back({(double)ncells / ((double)waves * slots * t.cells) * lanes, t.cells});
+  }
+  std::stable_sort(score.begin(), score.end(), [](const auto &x, const auto &y) { return x.first > y.first; });
+  std::vector<int> out{seen[0].cells};
+  for (size_t i = 0; i < score.size() && (int)i < keep; ++i) out.push_back(score[i].second);
+  return out;
+}
+
+}  // namespace sipg

@@ -1,0 +1,77 @@
+"""The autotuner's candidates are distinct launches (CPU; the rules alone, compiled with nvcc).
+
+Width settings (cells per block) are rounded to what a kernel lays out: curved
+passes to 512 threads, axis-aligned ones to bricks of cells.  Every candidate has
+to be another launch than the others, named by the cells that its blocks take,
+and that number as a setting has to give the launch again.
+"""
+import itertools
+import json
+import subprocess
+
+import pytest
+
+from paper_1910_01900_gb300 import build
+from paper_1910_01900_gb300.csrc_info import max_cells_per_block
+
+MESHES = [(4, 4, 4), (64, 64, 1), (16, 16, 16), (1, 7, 33), (5, 4, 6), (32, 31, 30)]
+KEEP = 4
+MAIN = r"""
+#include <cstdio>
+#include "dg_launch.cuh"
+using namespace sipg;
+template <typename T>
+void run(int n, bool curved, const int (&m)[3]) {
+  const int64_t cells = (int64_t)m[0] * m[1] * m[2];
+  const int most = max_cb(n, sizeof(T));
+  auto launch = [&](int cb) { return dg_tile_launch<T>(n, curved, m, cells, cb); };
+  printf("{\"key\": [%d, %d, %d, %d, %d, %d], \"widths\": [", (int)sizeof(T), n, (int)curved, m[0], m[1], m[2]);
+  const char *c = "";
+  for (int w : pick_widths(0, most, cells, 152, KEEP, launch, [&](const TileLaunch &t) { return 2048 / t.threads; }))
+    printf("%s%d", c, w), c = ", ";
+  printf("], \"launch\": [");
+  c = "";
+  for (int cb = 0; cb <= most; ++cb) {
+    const TileLaunch t = launch(cb);
+    printf("%s[%d, %d, %lld]", c, t.cells, t.threads, (long long)t.blocks), c = ", ";
+  }
+  printf("]}\n");
+}
+int main() {
+  const int meshes[][3] = MESHES;
+  for (int n = 2; n <= 9; ++n)
+    for (int curved = 0; curved < 2; ++curved)
+      for (auto &m : meshes) run<float>(n, curved, m), run<double>(n, curved, m);
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def rules(tmp_path_factory):
+    try:
+        nvcc = build._nvcc()
+    except RuntimeError:
+        pytest.skip("no nvcc")
+    d = tmp_path_factory.mktemp("rules")
+    src = MAIN.replace("MESHES", "{%s}" % ", ".join("{%d, %d, %d}" % m for m in MESHES)).replace("KEEP", str(KEEP))
+    (d / "main.cu").write_text(src)
+    subprocess.run([nvcc] + build.ARCH + ["-std=c++17", "-I", build.CSRC, str(d / "main.cu"), "-o", str(d / "main")],
+                   check=True, capture_output=True)
+    out = subprocess.run([str(d / "main")], check=True, capture_output=True, text=True).stdout
+    return {tuple(r["key"]): r for r in map(json.loads, out.splitlines())}
+
+
+@pytest.mark.parametrize("n,elem,curved", list(itertools.product(range(2, 10), (4, 8), (0, 1))))
+def test_candidates_are_distinct_launches(rules, n, elem, curved):
+    for m in MESHES:
+        r = rules[(elem, n, curved) + m]
+        launches = [tuple(t) for t in r["launch"]]   # of the settings 0 (default), 1, 2, ...
+        assert len(launches) == max_cells_per_block(n, elem) + 1
+        for setting, (cells, threads, blocks) in enumerate(launches):
+            assert cells <= max(setting or cells, 2 if elem == 4 and not curved else 1)
+            assert threads == cells * n * n // (1 if curved or elem == 8 else 2)
+            assert blocks * cells >= m[0] * m[1] * m[2]
+            assert launches[cells] == (cells, threads, blocks)
+        widths = r["widths"]
+        assert widths[0] == launches[0][0]
+        assert len(set(launches[w] for w in widths)) == len(widths) == min(KEEP + 1, len(set(launches)))
