@@ -120,8 +120,8 @@ typedef struct {
                               fastest; the
                               candidates are the widths whose last wave of
                               blocks leaves the fewest cell slots idle;
-                              cached per (degree, geometry, cells) for the
-                              process                                      */
+                              cached per (degree, geometry, mesh; curved:
+                              number of cells) for the process             */
   int fe_assemble;         /* FE levels of degree <= fe_assemble (0..3;
                               default 1) apply an assembled (2p+1)^3-point
                               stencil built at setup from the same element

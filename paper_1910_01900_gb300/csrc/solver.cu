@@ -13,7 +13,6 @@
 #include <mutex>
 #include <stdexcept>
 #include <string>
-#include <tuple>
 #include <type_traits>
 
 #include "geometry.h"
@@ -856,10 +855,9 @@ void alloc_work(sipg_ctx *c, Level &L) {
 // fixes how many cells an SM holds at once (the occupancy calculator's
 // resident blocks times cb) and hence how full the last wave of blocks is.
 // The candidates (pick_widths) are each timed on the level and the fastest kept.
-// Results are cached per (n, geometry, precision, pass, cells) for the
-// process, so contexts and batch members of equal shape tune once.
+// Results are cached per (n, geometry, precision, pass, mesh) for the process, so contexts and batch members of equal shape tune once.
 std::mutex g_tune_mu;
-std::map<std::tuple<int, int, int, int, int64_t>, int> g_tune;
+std::map<std::array<int64_t, 8>, int> g_tune;   // by tune_key
 
 template <typename T>
 std::vector<int> tile_candidates(const Level &L, int pass, int keep) {
@@ -885,7 +883,7 @@ template <typename T>
 void autotune_level(sipg_ctx *c, int l, int pass) {
   constexpr int pi = pidx<T>();
   Level &L = c->lv[l];
-  const auto key = std::make_tuple(L.n, (int)L.curved, pi, pass, L.ncells);
+  const auto key = tune_key(L.n, L.curved, pi, pass, L.ncells, L.m);
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune.find(key);

@@ -1,6 +1,7 @@
 // Which widths (cells per thread block) of a cell kernel are worth timing.
 #pragma once
 #include <algorithm>
+#include <array>
 #include <cstdint>
 #include <utility>
 #include <vector>
@@ -16,6 +17,15 @@ struct TileLaunch {
     return cells == o.cells && threads == o.threads && blocks == o.blocks;
   }
 };
+
+// What a timed choice depends on.  The blocks of axis-aligned cells are cut from
+// the mesh's sides (64 x 64 x 1 and 16^3 cells take other bricks), the others
+// from the cells in a row.
+inline std::array<int64_t, 8> tune_key(int n, bool curved, int precision, int pass, int64_t ncells, const int m[3]) {
+  std::array<int64_t, 8> k{n, curved, precision, pass, ncells, 0, 0, 0};
+  for (int d = 0; d < 3; ++d) k[5 + d] = curved ? 0 : m[d];
+  return k;
+}
 
 // The launch of the level's default setting, then up to keep others among the
 // settings 1 .. most whose waves of blocks leave the fewest cell slots idle,

@@ -75,3 +75,24 @@ def test_candidates_are_distinct_launches(rules, n, elem, curved):
         widths = r["widths"]
         assert widths[0] == launches[0][0]
         assert len(set(launches[w] for w in widths)) == len(widths) == min(KEEP + 1, len(set(launches)))
+
+
+def test_tuned_widths_of_one_mesh_are_not_another_meshes(tmp_path):
+    """Axis-aligned blocks depend on the mesh's sides, curved ones on the number of cells alone."""
+    try:
+        nvcc = build._nvcc()
+    except RuntimeError:
+        pytest.skip("no nvcc")
+    (tmp_path / "key.cpp").write_text("""
+#include "tile_rules.h"
+int main() {
+  const int a[3] = {64, 64, 1}, b[3] = {16, 16, 16}, c[3] = {1, 64, 64};
+  auto key = [](bool curved, const int *m) { return sipg::tune_key(4, curved, 1, 1, 4096, m); };
+  const bool ok = key(false, a) != key(false, b) && key(false, a) != key(false, c) && key(false, b) == key(false, b) &&
+                  key(true, a) == key(true, b) && key(true, b) != key(false, b);
+  return ok ? 0 : 1;
+}
+""")
+    subprocess.run([nvcc, "-std=c++17", "-I", build.CSRC, str(tmp_path / "key.cpp"), "-o", str(tmp_path / "key")],
+                   check=True, capture_output=True)
+    assert subprocess.run([str(tmp_path / "key")]).returncode == 0
