@@ -432,7 +432,8 @@ sipg_status sipg_mlp_features(sipg_ctx *ctx, const double *r_dev, float *feat_de
 /* Cells per thread block a cell kernel of a level uses in the given
  * precision (pass 0 DG evaluation, 1 DG integration on a DG level; 2 the FE
  * cell pass on an FE level; on axis-aligned cells pass 1 is the whole DG
- * operator, pass 0 is unused, and the FE pass takes its bricks from the mesh):
+ * operator, pass 0 is unused, and the FE operator takes bricks of cells cut
+ * from the mesh's sides; FP64 levels may take the cell pass instead):
  * a set value, else the autotuned width or the default (about 256 threads per
  * block, fewer cells per block on meshes that would otherwise give fewer blocks
  * than the GPU has SMs), those two as the cells that a block takes.  EINVAL for
@@ -440,8 +441,8 @@ sipg_status sipg_mlp_features(sipg_ctx *ctx, const double *r_dev, float *feat_de
 sipg_status sipg_tile_shape(const sipg_ctx *ctx, int level, int precision, int pass, int *cells_per_block);
 
 /* Sets that width, the most cells of a block (0 = the default above; at most
- * 768 threads of n^2 per cell, n = degree + 1, and 227 KB of shared memory, else
- * EINVAL).  A pass runs at the widest block within it that it lays out: the DG passes on
+ * 768 threads of n^2 per cell, n = degree + 1, and 227 KB of shared memory, or
+ * the default's own number, else EINVAL).  A pass runs at the widest block within it that it lays out: the DG passes on
  * curved cells at most 512 threads, axis-aligned cells bricks of 1 or 2 cells per
  * direction side by side (FP32: at least a pair).  The results do not depend on
  * it: every cell is computed by the same threads in the same order.  Drops

@@ -264,6 +264,54 @@ __host__ __device__ constexpr int fe_box_threads(int) { return sizeof(T) == 8 ? 
 template <typename T>
 __host__ __device__ constexpr int fe_box_blocks(int n) { return sizeof(T) == 8 ? 1 : (n <= 5 ? 4 : 3); }
 
+// Cells per direction of a brick.  kFEBoxBrick[p]: about 16 own nodes along x
+// and y and 8 along z, where a thin brick's tiles leave room for more blocks
+// per SM (FP32 smoothing step on 32^3 cells of degree 4: 27.2 us for 4 x 4 x 2
+// against 36.7 us for 4 x 4 x 4 and 35.3 us for 2 x 2 x 2).  Where that gives
+// fewer bricks than the GPU can use, the side of most cells is halved until it
+// does: FP32 below 140 bricks (16^3 of degree 4: 128 bricks 14.4 us, 256 12.9
+// us), FP64, where the halo's arithmetic costs more, below 100 (50 us against
+// 61 us) and at degree 1, where it costs little, below 200 (16^3: 128 bricks 10.3
+// us, 256 8.5 us, in two passes 9.5 us).  cb > 0: the first brick of that sequence
+// with at most cb cells.  Sides are evened out over the bricks of a direction.
+constexpr int kFEBoxBrick[kMaxN][3] = {{1, 1, 1}, {16, 8, 4}, {8, 4, 4}, {5, 4, 2}, {4, 4, 2},
+                                       {4, 2, 2}, {3, 2, 2},  {2, 2, 2}, {2, 2, 2}};
+constexpr int kFEBoxSmem = 96 * 1024;   // degree 8 in FP32: 85 KB
+template <typename T>
+static void fe_box_brick(int n, const int m[3], int cb, int brick[3]) {
+  const int p = n - 1, least = sizeof(T) == 4 ? 140 : (p == 1 ? 200 : 100);
+  int b[3] = {kFEBoxBrick[p][0], kFEBoxBrick[p][1], kFEBoxBrick[p][2]};
+  for (;;) {
+    int64_t bricks = 1;
+    for (int d = 0; d < 3; ++d) {
+      const int k = (m[d] + b[d] - 1) / b[d];
+      brick[d] = (m[d] + k - 1) / k;
+      bricks *= k;
+    }
+    int d = 2;
+    for (int e : {1, 0})
+      if (b[e] > b[d]) d = e;
+    if (b[d] == 1 || (cb > 0 ? brick[0] * brick[1] * brick[2] <= cb : bricks >= least)) break;
+    b[d] = (b[d] + 1) / 2;
+  }
+}
+
+// the launch of a brick: one round of the widest stage's lines, or two of half
+// its width
+template <typename T>
+static TileLaunch fe_box_launch(int n, const int m[3], const int brick[3]) {
+  TileLaunch t{brick[0] * brick[1] * brick[2], 0, 1};
+  int w[3];
+  for (int d = 0; d < 3; ++d) {
+    t.blocks *= (m[d] + brick[d] - 1) / brick[d];
+    w[d] = (brick[d] + 1 < m[d] ? brick[d] + 1 : m[d]) * (n - 1) + 1;
+  }
+  const int a = w[0] * w[1], b = w[1] * (brick[2] * (n - 1) + 1), lines = a > b ? a : b, rounds = lines > 256 ? 2 : 1;
+  t.threads = ((lines + rounds - 1) / rounds + 31) / 32 * 32;
+  if (t.threads > fe_box_threads<T>(n)) t.threads = fe_box_threads<T>(n);
+  return t;
+}
+
 template <typename T, int N>
 __global__ void __launch_bounds__(fe_box_threads<T>(N), fe_box_blocks<T>(N)) fe_box_kernel(const FEArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -842,56 +842,20 @@ static cudaError_t occ_fe_cells(int cb, int *blocks) {
                                                        (size_t)cb * kFECellValues<N, CURVED> * sizeof(T));
 }
 
-// Cells per direction of a brick.  kFEBoxBrick[p]: about 16 own nodes along x
-// and y and 8 along z, where a thin brick's tiles leave room for more blocks
-// per SM (FP32 smoothing step on 32^3 cells of degree 4: 27.2 us for 4 x 4 x 2
-// against 36.7 us for 4 x 4 x 4 and 35.3 us for 2 x 2 x 2).  Where that gives
-// fewer bricks than the GPU can use, the side of most cells is halved until it
-// does: FP32 below 140 bricks (16^3 of degree 4: 128 bricks 14.4 us, 256 12.9
-// us), FP64, where the halo's arithmetic costs more, below 100 (50 us against
-// 61 us) and at degree 1, where it costs little, below 200 (16^3: 128 bricks 10.3
-// us, 256 8.5 us, in two passes 9.5 us).  cb > 0: at most cb cells in all.  Sides are evened out over the
-// bricks of a direction.
-constexpr int kFEBoxBrick[kMaxN][3] = {{1, 1, 1}, {16, 8, 4}, {8, 4, 4}, {5, 4, 2}, {4, 4, 2},
-                                       {4, 2, 2}, {3, 2, 2},  {2, 2, 2}, {2, 2, 2}};
-constexpr int kFEBoxSmem = 96 * 1024;   // degree 8 in FP32: 85 KB
-template <typename T>
-void fe_box_brick(int n, const int m[3], int cb, int brick[3]) {
-  const int p = n - 1, least = sizeof(T) == 4 ? 140 : (p == 1 ? 200 : 100);
-  int b[3] = {kFEBoxBrick[p][0], kFEBoxBrick[p][1], kFEBoxBrick[p][2]};
-  for (;;) {
-    int64_t bricks = 1;
-    for (int d = 0; d < 3; ++d) bricks *= (m[d] + b[d] - 1) / b[d];
-    int d = 2;
-    for (int e : {1, 0})
-      if (b[e] > b[d]) d = e;
-    if (b[d] == 1 || (cb > 0 ? b[0] * b[1] * b[2] <= cb : bricks >= least)) break;
-    b[d] = (b[d] + 1) / 2;
-  }
-  for (int d = 0; d < 3; ++d) {
-    const int k = (m[d] + b[d] - 1) / b[d];
-    brick[d] = (m[d] + k - 1) / k;
-  }
-}
-
 template <typename T, int N>
 static cudaError_t run_fe_box(const FEArgs<T> &a, cudaStream_t s) {
-  int64_t blocks = 1;
-  int w[3];
-  for (int d = 0; d < 3; ++d) {
-    blocks *= (a.m[d] + a.brick[d] - 1) / a.brick[d];
-    w[d] = std::min(a.brick[d] + 1, a.m[d]) * (N - 1) + 1;
-  }
-  const int lines = std::max(w[0] * w[1], w[1] * (a.brick[2] * (N - 1) + 1));
-  if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
+  const TileLaunch t = fe_box_launch<T>(N, a.m, a.brick);
+  if (t.blocks > 0x7fffffff) return cudaErrorInvalidValue;
   const size_t smem = fe_box_values(N - 1, a.brick) * sizeof(T);
   if (smem > (size_t)kFEBoxSmem) return cudaErrorInvalidValue;
-  // one round of the widest stage's lines, or two of half its width
-  const int rounds = lines > 256 ? 2 : 1;
-  const int threads = std::min(fe_box_threads<T>(N), ((lines + rounds - 1) / rounds + 31) / 32 * 32);
-  fe_box_kernel<T, N><<<dim3((unsigned)blocks, a.nv), threads, smem, s>>>(a);
+  fe_box_kernel<T, N><<<dim3((unsigned)t.blocks, a.nv), t.threads, smem, s>>>(a);
   note_launch();
   return cudaGetLastError();
+}
+
+template <typename T>
+void fe_level_brick(int n, const int m[3], int cb, int brick[3]) {
+  fe_box_brick<T>(n, m, cb, brick);
 }
 
 template <typename T>
@@ -1073,7 +1037,12 @@ int fe_max_cells_per_block(int n) {
 }
 
 template <typename T>
-TileLaunch fe_tile(int n, bool curved, int64_t ncells, int cb) {
+TileLaunch fe_tile(int n, bool curved, const int m[3], int64_t ncells, int cb) {
+  if (!curved && !fe_two_pass<T>(n, ncells)) {
+    int b[3];
+    fe_box_brick<T>(n, m, cb, b);
+    return fe_box_launch<T>(n, m, b);
+  }
   int c = cb > 0 ? cb : default_cb(n);
   switch (n) {
 #define SIPG_FE_TILE(NN)                                                             \
@@ -1556,10 +1525,10 @@ cudaError_t launch_dg_transfer(const XferGeom &g, const T *P1, const T *in, T *o
 #define SIPG_FE_INST(T)                                                                                   \
   template cudaError_t launch_fe_cells<T>(int, bool, const FEArgs<T> &, bool, cudaStream_t, int);       \
   template int fe_max_cells_per_block<T>(int);                                                          \
-  template TileLaunch fe_tile<T>(int, bool, int64_t, int);                                              \
+  template TileLaunch fe_tile<T>(int, bool, const int *, int64_t, int);                                 \
   template cudaError_t fe_blocks_per_sm<T>(int, bool, int, int *);                                      \
   template bool fe_two_pass<T>(int, int64_t);                                                           \
-  template void fe_box_brick<T>(int, const int *, int, int *);                                          \
+  template void fe_level_brick<T>(int, const int *, int, int *);                                        \
   template cudaError_t launch_fe_box<T>(const FEArgs<T> &, cudaStream_t);                               \
   template cudaError_t launch_fe_gather<T>(const FEArgs<T> &, cudaStream_t);                            \
   template cudaError_t launch_fe_stencil_apply<T>(const FEArgs<T> &, const T *, cudaStream_t);          \

@@ -253,8 +253,9 @@ template <typename T>
 cudaError_t launch_fe_cells(int n, bool curved, const FEArgs<T> &a, bool diag_only, cudaStream_t s, int cb = 0);
 template <typename T>
 int fe_max_cells_per_block(int n);
+// what a width setting (0 = default) launches
 template <typename T>
-TileLaunch fe_tile(int n, bool curved, int64_t ncells, int cb);
+TileLaunch fe_tile(int n, bool curved, const int m[3], int64_t ncells, int cb);
 template <typename T>
 cudaError_t fe_blocks_per_sm(int n, bool curved, int cells, int *blocks);
 // whether an axis-aligned level takes the cell and node passes (else the one pass)
@@ -265,7 +266,7 @@ template <typename T>
 cudaError_t launch_fe_box(const FEArgs<T> &a, cudaStream_t s);
 // its brick of at most cb cells (0: the default) for a mesh of m cells
 template <typename T>
-void fe_box_brick(int n, const int m[3], int cb, int brick[3]);
+void fe_level_brick(int n, const int m[3], int cb, int brick[3]);
 // values of shared memory of a brick of b cells of degree p (two tiles)
 __host__ __device__ inline int64_t fe_box_values(const int p, const int b[3]) {
   return 2 * (int64_t)(((b[0] + 1) * p + 1) | 1) * ((b[1] + 1) * p + 1) * (b[2] * p + 1);

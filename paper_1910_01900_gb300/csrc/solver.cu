@@ -868,7 +868,7 @@ std::vector<int> tile_candidates(const Level &L, int pass, int keep) {
   return pick_widths(
       L.cb0[pidx<T>()][pass], most, L.ncells, nsm, keep,
       [&](int cb) {
-        return pass < 2 ? dg_tile<T>(L.n, L.curved, L.m, L.ncells, cb) : fe_tile<T>(L.n, L.curved, L.ncells, cb);
+        return pass < 2 ? dg_tile<T>(L.n, L.curved, L.m, L.ncells, cb) : fe_tile<T>(L.n, L.curved, L.m, L.ncells, cb);
       },
       [&](const TileLaunch &t) {
         int occ = 0;
@@ -972,9 +972,9 @@ void init_device_tables() {
 // the block shapes of an axis-aligned level for its widths
 void set_box(Level &L) {
   if (L.curved) return;
-  if (L.kind == 1) {   // cb0 stands for the rule that fits the mesh
-    fe_box_brick<double>(L.n, L.m, L.cb[0][2] == L.cb0[0][2] ? 0 : L.cb[0][2], L.brick[0]);
-    fe_box_brick<float>(L.n, L.m, L.cb[1][2] == L.cb0[1][2] ? 0 : L.cb[1][2], L.brick[1]);
+  if (L.kind == 1) {   // (a level in two passes has no brick)
+    fe_level_brick<double>(L.n, L.m, L.cb[0][2], L.brick[0]);
+    fe_level_brick<float>(L.n, L.m, L.cb[1][2], L.brick[1]);
     return;
   }
   L.box[0] = dg_box_shape<double>(L.n, L.m, L.cb[0][1]);
@@ -997,6 +997,8 @@ void default_tile_widths(sipg_ctx *c) {
         if (nsm > 0 && (L.ncells + cb - 1) / cb < nsm) cb = (int)std::max<int64_t>(1, (L.ncells + nsm - 1) / nsm);
         if (box)   // the cells of the block that this gives
           cb = (pi ? dg_tile<float>(L.n, false, L.m, L.ncells, cb) : dg_tile<double>(L.n, false, L.m, L.ncells, cb)).cells;
+        if (L.kind == 1 && (pi ? one_pass_fe<float>(L) : one_pass_fe<double>(L)))   // the brick that fits the mesh
+          cb = (pi ? fe_tile<float>(L.n, false, L.m, L.ncells, 0) : fe_tile<double>(L.n, false, L.m, L.ncells, 0)).cells;
         L.cb[pi][pass] = L.cb0[pi][pass] = cb;
       }
   for (Level &L : c->lv) set_box(L);
@@ -2430,7 +2432,9 @@ sipg_status sipg_set_tile_shape(sipg_ctx *c, int level, int precision, int pass,
   const int n = c->lv[level].n;
   const int mx = pass < 2 ? (precision == 0 ? dg_max_cells_per_block<double>(n) : dg_max_cells_per_block<float>(n))
                           : (precision == 0 ? fe_max_cells_per_block<double>(n) : fe_max_cells_per_block<float>(n));
-  if (cells_per_block < 0 || cells_per_block > mx) return SIPG_EINVAL;
+  // (a brick by default may hold more cells than a width that can be asked for)
+  if (cells_per_block < 0 || (cells_per_block > mx && cells_per_block != c->lv[level].cb0[precision][pass]))
+    return SIPG_EINVAL;
   c->lv[level].cb[precision][pass] = cells_per_block ? cells_per_block : c->lv[level].cb0[precision][pass];
   set_box(c->lv[level]);
   // captured V-cycles hold the old launch shapes
@@ -3063,7 +3067,7 @@ std::unique_ptr<BatchCycle<T>> batch_cycle_build(sipg_batch *B) {
     for (int p = 0; p < np; ++p) {
       const Level &F = B->ctx[p]->lv[B->ctx[p]->L - 1];
       if (C->solo[p] || !one_pass_fe<T>(F)) continue;
-      fe_box_brick<T>(F.n, F.m, most, C->brick[p].data());
+      fe_level_brick<T>(F.n, F.m, most, C->brick[p].data());
       total += bricks(p);
     }
     if (total >= kFEBatchBricks) break;

@@ -56,3 +56,33 @@ def test_batch_with_both_routes_equals_each_problems_cycle():
         B.contexts[i].vcycle(r, z)
         torch.cuda.synchronize()
         assert torch.equal(zs[i], z), probs[i]
+
+
+def test_widths_of_an_fe_level_are_the_cells_of_its_bricks():
+    """The default width is the cells of the brick that runs (4 x 4 x 2 of degree 4 here), it
+    can be set again although no other width above the limit can, and the full brick with a
+    remainder in every direction gives the general path's result in FP32 too."""
+    from paper_1910_01900_gb300 import Context
+    from paper_1910_01900_gb300.csrc_info import max_cells_per_block
+    from paper_1910_01900_gb300.native import SipgError
+    m, k = (21, 22, 11), 4
+    box, general = (Context(m, k, bc=BC, fe_assemble=0, lambda_override=2.0, **kw)
+                    for kw in (dict(), dict(deform=1, amp=0.0)))
+    level = box.num_levels - 2
+    assert box.tile_shape(1, 2, level) == 32 > max_cells_per_block(k + 1, 4)
+    u = torch.as_tensor(sipg_inputs.uniform(box.num_dofs(level), 5)).cuda()
+    ref = torch.empty_like(u)
+    general.level_apply(level, u, ref)
+    first = None
+    for cb in (0, 10, 1, 32):
+        box.set_tile_shape(1, 2, cb, level=level)
+        assert box.tile_shape(1, 2, level) == (cb or 32)
+        v = torch.full_like(u, float("nan"), dtype=torch.float32)
+        box.level_apply(level, u.float(), v)
+        torch.cuda.synchronize()
+        if first is None:
+            first = v
+            assert close(v.cpu().numpy().astype("float64"), ref.cpu().numpy()) <= 1e-5
+        assert torch.equal(v, first), cb
+    with pytest.raises(SipgError):
+        box.set_tile_shape(1, 2, 31, level=level)

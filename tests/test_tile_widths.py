@@ -19,6 +19,7 @@ KEEP = 4
 MAIN = r"""
 #include <cstdio>
 #include "dg_launch.cuh"
+#include "fe_box.cuh"
 using namespace sipg;
 template <typename T>
 void run(int n, bool curved, const int (&m)[3]) {
@@ -37,8 +38,22 @@ void run(int n, bool curved, const int (&m)[3]) {
   }
   printf("]}\n");
 }
+// FE levels of axis-aligned cells: the default brick, and the one of a width
+template <typename T>
+void bricks(int n, const int (&m)[3]) {
+  printf("{\"key\": [%d, %d, \"fe\", %d, %d, %d], \"bricks\": [", (int)sizeof(T), n, m[0], m[1], m[2]);
+  for (int cb = 0; cb <= 512; ++cb) {
+    int b[3];
+    fe_box_brick<T>(n, m, cb, b);
+    const TileLaunch t = fe_box_launch<T>(n, m, b);
+    printf("%s[%d, %d, %d, %d]", cb ? ", " : "", b[0], b[1], b[2], t.cells);
+  }
+  printf("]}\n");
+}
 int main() {
   const int meshes[][3] = MESHES;
+  for (int n = 2; n <= 9; ++n)
+    for (auto &m : meshes) bricks<float>(n, m), bricks<double>(n, m);
   for (int n = 2; n <= 9; ++n)
     for (int curved = 0; curved < 2; ++curved)
       for (auto &m : meshes) run<float>(n, curved, m), run<double>(n, curved, m);
@@ -75,6 +90,16 @@ def test_candidates_are_distinct_launches(rules, n, elem, curved):
         widths = r["widths"]
         assert widths[0] == launches[0][0]
         assert len(set(launches[w] for w in widths)) == len(widths) == min(KEEP + 1, len(set(launches)))
+
+
+@pytest.mark.parametrize("n,elem", list(itertools.product(range(2, 10), (4, 8))))
+def test_fe_brick_of_a_width(rules, n, elem):
+    """A width is the most cells of a brick, and the cells of a brick as a width give the brick again."""
+    for m in MESHES:
+        bricks = rules[(elem, n, "fe") + m]["bricks"]
+        for cb, (b0, b1, b2, cells) in enumerate(bricks):
+            assert cells == b0 * b1 * b2 and (cells <= cb or cb == 0)
+            assert bricks[cells] == bricks[cb]
 
 
 def test_tuned_widths_of_one_mesh_are_not_another_meshes(tmp_path):
