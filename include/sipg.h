@@ -115,11 +115,11 @@ typedef struct {
                               (the dense coarse solve works on FE_1)       */
   int autotune;            /* 1: at setup, time a few tile shapes (cells per
                               thread block) of every cell kernel of every
-                              level (the DG passes, the curved FE cell
-                              pass) in both precisions and keep the
-                              fastest; the
-                              candidates are the widths whose last wave of
-                              blocks leaves the fewest cell slots idle;
+                              level (the DG passes, the FE operator) in
+                              both precisions and keep the fastest; the
+                              candidates are the default and the widths
+                              whose last wave of blocks leaves the fewest
+                              cell slots idle;
                               cached per (degree, geometry, mesh; curved:
                               number of cells) for the process             */
   int fe_assemble;         /* FE levels of degree <= fe_assemble (0..3;

@@ -1063,11 +1063,17 @@ TileLaunch fe_tile(int n, bool curved, const int m[3], int64_t ncells, int cb) {
 }
 
 template <typename T>
-cudaError_t fe_blocks_per_sm(int n, bool curved, int cells, int *blocks) {
-#define SIPG_FE_OCC(NN)                                                                 \
-  case NN:                                                                              \
-    if (curved) return occ_fe_cells<T, NN, true>(cells, blocks);                        \
-    if constexpr (kBoxCells<T, NN>) return occ_fe_cells<T, NN, false>(cells, blocks);   \
+cudaError_t fe_blocks_per_sm(int n, bool curved, const int m[3], const TileLaunch &t, bool one_pass, int *blocks) {
+  int b[3];
+  if (one_pass) fe_box_brick<T>(n, m, t.cells, b);
+#define SIPG_FE_OCC(NN)                                                                                        \
+  case NN:                                                                                                     \
+    if constexpr (kOnePass<T, NN>)                                                                             \
+      if (one_pass)                                                                                            \
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fe_box_kernel<T, NN>, t.threads,          \
+                                                             fe_box_values(NN - 1, b) * sizeof(T));            \
+    if (curved) return occ_fe_cells<T, NN, true>(t.cells, blocks);                                             \
+    if constexpr (kBoxCells<T, NN>) return occ_fe_cells<T, NN, false>(t.cells, blocks);                        \
     return cudaErrorInvalidValue;
   switch (n) {
     SIPG_FE_OCC(2)
@@ -1526,7 +1532,7 @@ cudaError_t launch_dg_transfer(const XferGeom &g, const T *P1, const T *in, T *o
   template cudaError_t launch_fe_cells<T>(int, bool, const FEArgs<T> &, bool, cudaStream_t, int);       \
   template int fe_max_cells_per_block<T>(int);                                                          \
   template TileLaunch fe_tile<T>(int, bool, const int *, int64_t, int);                                 \
-  template cudaError_t fe_blocks_per_sm<T>(int, bool, int, int *);                                      \
+  template cudaError_t fe_blocks_per_sm<T>(int, bool, const int *, const TileLaunch &, bool, int *);    \
   template bool fe_two_pass<T>(int, int64_t);                                                           \
   template void fe_level_brick<T>(int, const int *, int, int *);                                        \
   template cudaError_t launch_fe_box<T>(const FEArgs<T> &, cudaStream_t);                               \

@@ -256,8 +256,9 @@ int fe_max_cells_per_block(int n);
 // what a width setting (0 = default) launches
 template <typename T>
 TileLaunch fe_tile(int n, bool curved, const int m[3], int64_t ncells, int cb);
+// resident blocks per SM of that launch of the cell pass or the one pass
 template <typename T>
-cudaError_t fe_blocks_per_sm(int n, bool curved, int cells, int *blocks);
+cudaError_t fe_blocks_per_sm(int n, bool curved, const int m[3], const TileLaunch &t, bool one_pass, int *blocks);
 // whether an axis-aligned level takes the cell and node passes (else the one pass)
 template <typename T>
 bool fe_two_pass(int n, int64_t cells);

@@ -864,17 +864,18 @@ std::vector<int> tile_candidates(const Level &L, int pass, int keep) {
   int dev = 0, nsm = 0;
   CK(cudaGetDevice(&dev));
   CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  const bool one_pass = pass == 2 && one_pass_fe<T>(L);
   const int most = pass < 2 ? dg_max_cells_per_block<T>(L.n) : fe_max_cells_per_block<T>(L.n);
   return pick_widths(
       L.cb0[pidx<T>()][pass], most, L.ncells, nsm, keep,
       [&](int cb) {
-        return pass < 2 ? dg_tile<T>(L.n, L.curved, L.m, L.ncells, cb) : fe_tile<T>(L.n, L.curved, L.m, L.ncells, cb);
+        return pass < 2 ? dg_tile<T>(L.n, L.curved, L.m, L.ncells, cb)
+                        : fe_tile<T>(L.n, L.curved, L.m, L.ncells, cb);
       },
       [&](const TileLaunch &t) {
         int occ = 0;
-        const int groups = t.threads / (L.n * L.n);
-        CK(pass < 2 ? dg_blocks_per_sm<T>(L.n, L.curved, pass, groups, &occ)
-                    : fe_blocks_per_sm<T>(L.n, L.curved, groups, &occ));
+        CK(pass < 2 ? dg_blocks_per_sm<T>(L.n, L.curved, pass, t.threads / (L.n * L.n), &occ)
+                    : fe_blocks_per_sm<T>(L.n, L.curved, L.m, t, one_pass, &occ));
         return occ;
       });
 }
@@ -906,7 +907,8 @@ void autotune_level(sipg_ctx *c, int l, int pass) {
   } else {
     f = fe_args<T>(c, L);
     f.u = u;
-    f.ebuf = v;   // the cell pass writes ncells n^3 values: the DG length of this mesh
+    f.ebuf = f.out = v;   // the cell pass writes ncells n^3 values: the DG length of this mesh
+    f.mode = 0;
   }
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
@@ -920,7 +922,10 @@ void autotune_level(sipg_ctx *c, int l, int pass) {
         CK(launch_dg_box<T>(L.n, a, c->stream));
       } else if (pass == 0) CK(launch_dg_eval<T>(L.n, a, c->stream, cb));
       else if (pass == 1) CK(launch_dg_integrate<T>(L.n, a, c->stream, cb));
-      else CK(launch_fe_cells<T>(L.n, L.curved, f, false, c->stream, cb));
+      else if (one_pass_fe<T>(L)) {
+        fe_level_brick<T>(L.n, L.m, cb, f.brick);
+        CK(launch_fe_box<T>(f, c->stream));
+      } else CK(launch_fe_cells<T>(L.n, L.curved, f, false, c->stream, cb));
     };
     if (pass == 1 && L.curved) CK(launch_dg_eval<T>(L.n, a, c->stream, 0));   // valid scratch for the integration
     run();
@@ -1120,10 +1125,10 @@ void setup(sipg_ctx *c) {
     for (int l = c->solver ? 1 : c->L; l <= c->L; ++l) {
       const int k = c->lv[l].kind;
       if (k == 1 && c->lv[l].deg <= P.fe_assemble) continue;   // assembled stencil: no cell pass to tune
-      // axis-aligned DG levels have one pass (1); an FE level's brick follows from the mesh
+      // axis-aligned DG levels have one pass (1)
       for (int pass = k == 0 ? (c->lv[l].curved ? 0 : 1) : 2; pass <= (k == 0 ? 1 : 2); ++pass) {
-        if (k == 0 || !one_pass_fe<double>(c->lv[l])) autotune_level<double>(c, l, pass);
-        if (k == 0 || !one_pass_fe<float>(c->lv[l])) autotune_level<float>(c, l, pass);
+        autotune_level<double>(c, l, pass);
+        autotune_level<float>(c, l, pass);
       }
       set_box(c->lv[l]);
     }

@@ -86,3 +86,22 @@ def test_widths_of_an_fe_level_are_the_cells_of_its_bricks():
         assert torch.equal(v, first), cb
     with pytest.raises(SipgError):
         box.set_tile_shape(1, 2, 31, level=level)
+
+
+@pytest.mark.parametrize("k", [2, 4, 6])
+def test_autotuned_fe_levels_give_the_same_results(k):
+    from paper_1910_01900_gb300 import Context
+    m = (9, 10, 12)
+    plain, tuned = (Context(m, k, bc=BC, fe_assemble=0, lambda_override=2.0, autotune=a) for a in (False, True))
+    for level in range(1, plain.num_levels - 1):
+        for dt, prec in ((torch.float64, 0), (torch.float32, 1)):
+            u = torch.as_tensor(sipg_inputs.uniform(plain.num_dofs(level), 40 + level)).cuda().to(dt)
+            v, w, x = (torch.full_like(u, float("nan")) for _ in range(3))
+            plain.level_apply(level, u, v)
+            tuned.level_apply(level, u, w)
+            width = tuned.tile_shape(prec, 2, level)
+            tuned.set_tile_shape(prec, 2, width, level=level)   # a tuned width can be set again
+            assert tuned.tile_shape(prec, 2, level) == width
+            tuned.level_apply(level, u, x)
+            torch.cuda.synchronize()
+            assert torch.equal(v, w) and torch.equal(v, x), (level, prec)

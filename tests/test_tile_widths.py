@@ -48,6 +48,16 @@ void bricks(int n, const int (&m)[3]) {
     const TileLaunch t = fe_box_launch<T>(n, m, b);
     printf("%s[%d, %d, %d, %d]", cb ? ", " : "", b[0], b[1], b[2], t.cells);
   }
+  auto launch = [&](int cb) {
+    int b[3];
+    fe_box_brick<T>(n, m, cb, b);
+    return fe_box_launch<T>(n, m, b);
+  };
+  printf("], \"widths\": [");
+  const char *c = "";
+  for (int w : pick_widths(launch(0).cells, max_cb(n, sizeof(T)), (int64_t)m[0] * m[1] * m[2], 152, KEEP, launch,
+                           [&](const TileLaunch &t) { return 2048 / t.threads; }))
+    printf("%s%d", c, w), c = ", ";
   printf("]}\n");
 }
 int main() {
@@ -100,6 +110,10 @@ def test_fe_brick_of_a_width(rules, n, elem):
         for cb, (b0, b1, b2, cells) in enumerate(bricks):
             assert cells == b0 * b1 * b2 and (cells <= cb or cb == 0)
             assert bricks[cells] == bricks[cb]
+        widths = rules[(elem, n, "fe") + m]["widths"]
+        settings = [0] + list(range(1, max_cells_per_block(n, elem) + 1))
+        assert widths[0] == bricks[0][3]
+        assert len(widths) == len(set(widths)) == min(KEEP + 1, len(set(bricks[c][3] for c in settings)))
 
 
 def test_tuned_widths_of_one_mesh_are_not_another_meshes(tmp_path):
