@@ -986,10 +986,7 @@ void set_box(Level &L) {
   L.box[1] = dg_box_shape<float>(L.n, L.m, L.cb[1][1]);
 }
 
-// Default tile widths of every level: the compiled default, lowered on
-// meshes that would give fewer blocks than SMs, so that every SM gets cells
-// (GB300 runs two FP64 FMAs per clock per SM: an FP64 pass over 64 cells in 4
-// blocks of 16 would use 4 of the 152 SMs).
+// Default tile widths of every level (default_width).
 void default_tile_widths(sipg_ctx *c) {
   int dev = 0, nsm = 0;
   CK(cudaGetDevice(&dev));
@@ -999,7 +996,7 @@ void default_tile_widths(sipg_ctx *c) {
       for (int pass = 0; pass < 3; ++pass) {
         const bool box = L.kind == 0 && !L.curved;
         int cb = pi ? dg_cells_per_block<float>(L.n, !box) : dg_cells_per_block<double>(L.n, !box);
-        if (nsm > 0 && (L.ncells + cb - 1) / cb < nsm) cb = (int)std::max<int64_t>(1, (L.ncells + nsm - 1) / nsm);
+        cb = default_width(cb, L.ncells, nsm);
         if (box)   // the cells of the block that this gives
           cb = (pi ? dg_tile<float>(L.n, false, L.m, L.ncells, cb) : dg_tile<double>(L.n, false, L.m, L.ncells, cb)).cells;
         if (L.kind == 1 && (pi ? one_pass_fe<float>(L) : one_pass_fe<double>(L)))   // the brick that fits the mesh

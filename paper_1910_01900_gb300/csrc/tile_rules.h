@@ -18,6 +18,15 @@ struct TileLaunch {
   }
 };
 
+// The default width of a level: that of the kernel, lowered on meshes that would
+// give fewer blocks than SMs, so that every SM gets cells (GB300 runs two FP64
+// FMAs per clock per SM: an FP64 pass over 64 cells in 4 blocks of 16 would use 4
+// of the 152 SMs).
+inline int default_width(int cb, int64_t ncells, int nsm) {
+  if (nsm > 0 && (ncells + cb - 1) / cb < nsm) cb = (int)std::max<int64_t>(1, (ncells + nsm - 1) / nsm);
+  return cb;
+}
+
 // What a timed choice depends on.  The blocks of axis-aligned cells are cut from
 // the mesh's sides (64 x 64 x 1 and 16^3 cells take other bricks), the others
 // from the cells in a row.
