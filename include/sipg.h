@@ -469,11 +469,11 @@ sipg_status sipg_fma_peak(int precision, void *stream, double *flops_per_s);
  * sipg_operator_apply for affine cells (mesh->deform must be 0), with
  * penalty_factor as in sipg_params.  The caller passes the device vectors u
  * and v (length m0 m1 m2 (degree+1)^3, DG order; overlapping ranges are
- * rejected with SIPG_EINVAL); every
- * other buffer lives in one static device array of 64 MiB that each GPU
- * loading the library holds until the process exits.  Problems whose scratch
- * (3 (k+1)^3 + 12 (k+1)^2 + 1 doubles per cell, plus small tables) exceeds
- * 64 MiB are rejected with SIPG_EINVAL (about 1.4 million DoF at degree 3).
+ * rejected with SIPG_EINVAL); the penalties, three doubles per cell, live in
+ * one static device array of 2.8 MB that each GPU loading the library holds
+ * until the process exits.  Problems of more than 64 MiB at 3 (k+1)^3 + 12 (k+1)^2
+ * + 1 doubles per cell (plus small tables) are rejected with SIPG_EINVAL (about
+ * 1.4 million DoF at degree 3).
  * The first call on a device looks up the array's device address and uploads
  * the 1D tables (both synchronous); make that first call before any stream
  * capture.  All calls share the one array: two calls whose work overlaps on

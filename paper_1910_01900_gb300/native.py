@@ -491,8 +491,8 @@ def operator_apply_noalloc(m, degree, u, v, lo=(0.0, 0.0, 0.0), hi=(1.0, 1.0, 1.
     """v = A u (FP64, affine cells) through sipg_operator_apply_noalloc.
 
     For callers that cannot allocate device memory when they need A u: the
-    library uses its static 64 MiB device scratch instead of allocating.
-    Calls that overlap on the GPU race (they share that scratch).
+    library uses a static device array (three penalties per cell) instead of
+    allocating.  Calls that overlap on the GPU race (they share that array).
     """
     import torch
     mesh = Mesh()

@@ -15,7 +15,9 @@ Axis-aligned cells take one pass of six line products (csrc/dg_box.cuh), all of
 it booked as the integration pass: per line and direction the n x (n + 4)
 flux product (even-odd, 2 (hc (hc + 2) + h (h + 2)) + 2n), two end derivatives
 (2n each) and 12 for the ends' coefficients, and the mass product
-(2 (hc^2 + h^2) + 2n), hc = ceil(n/2), h = floor(n/2).
+(2 (hc^2 + h^2) + 2n), hc = ceil(n/2), h = floor(n/2).  (Degrees 1 and 2 take
+five mass products instead of three, for their rounding; the count is the
+smaller number.)
 
 bytes_alg: read u and write v (2 words per DoF); curved cells add the stored
 geometry of the paper's scheme (J^-T and JxW per cell point, n^T J^-T and the
